@@ -54,6 +54,7 @@ int branch_streams(int n, cudaStream_t* streams, cudaEvent_t* events, cudaEvent_
 unsigned long long bound_hits_field(bool reset);
 unsigned long long bound_hits_observables(bool reset);
 unsigned long long bound_hits_smear(bool reset);
+unsigned long long bound_hits_smear_fx(bool reset);
 unsigned long long bound_hits_sweep(bool reset);
 unsigned long long bound_hits_sweep_f32(bool reset);
 unsigned long long bound_hits_sweep_df(bool reset);
@@ -266,6 +267,12 @@ int compute_wilson_loops_offaxis(const void* U, int prec, const Geom& g, int nfi
 // ---- smearing (mcg_smear.cu) ------------------------------------------------
 int run_smear(const void* Uin, void* Uout, int prec, const Geom& g, int nfields, double rho, double eps, int n,
               cudaStream_t st);
+
+// FP64 smearing in fixed point (mcg_smear_fx.cu), n >= 1 steps of a validated
+// field: whether rho, eps meet its operand bounds, and the steps.
+bool smear_fx_applies(double rho, double eps);
+int run_smear_fx(const void* Uin, void* Uout, const Geom& g, int nfields, double rho, double eps, int n,
+                 cudaStream_t st);
 
 // ---- differentiation (mcg_smear.cu) -----------------------------------------
 int run_smear_step_backward(const void* U, const double* Gout, double* Gin, const Geom& g, int nfields, double rho,

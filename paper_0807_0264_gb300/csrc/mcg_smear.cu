@@ -284,6 +284,9 @@ int run_smear(const void* Uin, void* Uout, int prec, const Geom& g, int nfields,
         MCG_CK(cudaMemcpyAsync(Uout, Uin, bytes, cudaMemcpyDeviceToDevice, st));
         return 0;
     }
+    // FP64 fields in fixed point where its operand bounds hold (the paper's
+    // parameters: 0.6 and 0.77 of the limit); other rho, eps in FP64
+    if (prec == MCG_F64 && smear_fx_applies(rho, eps)) return run_smear_fx(Uin, Uout, g, nfields, rho, eps, n, st);
     int rc = 0;
     void* tmp = nullptr;
     if (n >= 2) {
