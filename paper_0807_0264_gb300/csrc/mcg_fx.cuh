@@ -117,6 +117,28 @@ __device__ __forceinline__ fx fx_of(double d) { return fx_split(fx_from_bits((un
 __device__ __forceinline__ double fx_double(long long X) { return __longlong_as_double((long long)fx_to_bits(X)); }
 #endif
 
+#ifdef __CUDACC__
+// A matrix (entry (r, k) at src[r sr + k sc]) the fixed-point sweep does not
+// take: an entry above 1.03 in magnitude or not finite, or a row whose squared
+// norm is off 1 by 5 % (tiny rows would lose relative precision).
+__device__ __forceinline__ bool fx_bad_matrix(const double2* src, size_t sr, size_t sc) {
+    bool bad = false;
+#pragma unroll 1
+    for (int r = 0; r < 3; ++r) {
+        float n2 = 0.f;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const double2 d = src[r * sr + k * sc];
+            bad = bad || (__double2hiint(d.x) & 0x7fffffff) > 0x3ff07ae1 || (__double2hiint(d.y) & 0x7fffffff) > 0x3ff07ae1;
+            const float x = (float)fx_of(d.x).h, y = (float)fx_of(d.y).h;  // unit 2^-28
+            n2 = fmaf(x, x, fmaf(y, y, n2));
+        }
+        bad = bad || !(fabsf(n2 * 0x1p-56f - 1.f) < 0.05f);
+    }
+    return bad;
+}
+#endif
+
 // ---- 3 x 3 complex matrices (row-major) ---------------------------------------
 MCG_HD void cfx_mac(facc& re, facc& im, cfx a, cfx b) {
     fx_mac(re, a.re, b.re);

@@ -57,6 +57,7 @@ unsigned long long bound_hits_smear(bool reset);
 unsigned long long bound_hits_smear_fx(bool reset);
 unsigned long long bound_hits_sweep(bool reset);
 unsigned long long bound_hits_sweep_f32(bool reset);
+unsigned long long bound_hits_sweep_fx(bool reset);
 unsigned long long bound_hits_sweep_df(bool reset);
 void release_all();
 
@@ -107,6 +108,8 @@ struct SweepBatch {
     int reunit_every;
     double omega;  // over-relaxation parameter (1: plain relaxation)
     int solve32;   // FP64 sweeps: local problem built and solved in FP32
+    int tps = 0;              // threads per site of the fixed-point FP64 sweep (0: another kernel)
+    unsigned* bad = nullptr;  // unvalidated fields: sites left to the FP64 kernel
 };
 
 // Haar-random SU(3) transforms (FP64 gauge layout, the same in each of the
@@ -206,6 +209,18 @@ void launch_functional_df(const SweepBatch& bt, int nblocks, cudaStream_t st);
 int launch_to_df(const double* src, void* hi, void* lo, const Geom& g, int nmat, int nfields, cudaStream_t st);
 int launch_identity_df(void* hi, void* lo, const Geom& g, int nfields, cudaStream_t st);
 
+// The exact FP64 half-sweep in fixed point (mcg_sweep_fx.cu): threads per site
+// and per block for a number of sites of one parity, shared-memory set-up on
+// the current device, launch (nblocks of shape.nt / shape.tps sites).  With
+// bt.bad set (shape {2, 128}) sites with matrices that are not near-unitary
+// are left alone and counted there.
+struct FxShape {
+    int tps, nt;
+};
+FxShape fx_shape(long long sites);
+int prepare_halfsweep_fx();
+void launch_halfsweep_fx(FxShape shape, bool acc, const SweepBatch& bt, int parity, int nblocks, cudaStream_t st);
+
 // The compact FP32 half-sweep (mcg_sweep_f32.cu): raise its shared-memory
 // limit for nt threads per block (64, 128, 256) on the current device, and
 // launch one half-sweep of the batch (acc: with the fused R partials).
@@ -216,7 +231,6 @@ void launch_halfsweep_c12(int nt, bool acc, const SweepBatch& bt, int parity, in
 // each block covers (one thread per site in both precisions)
 int sweep_block(int prec);
 void set_sweep_block(int prec, int nt);
-int sweep_sites_per_block(int prec);
 
 // ---- input validation (mcg_field.cu) -----------------------------------------
 // Tolerances of the SU(3) check on caller-supplied fields: max |M M^dag - 1|

@@ -12,13 +12,14 @@
 // mu >= lambda_max(A)).
 //
 // Precision: the FP32 kernel does everything in FP32 (R accumulated in FP64).
-// The FP64 kernel builds A, b and applies G in FP64; the 4x4 solve is seeded
-// by an FP32 Jacobi eigen-decomposition + secular Newton and then refined to
-// FP64 accuracy by Newton steps on the KKT system whose residual is evaluated
-// in FP64 (the FP32 eigen-decomposition serves as the approximate inverse).
-// Solves the refinement cannot settle (near-degenerate or hard cases) rerun
-// in full FP64.  FP64 arithmetic is scarce on GB300, so the expensive part of
-// the solve stays on the FP32 pipe.
+// FP64 arithmetic is scarce on GB300 (one FMA per 80 cycles and scheduler).
+// The exact FP64 sweep therefore runs in fixed point on FP64 storage
+// (mcg_sweep_fx.cu); the kernel of this file serves the sweeps with the FP32
+// local solve (fp64_solve32), which apply G in FP64, and the sites of
+// unvalidated fields (slab half-sweeps) whose matrices are not near-unitary:
+// it builds A, b and applies G in FP64, its 4x4 solve seeded by FP32 Newton and
+// refined to FP64 accuracy by Newton steps on the KKT system.  Solves the
+// refinement cannot settle (near-degenerate or hard cases) rerun in full FP64.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -28,6 +29,7 @@
 #include <vector>
 
 #include "mcg_common.cuh"
+#include "mcg_fx.cuh"
 #include "mcg_internal.h"
 #include "mcg_sweep.cuh"
 
@@ -203,8 +205,12 @@ __device__ __forceinline__ int subgroup_step(L& lk, const int P, const int Q, co
 // ---------------------------------------------------------------------------
 // Shared memory per thread: 8 links + Omega (81 complex): 41.5 KB for 64 FP32
 // threads (5 blocks per SM), 83 KB for 128 FP32 or 64 FP64 threads (2 per SM).
-template <typename T, bool ACC, int NT, bool S32 = false>
+// S32: the local problem in FP32 (every site).  Otherwise: only the sites that
+// the fixed-point sweep of an unvalidated field left alone (bt.bad counts them,
+// zero for any SU(3) field), by the same test.
+template <typename T, bool ACC, int NT, bool S32>
 __global__ void __launch_bounds__(NT, 2) k_halfsweep(SweepBatch bt, int parity) {
+    if (!S32 && *bt.bad == 0) return;
     const int f = field_of_block(bt.desc, bt.nf, blockIdx.x);
     if (bt.state[f].done) return;  // block-uniform
     const FieldDesc fd = bt.desc[f];
@@ -225,10 +231,22 @@ __global__ void __launch_bounds__(NT, 2) k_halfsweep(SweepBatch bt, int parity) 
 
     double rsum = 0.0;
     int fb = 0;
+    int sb[4] = {0, 0, 0, 0};
     if (active) {
-        int sb[4];
 #pragma unroll
         for (int mu = 0; mu < 4; ++mu) sb[mu] = eo_neighbor(g, c, mu, -1);
+        if constexpr (!S32) {
+            const double2* Ud = reinterpret_cast<const double2*>(fd.U);
+            const size_t vh = (size_t)g.vh;
+            bool bad = fx_bad_matrix(reinterpret_cast<const double2*>(fd.G) + gidx(g, parity, 0, s), 3 * vh, vh);
+#pragma unroll 1
+            for (int mu = 0; mu < 4; ++mu)
+                bad = bad || fx_bad_matrix(Ud + lidx(g, mu, parity, 0, s), 3 * vh, vh) ||
+                      fx_bad_matrix(Ud + lidx(g, mu, parity ^ 1, 0, sb[mu]), vh, 3 * vh);
+            active = bad;
+        }
+    }
+    if (active) {
         // stage the 8 links and Omega in shared memory without passing
         // through registers
 #pragma unroll
@@ -720,7 +738,6 @@ static int g_sweep_nt[2] = {128, 128};
 
 int sweep_block(int prec) { return g_sweep_nt[prec == MCG_F64 ? 0 : 1]; }
 void set_sweep_block(int prec, int nt) { g_sweep_nt[prec == MCG_F64 ? 0 : 1] = nt; }
-int sweep_sites_per_block(int prec) { return sweep_block(prec); }
 
 template <typename K>
 static int raise_smem(K kernel, size_t smem) {
@@ -733,20 +750,19 @@ static size_t halfsweep_smem_f64(int nt) { return sizeof(cplx<double>) * 81 * nt
 
 // Raises the dynamic shared-memory limit of the half-sweep kernels for the
 // current device.  Called on every fix phase (never inside a stream capture):
-// the attribute is per device, and the call costs microseconds.
+// the attribute is per device, and the call costs microseconds.  FP64: the
+// sweeps with the FP32 local solve.
 template <typename T>
 static int prepare_halfsweep(int nt) {
     if constexpr (sizeof(T) == 8) {
         const size_t smem = halfsweep_smem_f64(nt);
         int rc = 0;
         if (nt == 128) {
-            if ((rc = raise_smem(k_halfsweep<T, false, 128>, smem)) || (rc = raise_smem(k_halfsweep<T, true, 128>, smem)) ||
-                (rc = raise_smem(k_halfsweep<T, false, 128, true>, smem)) ||
+            if ((rc = raise_smem(k_halfsweep<T, false, 128, true>, smem)) ||
                 (rc = raise_smem(k_halfsweep<T, true, 128, true>, smem)))
                 return rc;
         } else {
-            if ((rc = raise_smem(k_halfsweep<T, false, 64>, smem)) || (rc = raise_smem(k_halfsweep<T, true, 64>, smem)) ||
-                (rc = raise_smem(k_halfsweep<T, false, 64, true>, smem)) ||
+            if ((rc = raise_smem(k_halfsweep<T, false, 64, true>, smem)) ||
                 (rc = raise_smem(k_halfsweep<T, true, 64, true>, smem)))
                 return rc;
         }
@@ -761,26 +777,47 @@ template <typename T>
 static void launch_halfsweep(int nt, bool acc, const SweepBatch& bt, int parity, int nblocks, cudaStream_t st) {
     if constexpr (sizeof(T) == 8) {
         const size_t smem = halfsweep_smem_f64(nt);
-        const bool s32 = bt.solve32 != 0;
-        if (nt == 128) {
-            if (acc)
-                (s32 ? k_halfsweep<T, true, 128, true> : k_halfsweep<T, true, 128>)<<<nblocks, 128, smem, st>>>(bt, parity);
-            else
-                (s32 ? k_halfsweep<T, false, 128, true> : k_halfsweep<T, false, 128>)<<<nblocks, 128, smem, st>>>(bt,
-                                                                                                                parity);
+        if (bt.tps > 0) {
+            launch_halfsweep_fx(FxShape{bt.tps, nt}, acc, bt, parity, nblocks, st);
+        } else if (nt == 128) {
+            (acc ? k_halfsweep<T, true, 128, true> : k_halfsweep<T, false, 128, true>)<<<nblocks, 128, smem, st>>>(bt,
+                                                                                                              parity);
         } else {
-            if (acc)
-                (s32 ? k_halfsweep<T, true, 64, true> : k_halfsweep<T, true, 64>)<<<nblocks, 64, smem, st>>>(bt, parity);
-            else
-                (s32 ? k_halfsweep<T, false, 64, true> : k_halfsweep<T, false, 64>)<<<nblocks, 64, smem, st>>>(bt, parity);
+            (acc ? k_halfsweep<T, true, 64, true> : k_halfsweep<T, false, 64, true>)<<<nblocks, 64, smem, st>>>(bt,
+                                                                                                            parity);
         }
     } else {
         launch_halfsweep_c12(nt, acc, bt, parity, nblocks, st);
     }
 }
 
+// One exact FP64 half-sweep of a single field that was not validated: the
+// fixed-point kernel on the sites with near-unitary matrices, the FP64 kernel
+// on the others (blocks exit at entry when there are none).  fd.nblk: blocks of
+// 64 sites; the FP64 kernel covers its sites in blocks of 64 as well.  acc: R
+// partials, nblk * 4 of the first kernel, then nblk * 2 of the second.
+static int prepare_unvalidated() {
+    int rc = prepare_halfsweep_fx();
+    if (!rc) rc = raise_smem(k_halfsweep<double, false, 64, false>, halfsweep_smem_f64(64));
+    if (!rc) rc = raise_smem(k_halfsweep<double, true, 64, false>, halfsweep_smem_f64(64));
+    return rc;
+}
+constexpr int kUnvalidatedSites = 64, kUnvalidatedPartials = 6;  // per block
+static int launch_unvalidated(bool acc, SweepBatch bt, int parity, int nblocks, cudaStream_t st) {
+    MCG_CK(cudaMemsetAsync(bt.bad, 0, sizeof(unsigned), st));
+    double* rest = bt.partial + (size_t)nblocks * 4;
+    if (acc) MCG_CK(cudaMemsetAsync(rest, 0, sizeof(double) * 2 * nblocks, st));
+    launch_halfsweep_fx(FxShape{2, 128}, acc, bt, parity, nblocks, st);
+    bt.partial = rest;
+    (acc ? k_halfsweep<double, true, 64, false>
+         : k_halfsweep<double, false, 64, false>)<<<nblocks, 64, halfsweep_smem_f64(64), st>>>(bt, parity);
+    note_launches(2);
+    MCG_CK(cudaGetLastError());
+    return 0;
+}
+
 template <typename T>
-static int enqueue_sweep(const SweepBatch& bt, int nt, int spb, cudaStream_t st) {
+static int enqueue_sweep(const SweepBatch& bt, int nt, cudaStream_t st) {
     if constexpr (std::is_same<T, DoubleFloat>::value) {
         // no re-unitarisation inside the phase: the double-float links drift
         // from unitarity by ~1e-14 per sweep; the output is the FP64 field
@@ -794,7 +831,7 @@ static int enqueue_sweep(const SweepBatch& bt, int nt, int spb, cudaStream_t st)
         k_finalize<<<bt.nf, 256, 0, st>>>(bt, 0);
         // FP32 sweeps re-unitarise inside the half-sweep kernel
         if constexpr (sizeof(T) == 8)
-            if (bt.reunit_every > 0) k_reunit_pending<T><<<bt.total_blocks, spb, 0, st>>>(bt);
+            if (bt.reunit_every > 0) k_reunit_pending<T><<<bt.total_blocks, nt, 0, st>>>(bt);
     }
     return 0;
 }
@@ -808,13 +845,21 @@ int run_fix_phase(const std::vector<FieldDesc>& fields_in, FieldState* d_state, 
                   int check_every, bool fresh, cudaStream_t stream, bool solve32, const PhaseRestart* restart) {
     constexpr bool DF = std::is_same<T, DoubleFloat>::value;
     const int prec = (DF || sizeof(T) == 8) ? MCG_F64 : MCG_F32;
-    const int NT = DF ? df_threads() : sweep_block(prec);
-    const int SPB = DF ? NT : sweep_sites_per_block(prec);
     const int nf = (int)fields_in.size();
     std::vector<FieldDesc> fields = fields_in;
+    // the exact FP64 sweep: several threads per site
+    FxShape fx = {0, 0};
+    if (!DF && sizeof(T) == 8 && !solve32) {
+        long long sites = 0;
+        for (const auto& fd : fields) sites += fd.geo.vh;
+        fx = fx_shape(sites);
+    }
+    // threads and sites per block (one thread per site in the other kernels)
+    const int NT = DF ? df_threads() : (fx.tps ? fx.nt : sweep_block(prec));
+    const int sites_per_block = fx.tps ? fx.nt / fx.tps : NT;
     int total = 0;
     for (auto& fd : fields) {
-        fd.nblk = (fd.geo.vh + SPB - 1) / SPB;
+        fd.nblk = (fd.geo.vh + sites_per_block - 1) / sites_per_block;
         fd.blk0 = total;
         fd.omega = omega;
         total += fd.nblk;
@@ -823,7 +868,7 @@ int run_fix_phase(const std::vector<FieldDesc>& fields_in, FieldState* d_state, 
     int rc = 0;
     FieldDesc* d_desc = (FieldDesc*)scratch_device("fix.desc", sizeof(FieldDesc) * nf, &rc);
     if (rc) return rc;
-    double* d_partial = (double*)scratch_device("fix.partial", sizeof(double) * total * (SPB / 32), &rc);
+    double* d_partial = (double*)scratch_device("fix.partial", sizeof(double) * total * (NT / 32), &rc);
     if (rc) return rc;
     FieldDesc* h_desc = (FieldDesc*)scratch_host("fix.desc", sizeof(FieldDesc) * nf, &rc);
     if (rc) return rc;
@@ -853,7 +898,8 @@ int run_fix_phase(const std::vector<FieldDesc>& fields_in, FieldState* d_state, 
     bt.total_blocks = total;
     bt.state = d_state;
     bt.partial = d_partial;
-    bt.ppb = SPB / 32;
+    bt.ppb = NT / 32;
+    bt.tps = fx.tps;
     bt.R_hist = d_hist;
     bt.hist_len = hist_len;
     bt.tol = tol;
@@ -866,8 +912,8 @@ int run_fix_phase(const std::vector<FieldDesc>& fields_in, FieldState* d_state, 
         if ((rc = prepare_halfsweep_df())) return rc;
         launch_functional_df(bt, total, stream);
     } else {
-        if ((rc = prepare_halfsweep<T>(NT))) return rc;
-        k_functional<T><<<total, SPB, 0, stream>>>(bt);
+        if ((rc = fx.tps ? prepare_halfsweep_fx() : prepare_halfsweep<T>(NT))) return rc;
+        k_functional<T><<<total, NT, 0, stream>>>(bt);
     }
     k_finalize<<<nf, 256, 0, stream>>>(bt, fresh ? 1 : 2);
     MCG_CK(cudaGetLastError());
@@ -931,12 +977,12 @@ int run_fix_phase(const std::vector<FieldDesc>& fields_in, FieldState* d_state, 
         for (int f = 0; f < nf && qe == cudaSuccess; ++f) {
             qe = cudaStreamWaitEvent(bs[f], fork, 0);
             if (qe != cudaSuccess) break;
-            for (int i = 0; i < chunk; ++i) enqueue_sweep<T>(chains[f], NT, SPB, bs[f]);
+            for (int i = 0; i < chunk; ++i) enqueue_sweep<T>(chains[f], NT, bs[f]);
             qe = cudaEventRecord(be[f], bs[f]);
             if (qe == cudaSuccess) qe = cudaStreamWaitEvent(cs, be[f], 0);
         }
     } else {
-        for (int i = 0; i < chunk; ++i) enqueue_sweep<T>(bt, NT, SPB, cs);
+        for (int i = 0; i < chunk; ++i) enqueue_sweep<T>(bt, NT, cs);
     }
     cudaError_t ce = cudaStreamEndCapture(cs, &graph);
     if (qe != cudaSuccess || ce != cudaSuccess) {
@@ -1009,7 +1055,7 @@ int run_fix_phase(const std::vector<FieldDesc>& fields_in, FieldState* d_state, 
         // R of the reset field and a new phase start for it (its sweep count
         // goes on)
         if constexpr (std::is_same<T, float>::value) {
-            k_functional<T><<<fields[f].nblk, SPB, 0, stream>>>(chains[f]);
+            k_functional<T><<<fields[f].nblk, NT, 0, stream>>>(chains[f]);
             k_finalize<<<1, 256, 0, stream>>>(chains[f], 2);
             e = cudaGetLastError();
             if (e != cudaSuccess) return cuda_fail(e, "restart");
@@ -1118,22 +1164,26 @@ int run_fix_phase(const std::vector<FieldDesc>& fields_in, FieldState* d_state, 
 template <typename T>
 int time_halfsweep(void* U, void* G, const Geom& g, int parity, int nreps, int flush_l2, float* ms,
                    cudaStream_t stream) {
-    const int prec = sizeof(T) == 8 ? MCG_F64 : MCG_F32;
-    const int NT = sweep_block(prec);
-    const int SPB = sweep_sites_per_block(prec);
+    // FP64: the exact half-sweep (the caller's field was not validated)
+    constexpr bool F64 = sizeof(T) == 8;
+    const int NT = F64 ? 128 : sweep_block(MCG_F32);
+    const int spb = F64 ? kUnvalidatedSites : NT;
     int rc = 0;
     FieldDesc fd;
     fd.U = U;
     fd.G = G;
     fd.geo = g;
     fd.blk0 = 0;
-    fd.nblk = (g.vh + SPB - 1) / SPB;
+    fd.nblk = (g.vh + spb - 1) / spb;
     fd.norm = 1.0 / (9.0 * 8.0 * g.vh);
     FieldDesc* d_desc = (FieldDesc*)scratch_device("time.desc", sizeof(FieldDesc), &rc);
     if (rc) return rc;
     FieldState* d_state = (FieldState*)scratch_device("time.state", sizeof(FieldState), &rc);
     if (rc) return rc;
-    double* d_partial = (double*)scratch_device("time.partial", sizeof(double) * fd.nblk * (SPB / 32), &rc);
+    double* d_partial =
+        (double*)scratch_device("time.partial", sizeof(double) * fd.nblk * (F64 ? kUnvalidatedPartials : NT / 32), &rc);
+    if (rc) return rc;
+    unsigned* d_bad = (unsigned*)scratch_device("time.bad", sizeof(unsigned), &rc);
     if (rc) return rc;
     void* flush = nullptr;
     const size_t flush_bytes = (size_t)256 << 20;
@@ -1149,7 +1199,8 @@ int time_halfsweep(void* U, void* G, const Geom& g, int parity, int nreps, int f
     bt.total_blocks = fd.nblk;
     bt.state = d_state;
     bt.partial = d_partial;
-    bt.ppb = SPB / 32;
+    bt.ppb = NT / 32;
+    bt.bad = d_bad;
     bt.R_hist = nullptr;
     bt.hist_len = 0;
     bt.tol = 0;
@@ -1157,7 +1208,7 @@ int time_halfsweep(void* U, void* G, const Geom& g, int parity, int nreps, int f
     bt.reunit_every = 0;
     bt.omega = 1.0;
     bt.solve32 = 0;
-    if ((rc = prepare_halfsweep<T>(NT))) return rc;
+    if ((rc = F64 ? prepare_unvalidated() : prepare_halfsweep<T>(NT))) return rc;
     cudaEvent_t e0, e1;
     MCG_CK(cudaEventCreate(&e0));
     MCG_CK(cudaEventCreate(&e1));
@@ -1167,7 +1218,10 @@ int time_halfsweep(void* U, void* G, const Geom& g, int parity, int nreps, int f
             cudaMemsetAsync(flush, r & 0xff, flush_bytes, stream);
         }
         cudaEventRecord(e0, stream);
-        launch_halfsweep<T>(NT, parity != 0, bt, parity, fd.nblk, stream);
+        if (F64)
+            launch_unvalidated(parity != 0, bt, parity, fd.nblk, stream);
+        else
+            launch_halfsweep<T>(NT, parity != 0, bt, parity, fd.nblk, stream);
         cudaEventRecord(e1, stream);
         cudaError_t ce = cudaEventSynchronize(e1);
         if (ce != cudaSuccess) {
@@ -1179,7 +1233,7 @@ int time_halfsweep(void* U, void* G, const Geom& g, int parity, int nreps, int f
         cudaEventElapsedTime(&t, e0, e1);
         total += t;
     }
-    note_launches(nreps);
+    if (!F64) note_launches(nreps);
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     MCG_CK(cudaGetLastError());
@@ -1228,14 +1282,13 @@ int run_anneal(void* U, void* G, const Geom& g, int nfields, const double* T, in
 
 int run_halfsweep_slab(void* U, void* G, const Geom& g, int parity, int t_lo, int t_hi, bool want_R, double* R_host,
                        cudaStream_t stream) {
-    const int NT = sweep_block(MCG_F64);
     int rc = 0;
     FieldDesc fd;
     fd.U = U;
     fd.G = G;
     fd.geo = g;
     fd.blk0 = 0;
-    fd.nblk = (g.vh + NT - 1) / NT;
+    fd.nblk = (g.vh + kUnvalidatedSites - 1) / kUnvalidatedSites;
     fd.norm = 1.0 / (9.0 * 8.0 * g.vh);
     fd.t_lo = t_lo;
     fd.t_hi = t_hi;
@@ -1243,7 +1296,9 @@ int run_halfsweep_slab(void* U, void* G, const Geom& g, int parity, int t_lo, in
     if (rc) return rc;
     FieldState* d_state = (FieldState*)scratch_device("slab.state", sizeof(FieldState), &rc);
     if (rc) return rc;
-    double* d_partial = (double*)scratch_device("slab.partial", sizeof(double) * fd.nblk * (NT / 32), &rc);
+    double* d_partial = (double*)scratch_device("slab.partial", sizeof(double) * fd.nblk * kUnvalidatedPartials, &rc);
+    if (rc) return rc;
+    unsigned* d_bad = (unsigned*)scratch_device("slab.bad", sizeof(unsigned), &rc);
     if (rc) return rc;
     double* d_R = (double*)scratch_device("slab.R", sizeof(double), &rc);
     if (rc) return rc;
@@ -1259,7 +1314,8 @@ int run_halfsweep_slab(void* U, void* G, const Geom& g, int parity, int t_lo, in
     bt.total_blocks = fd.nblk;
     bt.state = d_state;
     bt.partial = d_partial;
-    bt.ppb = NT / 32;
+    bt.ppb = 4;
+    bt.bad = d_bad;
     bt.R_hist = nullptr;
     bt.hist_len = 0;
     bt.tol = 0;
@@ -1267,12 +1323,10 @@ int run_halfsweep_slab(void* U, void* G, const Geom& g, int parity, int t_lo, in
     bt.reunit_every = 0;
     bt.omega = 1.0;
     bt.solve32 = 0;
-    if ((rc = prepare_halfsweep<double>(NT))) return rc;
-    launch_halfsweep<double>(NT, want_R, bt, parity, fd.nblk, stream);
-    note_launches(1);
-    MCG_CK(cudaGetLastError());
+    if ((rc = prepare_unvalidated())) return rc;
+    if ((rc = launch_unvalidated(want_R, bt, parity, fd.nblk, stream))) return rc;
     if (want_R) {
-        k_sum_slab_partials<<<1, 256, 0, stream>>>(d_partial, fd.nblk * (NT / 32), d_R);
+        k_sum_slab_partials<<<1, 256, 0, stream>>>(d_partial, fd.nblk * kUnvalidatedPartials, d_R);
         note_launches(1);
         MCG_CK(cudaGetLastError());
         MCG_CK(cudaMemcpyAsync(R_host, d_R, sizeof(double), cudaMemcpyDeviceToHost, stream));

@@ -31,3 +31,60 @@ def test_fixed_point_smear(dims, rho, eps, n):
     S = mcg.mcg_unpack_links(mcg.mcg_smear(_pack(mcg, Us, dims), dims, rho, eps, n), dims).cpu().numpy()
     for U, s in zip(Us, S):
         assert np.abs(s - oracle.smear(dims, U, rho, eps, n)).max() < 2e-14 * n
+
+
+# lattices of the three shapes of the half-sweep (8, 4 and 2 threads per site), with and without a ragged last
+# block; a field near its maximum, whose local problems are well conditioned: the FP64 sweep's bar of 1e-11 per
+# link; nfields = 2 runs them as chains
+@pytest.mark.parametrize("dims,nf", [((2, 2, 2, 2), 1), ((6, 2, 10, 14), 2), ((10, 6, 14, 12), 1), ((14, 14, 14, 14), 1)])
+def test_fixed_point_sweep(dims, nf):
+    from paper_0807_0264_gb300 import mcg
+
+    Us = [synth.make_field(dims, 0.4, s, gauge=False) for s in range(nf)]
+    Ud, Gd = _pack(mcg, Us, dims), mcg.identity_gauge(dims, nf)
+    r = mcg.mcg_fix(Ud, Gd, dims, mcg.Params(tol=-1e300, max_sweeps=2, reunit_every=0))
+    Uo, Go = mcg.mcg_unpack_links(Ud, dims).cpu().numpy(), mcg.mcg_unpack_gauge(Gd, dims).cpu().numpy()
+    for f, U in enumerate(Us):
+        ref = oracle.fix(dims, U, tol=-1e300, max_sweeps=2, reunit_every=0)
+        assert np.abs(Uo[f] - ref["U"]).max() < 1e-11 and np.abs(Go[f] - ref["G"]).max() < 1e-11
+        assert abs(r["R"][f] - ref["R_hist"][-1]) < 1e-12 * ref["R_hist"][-1]
+
+
+# rough fields from random transforms: most local problems leave the warm start (the second seed, the Jacobi seed
+# and the FP64 solve all run).  A problem with relative gap g between the multiplier and lambda_max moves its
+# element by ~1e-15 / g and P(gap < g) ~ g, so one link in a thousand may pass 1e-12 tenfold: the bar on the
+# 99.9 % quantile; R is stationary in each element
+@pytest.mark.parametrize("seed", range(4))
+def test_fixed_point_sweep_rough(seed):
+    from paper_0807_0264_gb300 import mcg
+
+    dims = (6, 4, 6, 8)
+    U, G = synth.make_field(dims, 3.0, seed), synth.random_gauge(dims, 50 + seed)
+    Ud, Gd = _pack(mcg, [U], dims), mcg.mcg_pack_gauge(torch.from_numpy(G).unsqueeze(0).cuda(), dims)
+    r = mcg.mcg_fix(Ud, Gd, dims, mcg.Params(tol=-1e300, max_sweeps=1, reunit_every=0))
+    ref = oracle.fix(dims, U, G, tol=-1e300, max_sweeps=1, reunit_every=0)
+    err = np.abs(mcg.mcg_unpack_links(Ud, dims)[0].cpu().numpy() - ref["U"])
+    assert np.quantile(err, 0.999) < 1e-11
+    assert abs(r["R"][0] - ref["R_hist"][-1]) < 1e-11 * ref["R_hist"][-1]
+
+
+def test_unvalidated_sites_keep_the_fp64_kernel():
+    """mcg_halfsweep_slab takes any matrices: sites next to a link outside the fixed-point range (scaled by 3 and
+    by 1/4, zero) agree with the oracle as all others do (F scales with the square of the
+    links: 9 x the 1e-11 bar)."""
+    from paper_0807_0264_gb300 import mcg
+
+    dims = (4, 6, 2, 6)
+    U, G = synth.make_field(dims, 0.4, 5, gauge=False), synth.identity_gauge(dims)
+    U[7, 2] *= 3.0
+    U[20, 0] *= 0.25
+    U[100, 3] = 0.0
+    Ud, Gd = _pack(mcg, [U], dims), mcg.mcg_pack_gauge(torch.from_numpy(G).unsqueeze(0).cuda(), dims)
+    Uo, Go = U.copy(), G.copy()
+    for parity in (0, 1):
+        R = mcg.mcg_halfsweep_slab(Ud, Gd, dims, parity, 0, dims[3], want_R=parity == 1)
+        oracle.halfsweep_slab(dims, Uo, Go, parity, 0, dims[3])
+    assert np.abs(mcg.mcg_unpack_links(Ud, dims)[0].cpu().numpy() - Uo).max() < 9e-11
+    assert np.abs(mcg.mcg_unpack_gauge(Gd, dims)[0].cpu().numpy() - Go).max() < 9e-11
+    ref = (np.abs(np.trace(Uo, axis1=-2, axis2=-1)) ** 2).sum()
+    assert abs(R - ref) < 1e-11 * ref
