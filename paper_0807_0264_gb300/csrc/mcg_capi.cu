@@ -259,6 +259,7 @@ struct FieldSpec {
     void* U;
     void* G;
     Geom g;
+    bool keep_fp64 = false;  // a later FP32 phase starts from the result: FP64 arithmetic (mcg_field_fx.cu)
 };
 
 // MCG relaxation of a batch of fields (all of one precision, any sizes), one
@@ -364,7 +365,8 @@ static int fix_fields(const std::vector<FieldSpec>& fs, int prec, const mcg_para
         for (int f = 0; f < nf; ++f) s32[f] = h_state[f].sweep;
         // hand-off: FP64 re-unitarised transform applied to the FP64 links
         for (int f = 0; f < nf; ++f)
-            if ((rc = launch_handoff(fds[f].G, nullptr, (double*)fs[f].U, (double*)fs[f].G, fs[f].g, 1, st)))
+            if ((rc = launch_handoff(fds[f].G, nullptr, (double*)fs[f].U, (double*)fs[f].G, fs[f].g, 1,
+                                     fs[f].keep_fp64, st)))
                 return rc;
         fresh = false;
     }
@@ -405,7 +407,8 @@ static int fix_fields(const std::vector<FieldSpec>& fs, int prec, const mcg_para
                                         prm->max_sweeps, prm->check_every, fresh, st);
         if (rc) return rc;
         for (int f = 0; f < nf; ++f)
-            if ((rc = launch_handoff(fds[f].G, fds[f].Glo, (double*)fs[f].U, (double*)fs[f].G, fs[f].g, 1, st)))
+            if ((rc = launch_handoff(fds[f].G, fds[f].Glo, (double*)fs[f].U, (double*)fs[f].G, fs[f].g, 1,
+                                     fs[f].keep_fp64, st)))
                 return rc;
     } else if (prec == MCG_F64) {
         std::vector<FieldDesc> fds(nf);
@@ -416,7 +419,8 @@ static int fix_fields(const std::vector<FieldSpec>& fs, int prec, const mcg_para
             fds[f].norm = 1.0 / (9.0 * 8.0 * fs[f].g.vh);
         }
         rc = run_fix_phase<double>(fds, d_state, h_state, d_hist, hist_len, prm->tol, 1, 1.0, prm->reunit_every,
-                                   prm->max_sweeps, prm->check_every, fresh, st, prm->fp64_solve32 != 0);
+                                   prm->max_sweeps, prm->check_every, fresh, st, prm->fp64_solve32 != 0, nullptr,
+                                   std::any_of(fs.begin(), fs.end(), [](const FieldSpec& f) { return f.keep_fp64; }));
     } else {
         // FP32 fields: compact copies in, full layout (row 2 rebuilt) out
         std::vector<FieldDesc> fds;
@@ -453,10 +457,11 @@ static int fix_fields(const std::vector<FieldSpec>& fs, int prec, const mcg_para
 // uniform batch: nfields fields of lat's dims stored back to back
 static int fix_impl(void* U, void* G, const mcg_lattice* lat, const Geom& g, const mcg_params* prm, double* R_out,
                     int* sweeps_out, int* sweeps32_out, double* R_hist, cudaStream_t st, int* converged_out = nullptr,
-                    int* restarts_out = nullptr) {
+                    int* restarts_out = nullptr, bool keep_fp64 = false) {
     const size_t eb = elem_bytes(lat->precision);
     std::vector<FieldSpec> fs(lat->nfields);
     for (int f = 0; f < lat->nfields; ++f) {
+        fs[f].keep_fp64 = keep_fp64;
         fs[f].U = (char*)U + eb * link_elems(g) * f;
         fs[f].G = (char*)G + eb * gauge_elems(g) * f;
         fs[f].g = g;
@@ -753,6 +758,9 @@ int mcg_precondition_fix(void* U, void* G, int8_t* Z, const mcg_lattice* lat, co
     int status = MCG_OK;
     const double norm = 1.0 / (9.0 * 8.0 * g.vh);
     if ((rc = launch_identity_gauge(G, prec, g, nf, stream))) return rc;
+    // the second fix starts with an FP32 phase (or is FP32): what leads to it
+    // stays in FP64 arithmetic
+    const bool keep = prec == MCG_F32 || params->fp32_sweeps > 0;
     if (nsmear > 0) {
         // S = smear(U) in the smear precision; the smeared field is then fixed
         // in the field's precision with the caller's schedule (transform W)
@@ -770,18 +778,19 @@ int mcg_precondition_fix(void* U, void* G, int8_t* Z, const mcg_lattice* lat, co
             if ((rc = launch_convert(U, prec, Uc, smear_precision, le * nf, stream))) return rc;
             src = Uc;
         }
-        if ((rc = run_smear(src, S, smear_precision, g, nf, rho, eps, nsmear, stream))) return rc;
+        if ((rc = run_smear(src, S, smear_precision, g, nf, rho, eps, nsmear, stream, keep))) return rc;
         if ((rc = launch_convert(S, smear_precision, Sp, prec, le * nf, stream))) return rc;
         if (smear_precision != prec && (rc = launch_reunitarise(Sp, 0, prec, g, nf, stream))) return rc;
         if ((rc = launch_identity_gauge(W, prec, g, nf, stream))) return rc;
         rc = fix_impl(Sp, W, lat, g, params, Rs.data(), sw_s.data(), sw32_s.data(), nullptr, stream, conv_s.data(),
-                      rs_s.data());
+                      rs_s.data(), keep);
         if (rc != MCG_OK && rc != MCG_NOT_CONVERGED) return rc;
         if (rc == MCG_NOT_CONVERGED) status = MCG_NOT_CONVERGED;
         // G <- reunit(W), then U <- U^G (the preconditioning transform)
         MCG_CK(cudaMemcpyAsync(G, W, eb * ge * nf, cudaMemcpyDeviceToDevice, stream));
         if ((rc = launch_reunitarise(G, 1, prec, g, nf, stream))) return rc;
-        if ((rc = launch_apply_gauge(U, G, prec, g, nf, stream))) return rc;
+        if ((rc = keep ? launch_apply_gauge(U, G, prec, g, nf, stream) : launch_apply_gauge_fx(U, G, g, nf, stream)))
+            return rc;
     }
     // fix the preconditioned original field, accumulating into G
     rc = fix_impl(U, G, lat, g, params, Rf.data(), sw_f.data(), sw32_f.data(), nullptr, stream, conv_f.data(),
@@ -823,7 +832,7 @@ long long mcg_bounds_violations(int reset) {
 #ifdef MCG_CHECK
     cudaDeviceSynchronize();
     const bool r = reset != 0;
-    return (long long)(bound_hits_field(r) + bound_hits_observables(r) + bound_hits_smear(r) + bound_hits_smear_fx(r) +
+    return (long long)(bound_hits_field(r) + bound_hits_field_fx(r) + bound_hits_observables(r) + bound_hits_smear(r) + bound_hits_smear_fx(r) +
                        bound_hits_sweep(r) + bound_hits_sweep_f32(r) + bound_hits_sweep_fx(r) +
                        bound_hits_sweep_df(r));
 #else
@@ -948,6 +957,7 @@ int mcg_precondition_levels(const void* U, void* U_out, void* G_out, int8_t* Z_o
     for (int l = 0; l < nlevels; ++l)
         MCG_CK(cudaMemcpyAsync((char*)U_out + eb * le * l, U, eb * le, cudaMemcpyDeviceToDevice, stream));
     if ((rc = launch_identity_gauge(G_out, prec, g, nlevels, stream))) return rc;
+    const bool keep = prec == MCG_F32 || params->fp32_sweeps > 0;  // as in mcg_precondition_fix
     void* Sp = nullptr;  // the smeared fields, then their transforms
     void* W = nullptr;
     if (ns > 0) {
@@ -964,7 +974,7 @@ int mcg_precondition_levels(const void* U, void* U_out, void* G_out, int8_t* Z_o
         for (int k = 0; k < ns; ++k) {
             const int steps = nsmear[smeared[k]] - done_steps;
             if (steps > 0) {
-                if ((rc = run_smear(cur, tmp, smear_precision, g, 1, rho, eps, steps, stream))) return rc;
+                if ((rc = run_smear(cur, tmp, smear_precision, g, 1, rho, eps, steps, stream, keep))) return rc;
                 std::swap(cur, tmp);
                 done_steps += steps;
             }
@@ -979,7 +989,7 @@ int mcg_precondition_levels(const void* U, void* U_out, void* G_out, int8_t* Z_o
     // does not depend on the batch.
     std::vector<FieldSpec> b1, b2;
     std::vector<int> plain_levels;
-    for (int k = 0; k < ns; ++k) b1.push_back({(char*)Sp + eb * le * k, (char*)W + eb * ge * k, g});
+    for (int k = 0; k < ns; ++k) b1.push_back({(char*)Sp + eb * le * k, (char*)W + eb * ge * k, g, keep});
     for (int l = 0; l < nlevels; ++l)
         if (nsmear[l] == 0) {
             b1.push_back({(char*)U_out + eb * le * l, (char*)G_out + eb * ge * l, g});
@@ -1015,7 +1025,8 @@ int mcg_precondition_levels(const void* U, void* U_out, void* G_out, int8_t* Z_o
             char* Ul = (char*)U_out + eb * le * smeared[k];
             MCG_CK(cudaMemcpyAsync(Gl, (char*)W + eb * ge * k, eb * ge, cudaMemcpyDeviceToDevice, stream));
             if ((rc = launch_reunitarise(Gl, 1, prec, g, 1, stream))) return rc;
-            if ((rc = launch_apply_gauge(Ul, Gl, prec, g, 1, stream))) return rc;
+            if ((rc = keep ? launch_apply_gauge(Ul, Gl, prec, g, 1, stream) : launch_apply_gauge_fx(Ul, Gl, g, 1, stream)))
+                return rc;
             b2.push_back({Ul, Gl, g});
         }
         std::vector<double> R2(ns);
@@ -1097,8 +1108,11 @@ int mcg_gribov_search(const mcg_field* copies, int ncopies, const int* config_of
             return rc;
     // each copy starts as U^Omega0 with its own random Omega0; the fix then
     // accumulates onto Omega0, so G ends as the total transform of the copy
+    const bool keep = precision == MCG_F32 || params->fp32_sweeps > 0;  // the copies start an FP32 phase
     for (int f = 0; f < ncopies; ++f)
-        if ((rc = launch_apply_gauge(fs[f].U, fs[f].G, precision, fs[f].g, 1, stream))) return rc;
+        if ((rc = keep ? launch_apply_gauge(fs[f].U, fs[f].G, precision, fs[f].g, 1, stream)
+                       : launch_apply_gauge_fx(fs[f].U, fs[f].G, fs[f].g, 1, stream)))
+            return rc;
     std::vector<double> R(ncopies);
     std::vector<int> sw(ncopies);
     int st = fix_fields(fs, precision, params, R.data(), sw.data(), nullptr, nullptr, stream);

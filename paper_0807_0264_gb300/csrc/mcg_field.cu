@@ -1,5 +1,6 @@
 // Field-level kernels: layout conversion, gauge transforms, re-unitarisation,
-// plaquette, the MCG functional, Z3 center projection and P-vortex counting.
+// the MCG functional, Z3 center projection and P-vortex counting (the plaquette
+// and the gauge transforms in fixed point: mcg_field_fx.cu).
 // All are HBM-bound streaming kernels (one thread per site of one parity).
 #include <cuda_runtime.h>
 
@@ -301,60 +302,8 @@ __global__ void __launch_bounds__(FT) k_identity_c12(float4* __restrict__ W, Geo
 }
 
 // ---------------------------------------------------------------------------
-// plaquette and functional: per-field sums via per-block partials
+// functional: per-field sums via per-block partials
 // ---------------------------------------------------------------------------
-template <typename T>
-__global__ void __launch_bounds__(FT) k_plaquette(const cplx<T>* __restrict__ U, Geom g, int bpf,
-                                                  double* __restrict__ partial) {
-    const int f = blockIdx.x / bpf;
-    const int s2 = (blockIdx.x - f * bpf) * FT + threadIdx.x;  // 0 .. 2*vh-1
-    const cplx<T>* Uf = U + (size_t)f * link_elems(g);
-    double acc = 0.0;
-    if (s2 < 2 * g.vh) {
-        const int p = s2 / g.vh, s = s2 - p * g.vh;
-        int c[4];
-        eo_coords(g, p, s, c);
-        for (int mu = 0; mu < 4; ++mu) {
-            const int smu = eo_neighbor(g, c, mu, +1);
-            cplx<double> a[9], t[9];
-#pragma unroll
-            for (int e = 0; e < 9; ++e) {
-                const cplx<T> v = Uf[lidx(g, mu, p, e, s)];
-                a[e] = mk((double)v.x, (double)v.y);
-            }
-            for (int nu = mu + 1; nu < 4; ++nu) {
-                const int snu = eo_neighbor(g, c, nu, +1);
-                cplx<double> b[9], m[9], q[9];
-#pragma unroll
-                for (int e = 0; e < 9; ++e) {
-                    const cplx<T> v = Uf[lidx(g, nu, p ^ 1, e, smu)];
-                    b[e] = mk((double)v.x, (double)v.y);
-                }
-                m3_mul(a, b, t);  // U_mu(x) U_nu(x+mu)
-#pragma unroll
-                for (int e = 0; e < 9; ++e) {
-                    const cplx<T> v = Uf[lidx(g, mu, p ^ 1, e, snu)];
-                    m[e] = mk((double)v.x, (double)v.y);
-                }
-                m3_mul_nd(t, m, q);  // ... U_mu(x+nu)^dag
-#pragma unroll
-                for (int e = 0; e < 9; ++e) {
-                    const cplx<T> v = Uf[lidx(g, nu, p, e, s)];
-                    m[e] = mk((double)v.x, (double)v.y);
-                }
-                // Re tr(q m^dag) = sum_ij Re(q_ij conj(m_ij))
-                double tr = 0.0;
-#pragma unroll
-                for (int e = 0; e < 9; ++e) tr += q[e].x * m[e].x + q[e].y * m[e].y;
-                acc += tr / 3.0;
-            }
-        }
-    }
-    __shared__ double red[FT / 32];
-    const double tot = block_sum(acc, red);
-    if (threadIdx.x == 0) partial[blockIdx.x] = tot;
-}
-
 template <typename T>
 __global__ void __launch_bounds__(FT) k_functional_all(const cplx<T>* __restrict__ U, Geom g, int bpf,
                                                        double* __restrict__ partial) {
@@ -726,10 +675,7 @@ static int reduce_per_field(int which, const void* U, int prec, const Geom& g, i
     if (rc) return rc;
     const int nb = bpf * nfields;
     if (which == 0) {
-        if (prec == MCG_F64)
-            k_plaquette<double><<<nb, FT, 0, st>>>((const cplx<double>*)U, g, bpf, partial);
-        else
-            k_plaquette<float><<<nb, FT, 0, st>>>((const cplx<float>*)U, g, bpf, partial);
+        launch_plaquette_partials(U, prec, g, bpf, nfields, partial, st);
     } else {
         if (prec == MCG_F64)
             k_functional_all<double><<<nb, FT, 0, st>>>((const cplx<double>*)U, g, bpf, partial);
@@ -782,7 +728,8 @@ int compute_center(const void* U, int prec, int8_t* Z, const Geom& g, int nfield
 }
 
 int launch_handoff(const void* W32, const void* W32lo, double* U64, double* G64, const Geom& g, int nfields,
-                   cudaStream_t st) {
+                   bool keep_fp64, cudaStream_t st) {
+    if (!keep_fp64) return launch_handoff_fx(W32, W32lo, U64, G64, g, nfields, st);
     int rc = 0;
     cplx<double>* W64 =
         (cplx<double>*)scratch_device("handoff.W64", sizeof(cplx<double>) * gauge_elems(g) * nfields, &rc);
@@ -899,11 +846,7 @@ extern "C" int mcg_plaquette_static(const void* U, double* out, const mcg_lattic
     if ((rc = static_partials_address(&partial))) return rc;
     // every partial slot read below is written by its block first: nothing in
     // the shared array has to start at zero
-    const int nb = (int)bpf * lat->nfields;
-    if (lat->precision == MCG_F64)
-        k_plaquette<double><<<nb, FT, 0, stream>>>((const cplx<double>*)U, g, (int)bpf, partial);
-    else
-        k_plaquette<float><<<nb, FT, 0, stream>>>((const cplx<float>*)U, g, (int)bpf, partial);
+    launch_plaquette_partials(U, lat->precision, g, (int)bpf, lat->nfields, partial, stream);
     k_static_finish<<<lat->nfields, 256, 0, stream>>>(partial, (int)bpf, 1.0 / (6.0 * (double)V), out);
     MCG_CK(cudaGetLastError());
     note_launches(2);

@@ -1,0 +1,265 @@
+// Field kernels in fixed-point arithmetic (mcg_fx.cuh): gauge transforms of FP64
+// fields, the mixed-precision hand-off and the plaquette.  Fields of these entry
+// points are not always validated: a thread that meets a matrix that is not
+// near-unitary does its link or plaquette in FP64.
+//
+// A transformed field that an FP32 phase starts from keeps the FP64 kernels of
+// mcg_field.cu: the over-relaxed FP32 sweeps of an unfixed field follow the last
+// bit of their input (one entry rounded the other way moved the links of a
+// 20^3 x 40 field by 1.4e-7 after 150 sweeps), so those results stay what they
+// were.
+#include <cuda_runtime.h>
+
+#include "mcg_common.cuh"
+#include "mcg_fx.cuh"
+#include "mcg_internal.h"
+
+namespace mcg {
+
+namespace {
+
+template <typename T>
+struct Vec2;
+template <>
+struct Vec2<double> {
+    typedef double2 type;
+};
+template <>
+struct Vec2<float> {
+    typedef float2 type;
+};
+
+inline unsigned blocks(long long n, int nt) { return (unsigned)((n + nt - 1) / nt); }
+
+// ---- gauge transform: U_mu(x) <- Omega(x) U_mu(x) Omega(x+mu)^dag ----------------
+__device__ __noinline__ void apply_link_f64(double2* u, const double2* w, const double2* wf, size_t vh) {
+    cplx<double> a[9], b[9], t[9];
+#pragma unroll
+    for (int e = 0; e < 9; ++e) {
+        a[e] = mk(w[e * vh].x, w[e * vh].y);
+        b[e] = mk(u[e * vh].x, u[e * vh].y);
+    }
+    m3_mul(a, b, t);
+#pragma unroll
+    for (int e = 0; e < 9; ++e) b[e] = mk(wf[e * vh].x, wf[e * vh].y);
+    m3_mul_nd(t, b, a);
+#pragma unroll
+    for (int e = 0; e < 9; ++e) u[e * vh] = make_double2(a[e].x, a[e].y);
+}
+
+// One thread per link.  WFX: the transform in fixed point, of an SU(3) field (the
+// hand-off).  Two products and 18 to 54 conversions per link, bound by the
+// integer multiplier.  A thread per link: the products need no more registers
+// than three blocks of 128 per SM leave, and small lattices fill more SMs.
+template <bool WFX>
+__global__ void __launch_bounds__(128, 3) k_apply_gauge_fx(double2* Uall, const void* Gall, Geom g, int nfields) {
+    const long long id = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (id >= 8LL * g.vh * nfields) return;
+    const int f = (int)(id / (8LL * g.vh));
+    int r = (int)(id - (long long)f * 8 * g.vh);
+    const int mu = r / (2 * g.vh);
+    r -= mu * 2 * g.vh;
+    const int p = r / g.vh, s = r - p * g.vh;
+    const size_t vh = (size_t)g.vh;
+    int c[4];
+    eo_coords(g, p, s, c);
+    const size_t iw = (size_t)f * gauge_elems(g) + gidx(g, p, 0, s);
+    const size_t iwf = (size_t)f * gauge_elems(g) + gidx(g, p ^ 1, 0, eo_neighbor(g, c, mu, +1));
+    double2* u = Uall + (size_t)f * link_elems(g) + lidx(g, mu, p, 0, s);
+    cfx a[9], b[9];
+    bool bad = false;
+    if (WFX) {
+        const int4* w = reinterpret_cast<const int4*>(Gall) + iw;
+#pragma unroll
+        for (int e = 0; e < 9; ++e) a[e] = fx_load(w + e * vh);
+    } else {
+        bad = fx_load_matrix(reinterpret_cast<const double2*>(Gall) + iw, 3 * vh, vh, a);
+    }
+    const bool ubad = fx_load_matrix(u, 3 * vh, vh, b);
+    if (!WFX) bad = bad || ubad;
+    m3fx_mul_inplace<false>(a, b);
+    if (WFX) {
+        const int4* w = reinterpret_cast<const int4*>(Gall) + iwf;
+#pragma unroll
+        for (int e = 0; e < 9; ++e) b[e] = fx_load(w + e * vh);
+    } else {
+        bad = fx_load_matrix(reinterpret_cast<const double2*>(Gall) + iwf, 3 * vh, vh, b) || bad;
+    }
+    if (!WFX && bad) {
+        apply_link_f64(u, reinterpret_cast<const double2*>(Gall) + iw, reinterpret_cast<const double2*>(Gall) + iwf, vh);
+        return;
+    }
+    m3fx_mul_inplace<true>(a, b);
+#pragma unroll
+    for (int e = 0; e < 9; ++e) fx_store(u + e * vh, a[e]);
+}
+
+// ---- hand-off of the mixed schedule, pass 1 --------------------------------------
+// W (compact: rows 0 and 1, FP32 or hi + lo) re-unitarised, to scratch in fixed
+// point; Omega <- reunit(W Omega).  W is unitary to FP32 rounding, Omega a
+// validated transform.
+__global__ void __launch_bounds__(128, 3) k_handoff_gauge_fx(const float4* __restrict__ W,
+                                                              const float4* __restrict__ Wlo, int4* __restrict__ Wfx,
+                                                              double2* __restrict__ G, Geom g, int nfields) {
+    const long long n = 2LL * g.vh * nfields;
+    const long long id = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (id >= n) return;
+    const int f = (int)(id / (2LL * g.vh));
+    const int r = (int)(id - (long long)f * 2 * g.vh);
+    const int p = r / g.vh, s = r - p * g.vh;
+    const size_t off = (size_t)f * gauge_elems(g) + gidx(g, p, 0, s), vh = (size_t)g.vh;
+    const size_t coff = (size_t)f * c12_gauge_chunks(g) + c12_gidx(g, p, 0, s);
+    cfx w[9], o[9];
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+        const float4 v = W[coff + q * vh];
+        w[2 * q].re = fx_of(v.x);
+        w[2 * q].im = fx_of(v.y);
+        w[2 * q + 1].re = fx_of(v.z);
+        w[2 * q + 1].im = fx_of(v.w);
+        if (Wlo) {
+            const float4 l = Wlo[coff + q * vh];
+            w[2 * q].re = fx_split(fx_join(w[2 * q].re) + fx_join(fx_of(l.x)));
+            w[2 * q].im = fx_split(fx_join(w[2 * q].im) + fx_join(fx_of(l.y)));
+            w[2 * q + 1].re = fx_split(fx_join(w[2 * q + 1].re) + fx_join(fx_of(l.z)));
+            w[2 * q + 1].im = fx_split(fx_join(w[2 * q + 1].im) + fx_join(fx_of(l.w)));
+        }
+    }
+    m3fx_reunitarise(w);
+#pragma unroll
+    for (int e = 0; e < 9; ++e) {
+        Wfx[off + e * vh] = fx_pack(w[e]);
+        const double2 v = G[off + e * vh];
+        o[e].re = fx_of(v.x);
+        o[e].im = fx_of(v.y);
+    }
+    m3fx_mul_inplace<false>(w, o);
+    m3fx_reunitarise(w);
+#pragma unroll
+    for (int e = 0; e < 9; ++e) fx_store(G + off + e * vh, w[e]);
+}
+
+// ---- plaquette -------------------------------------------------------------------
+template <typename V>
+__device__ __noinline__ double plaquette_f64(const V* a, const V* b, const V* c, const V* d, size_t vh) {
+    cplx<double> x[9], y[9], t[9], q[9];
+#pragma unroll
+    for (int e = 0; e < 9; ++e) {
+        x[e] = mk((double)a[e * vh].x, (double)a[e * vh].y);
+        y[e] = mk((double)b[e * vh].x, (double)b[e * vh].y);
+    }
+    m3_mul(x, y, t);
+#pragma unroll
+    for (int e = 0; e < 9; ++e) y[e] = mk((double)c[e * vh].x, (double)c[e * vh].y);
+    m3_mul_nd(t, y, q);
+    double tr = 0.0;
+#pragma unroll
+    for (int e = 0; e < 9; ++e) tr += q[e].x * (double)d[e * vh].x + q[e].y * (double)d[e * vh].y;
+    return tr;
+}
+
+// Per-block partial of the sum over sites of (1/3) Re tr of the six plaquettes:
+// X = U_mu(x) U_nu(x+mu) and Y = U_nu(x) U_mu(x+nu) row by row, sum Re X Y^*.
+// bpf blocks of 256 sites per field.  Measured on 20^3 x 40: 353 us (the FP64
+// kernel 917 us, FP64 pipe 93 %); one block per SM instead of two: 412 us.
+template <typename T>
+__global__ void __launch_bounds__(256, 2) k_plaquette_fx(const void* Uall, Geom g, int bpf,
+                                                         double* __restrict__ partial) {
+    typedef typename Vec2<T>::type V;
+    const int f = blockIdx.x / bpf;
+    const int s2 = (blockIdx.x - f * bpf) * 256 + threadIdx.x;  // 0 .. 2*vh-1
+    const V* U = reinterpret_cast<const V*>(Uall) + (size_t)f * link_elems(g);
+    const size_t vh = (size_t)g.vh;
+    double slow = 0.0;
+    long long acc = 0;  // units of 2^-57: at most 6 * 3.2
+    if (s2 < 2 * g.vh) {
+        const int p = s2 / g.vh, s = s2 - p * g.vh;
+        int c[4];
+        eo_coords(g, p, s, c);
+#pragma unroll 1
+        for (int mu = 0; mu < 3; ++mu) {
+            const int smu = eo_neighbor(g, c, mu, +1);
+#pragma unroll 1
+            for (int nu = mu + 1; nu < 4; ++nu) {
+                const V* ua = U + lidx(g, mu, p, 0, s);
+                const V* ub = U + lidx(g, nu, p ^ 1, 0, smu);
+                const V* uc = U + lidx(g, mu, p ^ 1, 0, eo_neighbor(g, c, nu, +1));
+                const V* ud = U + lidx(g, nu, p, 0, s);
+                cfx b[9], m[9];
+                bool bad = fx_load_matrix(ub, 3 * vh, vh, b);
+                bad = fx_load_matrix(uc, 3 * vh, vh, m) || bad;
+                facc t = facc_zero();
+#pragma unroll 1
+                for (int i = 0; i < 3; ++i) {
+                    cfx ra[3], rd[3], x[3], y[3];
+                    float na = 0.f, nd = 0.f;
+                    unsigned big = 0;
+#pragma unroll
+                    for (int k = 0; k < 3; ++k) {
+                        const V va = ua[(3 * i + k) * vh], vd = ud[(3 * i + k) * vh];
+                        big = max(max(big, max(fx_magnitude(va.x), fx_magnitude(va.y))),
+                                  max(fx_magnitude(vd.x), fx_magnitude(vd.y)));
+                        ra[k].re = fx_of(va.x);
+                        ra[k].im = fx_of(va.y);
+                        rd[k].re = fx_of(vd.x);
+                        rd[k].im = fx_of(vd.y);
+                        na = fmaf((float)ra[k].re.h, (float)ra[k].re.h, fmaf((float)ra[k].im.h, (float)ra[k].im.h, na));
+                        nd = fmaf((float)rd[k].re.h, (float)rd[k].re.h, fmaf((float)rd[k].im.h, (float)rd[k].im.h, nd));
+                    }
+                    bad = bad || big > kFxMagnitude || !(fabsf(na * 0x1p-56f - 1.f) < 0.05f) ||
+                          !(fabsf(nd * 0x1p-56f - 1.f) < 0.05f);
+                    m3fx_row<false>(ra, b, x);
+                    m3fx_row<false>(rd, m, y);
+#pragma unroll
+                    for (int k = 0; k < 3; ++k) {
+                        fx_mac(t, x[k].re, y[k].re);
+                        fx_mac(t, x[k].im, y[k].im);
+                    }
+                }
+                if (bad)
+                    slow += plaquette_f64(ua, ub, uc, ud, vh);
+                else
+                    acc += facc_get(t) >> 3;
+            }
+        }
+    }
+    __shared__ double red[8];
+    const double tot = block_sum((fx_double(acc) * 8.0 + slow) / 3.0, red);
+    if (threadIdx.x == 0) partial[blockIdx.x] = tot;
+}
+
+}  // namespace
+
+int launch_apply_gauge_fx(void* U, const void* G, const Geom& g, int nfields, cudaStream_t st) {
+    k_apply_gauge_fx<false><<<blocks(8LL * g.vh * nfields, 128), 128, 0, st>>>((double2*)U, G, g, nfields);
+    MCG_CK(cudaGetLastError());
+    note_launches(1);
+    return 0;
+}
+
+int launch_handoff_fx(const void* W32, const void* W32lo, double* U64, double* G64, const Geom& g, int nfields,
+                      cudaStream_t st) {
+    int rc = 0;
+    int4* Wfx = (int4*)scratch_device("handoff.W64", sizeof(int4) * gauge_elems(g) * nfields, &rc);
+    if (rc) return rc;
+    k_handoff_gauge_fx<<<blocks(2LL * g.vh * nfields, 128), 128, 0, st>>>(
+        (const float4*)W32, (const float4*)W32lo, Wfx, (double2*)G64, g, nfields);
+    k_apply_gauge_fx<true><<<blocks(8LL * g.vh * nfields, 128), 128, 0, st>>>((double2*)U64, Wfx, g, nfields);
+    MCG_CK(cudaGetLastError());
+    note_launches(2);
+    return 0;
+}
+
+void launch_plaquette_partials(const void* U, int prec, const Geom& g, int bpf, int nfields, double* partial,
+                               cudaStream_t st) {
+    const unsigned nb = (unsigned)bpf * nfields;
+    if (prec == MCG_F64)
+        k_plaquette_fx<double><<<nb, 256, 0, st>>>(U, g, bpf, partial);
+    else
+        k_plaquette_fx<float><<<nb, 256, 0, st>>>(U, g, bpf, partial);
+}
+
+// index-check counter of this unit (MCG_CHECK builds)
+MCG_BOUND_READER(bound_hits_field_fx)
+
+}  // namespace mcg

@@ -30,6 +30,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "mcg_common.cuh"
+
 namespace mcg {
 
 #define MCG_HD __host__ __device__ __forceinline__
@@ -117,28 +119,6 @@ __device__ __forceinline__ fx fx_of(double d) { return fx_split(fx_from_bits((un
 __device__ __forceinline__ double fx_double(long long X) { return __longlong_as_double((long long)fx_to_bits(X)); }
 #endif
 
-#ifdef __CUDACC__
-// A matrix (entry (r, k) at src[r sr + k sc]) the fixed-point sweep does not
-// take: an entry above 1.03 in magnitude or not finite, or a row whose squared
-// norm is off 1 by 5 % (tiny rows would lose relative precision).
-__device__ __forceinline__ bool fx_bad_matrix(const double2* src, size_t sr, size_t sc) {
-    bool bad = false;
-#pragma unroll 1
-    for (int r = 0; r < 3; ++r) {
-        float n2 = 0.f;
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            const double2 d = src[r * sr + k * sc];
-            bad = bad || (__double2hiint(d.x) & 0x7fffffff) > 0x3ff07ae1 || (__double2hiint(d.y) & 0x7fffffff) > 0x3ff07ae1;
-            const float x = (float)fx_of(d.x).h, y = (float)fx_of(d.y).h;  // unit 2^-28
-            n2 = fmaf(x, x, fmaf(y, y, n2));
-        }
-        bad = bad || !(fabsf(n2 * 0x1p-56f - 1.f) < 0.05f);
-    }
-    return bad;
-}
-#endif
-
 // ---- 3 x 3 complex matrices (row-major) ---------------------------------------
 MCG_HD void cfx_mac(facc& re, facc& im, cfx a, cfx b) {
     fx_mac(re, a.re, b.re);
@@ -186,5 +166,143 @@ MCG_HD void m3fx_mul_inplace(cfx* a, const cfx* b) {
         for (int j = 0; j < 3; ++j) a[3 * i + j] = t[j];
     }
 }
+
+// ---- near-unitary matrices: re-unitarisation -----------------------------------
+// 1 / sqrt(1 + d) - 1 for |d| < 2^-12, both in units of 2^-60: the binomial series
+// to d^4 (the next term is below 2^-62)
+MCG_HD long long fx_rsqrt1(long long d) {
+    const fx s = fx_split(d);
+    long long e = fx_mul(s, fx_split(35LL << 53)) - (5LL << 56);
+    e = fx_mul(s, fx_split(e)) + (3LL << 57);
+    e = fx_mul(s, fx_split(e)) - (1LL << 59);
+    return fx_mul(s, fx_split(e));
+}
+MCG_HD long long fx_row_norm2(const cfx* r) {
+    facc n = facc_zero();
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        fx_mac(n, r[k].re, r[k].re);
+        fx_mac(n, r[k].im, r[k].im);
+    }
+    return facc_get(n);
+}
+MCG_HD void fx_scale_row(cfx* r, long long e) {  // r += e r
+    const fx s = fx_split(e);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        r[k].re = fx_split(fx_join(r[k].re) + fx_mul(s, r[k].re));
+        r[k].im = fx_split(fx_join(r[k].im) + fx_mul(s, r[k].im));
+    }
+}
+MCG_HD bool fx_far(long long d) { return d > (1LL << 48) || d < -(1LL << 48); }
+// Row 0 normalised, row 1 orthogonalised and normalised, row 2 = conj(row0 x
+// row1), as m3_reunitarise.  True (and m undefined) when a norm is off 1 by more
+// than 2^-12: the caller takes the FP64 form.
+MCG_HD bool m3fx_reunitarise(cfx* m) {
+    const long long one = 1LL << 60, d0 = fx_row_norm2(m) - one;
+    fx_scale_row(m, fx_rsqrt1(d0));
+    facc px = facc_zero(), py = facc_zero();  // conj(r0) . r1
+#pragma unroll
+    for (int k = 0; k < 3; ++k) cfx_macc(px, py, m[3 + k], m[k]);
+    const fx qx = fx_split(facc_get(px)), qy = fx_split(facc_get(py));
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        facc x = facc_zero(), y = facc_zero();
+        cfx p;
+        p.re = qx;
+        p.im = qy;
+        cfx_mac(x, y, p, m[k]);
+        m[3 + k].re = fx_split(fx_join(m[3 + k].re) - facc_get(x));
+        m[3 + k].im = fx_split(fx_join(m[3 + k].im) - facc_get(y));
+    }
+    const long long d1 = fx_row_norm2(m + 3) - one;
+    fx_scale_row(m + 3, fx_rsqrt1(d1));
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const int i = (k + 1) % 3, j = (k + 2) % 3;
+        facc x = facc_zero(), y = facc_zero(), u = facc_zero(), v = facc_zero();
+        cfx_mac(x, y, m[i], m[3 + j]);
+        cfx_mac(u, v, m[j], m[3 + i]);
+        m[6 + k].re = fx_split(facc_get(x) - facc_get(u));
+        m[6 + k].im = fx_split(facc_get(v) - facc_get(y));
+    }
+    return fx_far(d0) || fx_far(d1);
+}
+
+#ifdef __CUDACC__
+// ---- loads of FP64 and FP32 matrices ---------------------------------------------
+// Matrices the fixed-point kernels do not take (callers' unvalidated fields): an
+// entry above 1.03 in magnitude or not finite, or a row whose squared norm is
+// off 1 by 5 % (tiny rows would lose relative precision).
+__device__ __forceinline__ unsigned fx_magnitude(double d) { return __double2hiint(d) & 0x7fffffff; }
+__device__ __forceinline__ unsigned fx_magnitude(float f) {  // as the high word of the same double, roughly
+    return ((__float_as_uint(f) & 0x7fffffff) >> 3) + 0x38000000u;
+}
+__device__ __forceinline__ fx fx_of(float f) {
+    const float s = f * 0x1p28f;
+    const int h = __float2int_rn(s);
+    return fx_split(((long long)h << 32) + 2 * (long long)__float2int_rn((s - (float)h) * 0x1p31f));
+}
+constexpr unsigned kFxMagnitude = 0x3ff07ae1;  // 1.03
+__device__ __forceinline__ bool fx_bad_rows(const cfx* m) {
+    bool bad = false;
+#pragma unroll
+    for (int r = 0; r < 3; ++r) {
+        float n2 = 0.f;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const float x = (float)m[3 * r + k].re.h, y = (float)m[3 * r + k].im.h;  // unit 2^-28
+            n2 = fmaf(x, x, fmaf(y, y, n2));
+        }
+        bad = bad || !(fabsf(n2 * 0x1p-56f - 1.f) < 0.05f);
+    }
+    return bad;
+}
+// entry (r, k) at src[r sr + k sc] to m; true: not near-unitary
+template <typename C>
+__device__ __forceinline__ bool fx_load_matrix(const C* __restrict__ src, size_t sr, size_t sc, cfx* m) {
+    unsigned big = 0;
+#pragma unroll
+    for (int r = 0; r < 3; ++r)
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const C d = src[r * sr + k * sc];
+            big = max(big, max(fx_magnitude(d.x), fx_magnitude(d.y)));
+            m[3 * r + k].re = fx_of(d.x);
+            m[3 * r + k].im = fx_of(d.y);
+        }
+    return big > kFxMagnitude || fx_bad_rows(m);
+}
+__device__ __forceinline__ bool fx_bad_matrix(const double2* src, size_t sr, size_t sc) {
+    cfx m[9];
+    return fx_load_matrix(src, sr, sc, m);
+}
+// X 2^-60 rounded to FP32 (ties away from zero)
+__device__ __forceinline__ float fx_single(long long X) {
+    const long long sg = X >> 63;
+    const unsigned long long m = (unsigned long long)((X ^ sg) - sg);
+    const int z = __clzll((long long)m);
+    const unsigned t = (unsigned)((z > 0 ? m << ((z - 1) & 63) : m >> 1) >> 32);  // top bit 30
+    // the bits below the upper word only matter for a tie, which then rounds up as well
+    const unsigned q = ((t + (1u << 6)) >> 7) + ((unsigned)(129 - z) << 23);
+    return __uint_as_float(X == 0 ? 0u : (q | ((unsigned)sg & 0x80000000u)));
+}
+__device__ __forceinline__ void fx_store(double2* p, cfx v) {
+    *p = make_double2(fx_double(fx_join(v.re)), fx_double(fx_join(v.im)));
+}
+__device__ __forceinline__ void fx_store(float2* p, cfx v) {
+    *p = make_float2(fx_single(fx_join(v.re)), fx_single(fx_join(v.im)));
+}
+__device__ __forceinline__ cfx fx_load(const int4* p) {
+    const int4 v = *p;
+    cfx r;
+    r.re.h = v.x;
+    r.re.l = v.y;
+    r.im.h = v.z;
+    r.im.l = v.w;
+    return r;
+}
+__device__ __forceinline__ int4 fx_pack(cfx a) { return make_int4(a.re.h, a.re.l, a.im.h, a.im.l); }
+#endif
 
 }  // namespace mcg

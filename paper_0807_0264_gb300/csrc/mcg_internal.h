@@ -52,6 +52,7 @@ cudaStream_t capture_stream(int* rc);
 int branch_streams(int n, cudaStream_t* streams, cudaEvent_t* events, cudaEvent_t* fork, int* rc);
 // index-check counters of the kernel units (0 unless built with MCG_CHECK)
 unsigned long long bound_hits_field(bool reset);
+unsigned long long bound_hits_field_fx(bool reset);
 unsigned long long bound_hits_observables(bool reset);
 unsigned long long bound_hits_smear(bool reset);
 unsigned long long bound_hits_smear_fx(bool reset);
@@ -164,12 +165,13 @@ inline double restart_omega(double omega, double domega, int k) {
 // field is done: converged (dV_U < tol) or at abs_cap sweeps counted from the
 // start of the history.  `fresh`: start a new history (sweep = 0); otherwise
 // continue the sweep count in `state` (a new phase).  restart (T = float
-// only, may be null): see PhaseRestart.  Returns 0 or an error.
+// only, may be null): see PhaseRestart.  keep_fp64 (T = double): the FP64 kernel
+// in place of the fixed-point one.  Returns 0 or an error.
 template <typename T>
 int run_fix_phase(const std::vector<FieldDesc>& fields, FieldState* d_state, FieldState* h_state, double* d_hist,
                   int hist_len, double tol, int window, double omega, int reunit_every, int abs_cap,
                   int check_every, bool fresh, cudaStream_t stream, bool solve32 = false,
-                  const PhaseRestart* restart = nullptr);
+                  const PhaseRestart* restart = nullptr, bool keep_fp64 = false);
 
 // Time `nreps` launches of one half-sweep kernel (parity 1 includes the fused
 // R reduction) on a single field, each bracketed by CUDA events on `stream`;
@@ -254,15 +256,24 @@ int launch_convert(const void* src, int src_prec, void* dst, int dst_prec, size_
 int launch_identity_gauge(void* G, int prec, const Geom& g, int nfields, cudaStream_t st);
 int launch_apply_gauge(void* U, const void* G, int prec, const Geom& g, int nfields, cudaStream_t st);
 int launch_reunitarise(void* M, int which, int prec, const Geom& g, int nfields, cudaStream_t st);
+// the same for FP64 fields in fixed point (mcg_field_fx.cu)
+int launch_apply_gauge_fx(void* U, const void* G, const Geom& g, int nfields, cudaStream_t st);
+// sums over sites of (1/3) Re tr of the six plaquettes, one per block of 256
+// sites, bpf blocks per field
+void launch_plaquette_partials(const void* U, int prec, const Geom& g, int bpf, int nfields, double* partial,
+                               cudaStream_t st);
 int compute_plaquette(const void* U, int prec, const Geom& g, int nfields, double* out_host, cudaStream_t st);
 int compute_functional(const void* U, int prec, const Geom& g, int nfields, double* out_host, cudaStream_t st);
 int compute_center(const void* U, int prec, int8_t* Z, const Geom& g, int nfields, long long* counts_host,
                    cudaStream_t st);
 // FP32 transform W of this call (compact form) -> FP64: W64 = reunit(W);
 // U64 <- W64 U64 W64(x+mu)^dag; G64 <- reunit(W64 G64).  W32lo (may be null):
-// lo parts of a double-float W (W = hi + lo).
+// lo parts of a double-float W (W = hi + lo).  keep_fp64: in FP64 (a later FP32
+// phase starts from the result), else in fixed point.
 int launch_handoff(const void* W32, const void* W32lo, double* U64, double* G64, const Geom& g, int nfields,
-                   cudaStream_t st);
+                   bool keep_fp64, cudaStream_t st);
+int launch_handoff_fx(const void* W32, const void* W32lo, double* U64, double* G64, const Geom& g, int nfields,
+                      cudaStream_t st);
 // compact FP32 working storage (rows 0 and 1 of each matrix) of the FP32
 // sweep phase: from / to the full layout; nmat = 4 for links, 1 for a gauge
 // transform
@@ -279,8 +290,9 @@ int compute_wilson_loops_offaxis(const void* U, int prec, const Geom& g, int nfi
                                  int Tmax, double* W_host, cudaStream_t st);
 
 // ---- smearing (mcg_smear.cu) ------------------------------------------------
+// keep_fp64: FP64 fields in FP64 (an FP32 phase starts from the result)
 int run_smear(const void* Uin, void* Uout, int prec, const Geom& g, int nfields, double rho, double eps, int n,
-              cudaStream_t st);
+              cudaStream_t st, bool keep_fp64 = false);
 
 // FP64 smearing in fixed point (mcg_smear_fx.cu), n >= 1 steps of a validated
 // field: whether rho, eps meet its operand bounds, and the steps.

@@ -278,7 +278,7 @@ __global__ void __launch_bounds__(ST) k_smear_step(const cplx<T>* __restrict__ U
 }
 
 int run_smear(const void* Uin, void* Uout, int prec, const Geom& g, int nfields, double rho, double eps, int n,
-              cudaStream_t st) {
+              cudaStream_t st, bool keep_fp64) {
     const size_t bytes = (prec == MCG_F64 ? 16 : 8) * link_elems(g) * (size_t)nfields;
     if (n <= 0) {
         MCG_CK(cudaMemcpyAsync(Uout, Uin, bytes, cudaMemcpyDeviceToDevice, st));
@@ -286,7 +286,8 @@ int run_smear(const void* Uin, void* Uout, int prec, const Geom& g, int nfields,
     }
     // FP64 fields in fixed point where its operand bounds hold (the paper's
     // parameters: 0.6 and 0.77 of the limit); other rho, eps in FP64
-    if (prec == MCG_F64 && smear_fx_applies(rho, eps)) return run_smear_fx(Uin, Uout, g, nfields, rho, eps, n, st);
+    if (prec == MCG_F64 && !keep_fp64 && smear_fx_applies(rho, eps))
+        return run_smear_fx(Uin, Uout, g, nfields, rho, eps, n, st);
     int rc = 0;
     void* tmp = nullptr;
     if (n >= 2) {
@@ -745,7 +746,7 @@ int run_ascent_step(void* U, void* G, const double* grad, double alpha, int prec
         k_ascent_gauge<float><<<nb, 256, 0, st>>>(grad, alpha, (cplx<float>*)G, (cplx<float>*)W, g, nfields);
     MCG_CK(cudaGetLastError());
     note_launches(1);
-    return launch_apply_gauge(U, W, prec, g, nfields, st);
+    return prec == MCG_F64 ? launch_apply_gauge_fx(U, W, g, nfields, st) : launch_apply_gauge(U, W, prec, g, nfields, st);
 }
 
 // index-check counter of this unit (MCG_CHECK builds)

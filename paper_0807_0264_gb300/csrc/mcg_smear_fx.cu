@@ -38,17 +38,6 @@ struct FxSmear {
     int nterms;          // even
 };
 
-__device__ __forceinline__ cfx fx_load(const int4* p) {
-    const int4 v = *p;
-    cfx r;
-    r.re.h = v.x;
-    r.re.l = v.y;
-    r.im.h = v.z;
-    r.im.l = v.w;
-    return r;
-}
-__device__ __forceinline__ int4 fx_pack(cfx a) { return make_int4(a.re.h, a.re.l, a.im.h, a.im.l); }
-
 // factor f of a staple path of the link (mu, c): its matrix, daggered (a
 // transposed read with the imaginary parts negated) where the path asks for it
 __device__ __forceinline__ void fx_factor(const int4* __restrict__ U, const Geom& g, const int c[4], int mu, int nu,

@@ -205,12 +205,13 @@ __device__ __forceinline__ int subgroup_step(L& lk, const int P, const int Q, co
 // ---------------------------------------------------------------------------
 // Shared memory per thread: 8 links + Omega (81 complex): 41.5 KB for 64 FP32
 // threads (5 blocks per SM), 83 KB for 128 FP32 or 64 FP64 threads (2 per SM).
-// S32: the local problem in FP32 (every site).  Otherwise: only the sites that
-// the fixed-point sweep of an unvalidated field left alone (bt.bad counts them,
-// zero for any SU(3) field), by the same test.
+// S32: the local problem in FP32.  Otherwise the exact local problem in FP64:
+// fields that an FP32 phase starts from later (see mcg_field_fx.cu), and, with
+// bt.bad set, only the sites that the fixed-point sweep of an unvalidated field
+// left alone (bt.bad counts them, zero for any SU(3) field), by the same test.
 template <typename T, bool ACC, int NT, bool S32>
 __global__ void __launch_bounds__(NT, 2) k_halfsweep(SweepBatch bt, int parity) {
-    if (!S32 && *bt.bad == 0) return;
+    if (!S32 && bt.bad && *bt.bad == 0) return;
     const int f = field_of_block(bt.desc, bt.nf, blockIdx.x);
     if (bt.state[f].done) return;  // block-uniform
     const FieldDesc fd = bt.desc[f];
@@ -235,7 +236,7 @@ __global__ void __launch_bounds__(NT, 2) k_halfsweep(SweepBatch bt, int parity) 
     if (active) {
 #pragma unroll
         for (int mu = 0; mu < 4; ++mu) sb[mu] = eo_neighbor(g, c, mu, -1);
-        if constexpr (!S32) {
+        if (!S32 && bt.bad) {
             const double2* Ud = reinterpret_cast<const double2*>(fd.U);
             const size_t vh = (size_t)g.vh;
             bool bad = fx_bad_matrix(reinterpret_cast<const double2*>(fd.G) + gidx(g, parity, 0, s), 3 * vh, vh);
@@ -750,19 +751,22 @@ static size_t halfsweep_smem_f64(int nt) { return sizeof(cplx<double>) * 81 * nt
 
 // Raises the dynamic shared-memory limit of the half-sweep kernels for the
 // current device.  Called on every fix phase (never inside a stream capture):
-// the attribute is per device, and the call costs microseconds.  FP64: the
-// sweeps with the FP32 local solve.
+// the attribute is per device, and the call costs microseconds.
 template <typename T>
 static int prepare_halfsweep(int nt) {
     if constexpr (sizeof(T) == 8) {
         const size_t smem = halfsweep_smem_f64(nt);
         int rc = 0;
         if (nt == 128) {
-            if ((rc = raise_smem(k_halfsweep<T, false, 128, true>, smem)) ||
+            if ((rc = raise_smem(k_halfsweep<T, false, 128, false>, smem)) ||
+                (rc = raise_smem(k_halfsweep<T, true, 128, false>, smem)) ||
+                (rc = raise_smem(k_halfsweep<T, false, 128, true>, smem)) ||
                 (rc = raise_smem(k_halfsweep<T, true, 128, true>, smem)))
                 return rc;
         } else {
-            if ((rc = raise_smem(k_halfsweep<T, false, 64, true>, smem)) ||
+            if ((rc = raise_smem(k_halfsweep<T, false, 64, false>, smem)) ||
+                (rc = raise_smem(k_halfsweep<T, true, 64, false>, smem)) ||
+                (rc = raise_smem(k_halfsweep<T, false, 64, true>, smem)) ||
                 (rc = raise_smem(k_halfsweep<T, true, 64, true>, smem)))
                 return rc;
         }
@@ -780,11 +784,13 @@ static void launch_halfsweep(int nt, bool acc, const SweepBatch& bt, int parity,
         if (bt.tps > 0) {
             launch_halfsweep_fx(FxShape{bt.tps, nt}, acc, bt, parity, nblocks, st);
         } else if (nt == 128) {
-            (acc ? k_halfsweep<T, true, 128, true> : k_halfsweep<T, false, 128, true>)<<<nblocks, 128, smem, st>>>(bt,
-                                                                                                              parity);
+            const auto k = bt.solve32 ? (acc ? k_halfsweep<T, true, 128, true> : k_halfsweep<T, false, 128, true>)
+                                      : (acc ? k_halfsweep<T, true, 128, false> : k_halfsweep<T, false, 128, false>);
+            k<<<nblocks, 128, smem, st>>>(bt, parity);
         } else {
-            (acc ? k_halfsweep<T, true, 64, true> : k_halfsweep<T, false, 64, true>)<<<nblocks, 64, smem, st>>>(bt,
-                                                                                                            parity);
+            const auto k = bt.solve32 ? (acc ? k_halfsweep<T, true, 64, true> : k_halfsweep<T, false, 64, true>)
+                                      : (acc ? k_halfsweep<T, true, 64, false> : k_halfsweep<T, false, 64, false>);
+            k<<<nblocks, 64, smem, st>>>(bt, parity);
         }
     } else {
         launch_halfsweep_c12(nt, acc, bt, parity, nblocks, st);
@@ -842,14 +848,15 @@ constexpr int kMaxChains = 16;
 template <typename T>
 int run_fix_phase(const std::vector<FieldDesc>& fields_in, FieldState* d_state, FieldState* h_state, double* d_hist,
                   int hist_len, double tol, int window, double omega, int reunit_every, int abs_cap,
-                  int check_every, bool fresh, cudaStream_t stream, bool solve32, const PhaseRestart* restart) {
+                  int check_every, bool fresh, cudaStream_t stream, bool solve32, const PhaseRestart* restart,
+                  bool keep_fp64) {
     constexpr bool DF = std::is_same<T, DoubleFloat>::value;
     const int prec = (DF || sizeof(T) == 8) ? MCG_F64 : MCG_F32;
     const int nf = (int)fields_in.size();
     std::vector<FieldDesc> fields = fields_in;
     // the exact FP64 sweep: several threads per site
     FxShape fx = {0, 0};
-    if (!DF && sizeof(T) == 8 && !solve32) {
+    if (!DF && sizeof(T) == 8 && !solve32 && !keep_fp64) {
         long long sites = 0;
         for (const auto& fd : fields) sites += fd.geo.vh;
         fx = fx_shape(sites);
@@ -1393,12 +1400,12 @@ template int time_halfsweep<float>(void*, void*, const Geom&, int, int, int, flo
 template int time_halfsweep<double>(void*, void*, const Geom&, int, int, int, float*, cudaStream_t);
 
 template int run_fix_phase<float>(const std::vector<FieldDesc>&, FieldState*, FieldState*, double*, int, double,
-                                  int, double, int, int, int, bool, cudaStream_t, bool, const PhaseRestart*);
+                                  int, double, int, int, int, bool, cudaStream_t, bool, const PhaseRestart*, bool);
 template int run_fix_phase<DoubleFloat>(const std::vector<FieldDesc>&, FieldState*, FieldState*, double*, int,
                                         double, int, double, int, int, int, bool, cudaStream_t, bool,
-                                        const PhaseRestart*);
+                                        const PhaseRestart*, bool);
 template int run_fix_phase<double>(const std::vector<FieldDesc>&, FieldState*, FieldState*, double*, int, double,
-                                   int, double, int, int, int, bool, cudaStream_t, bool, const PhaseRestart*);
+                                   int, double, int, int, int, bool, cudaStream_t, bool, const PhaseRestart*, bool);
 
 // index-check counter of this unit (MCG_CHECK builds)
 MCG_BOUND_READER(bound_hits_sweep)

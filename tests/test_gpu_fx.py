@@ -88,3 +88,33 @@ def test_unvalidated_sites_keep_the_fp64_kernel():
     assert np.abs(mcg.mcg_unpack_gauge(Gd, dims)[0].cpu().numpy() - Go).max() < 9e-11
     ref = (np.abs(np.trace(Uo, axis1=-2, axis2=-1)) ** 2).sum()
     assert abs(R - ref) < 1e-11 * ref
+
+
+# near-unitary fields take the fixed-point kernels, the others (one field scaled, one with a zero and a scaled
+# link) FP64 per link or plaquette; FP32 fields are exact inputs of both.  Rounding: ~30 operations of 1.1e-16 on
+# entries of the size of a plaquette's factors (a transformed link), averaged over the plaquettes
+@pytest.mark.parametrize("dims", [(2, 2, 2, 2), (6, 2, 10, 4), (10, 6, 14, 12)])
+@pytest.mark.parametrize("scale", [1.0, 1e-3, 7.0, None])
+def test_fixed_point_plaquette_and_transforms(dims, scale):
+    from paper_0807_0264_gb300 import mcg
+
+    U = synth.make_field(dims, 0.7, 8)
+    if scale is None:
+        U[3, 1] *= 40.0
+        U[9, 2] = 0.0
+    else:
+        U *= scale
+    Ud = _pack(mcg, [U, U], dims)
+    ref, top = oracle.plaquette(dims, U), max(1.0, np.abs(U).max()) ** 4 if scale is None else scale**4
+    assert np.abs(np.array(mcg.mcg_plaquette(Ud, dims)) - ref).max() < 1e-14 * top
+    U32 = mcg.mcg_convert(Ud, mcg.F32)
+    ref32 = oracle.plaquette(dims, mcg.mcg_unpack_links(U32, dims)[0].cpu().numpy())
+    assert np.abs(np.array(mcg.mcg_plaquette(U32, dims)) - ref32).max() < 1e-14 * top
+    # an ascent step: W = exp(i alpha grad.lambda / 2) on the links and on Omega
+    G = mcg.identity_gauge(dims, 2)
+    grad = torch.randn(2, np.prod(dims), 8, dtype=torch.float64, device="cuda", generator=torch.Generator("cuda").manual_seed(1))
+    mcg.mcg_ascent_step(Ud, G, grad, dims, 0.1)
+    W = mcg.mcg_unpack_gauge(G, dims).cpu().numpy()
+    got = mcg.mcg_unpack_links(Ud, dims).cpu().numpy()
+    for f in range(2):
+        assert np.abs(got[f] - oracle.apply_gauge(dims, U, W[f])).max() < 1e-14 * max(1.0, np.abs(U).max())
