@@ -56,6 +56,7 @@ unsigned long long bound_hits_field_fx(bool reset);
 unsigned long long bound_hits_observables(bool reset);
 unsigned long long bound_hits_smear(bool reset);
 unsigned long long bound_hits_smear_fx(bool reset);
+unsigned long long bound_hits_smear_bwd_fx(bool reset);
 unsigned long long bound_hits_sweep(bool reset);
 unsigned long long bound_hits_sweep_f32(bool reset);
 unsigned long long bound_hits_sweep_fx(bool reset);
@@ -301,6 +302,10 @@ int run_smear_fx(const void* Uin, void* Uout, const Geom& g, int nfields, double
                  cudaStream_t st);
 
 // ---- differentiation (mcg_smear.cu) -----------------------------------------
+// in fixed point (mcg_smear_bwd_fx.cu), for rho, eps of smear_fx_applies;
+// *bad: device count of matrices it does not take (then Gin is not written)
+int run_smear_backward_fx(const void* U, const double* Gout, double* Gin, const Geom& g, int nfields, double rho,
+                          double eps, unsigned** bad, cudaStream_t st);
 int run_smear_step_backward(const void* U, const double* Gout, double* Gin, const Geom& g, int nfields, double rho,
                             double eps, cudaStream_t st);
 int run_functional_matrix_grad(const void* U, int prec, double* G, const Geom& g, int nfields, cudaStream_t st);

@@ -426,12 +426,17 @@ __device__ __forceinline__ void atomic_add_link(double* __restrict__ G, const Ge
         }
 }
 
-// Reverse-mode derivative of one smearing step U' = exp(iQ(U)) U (FP64).
-// Gin must be zeroed; every contribution is added atomically.
+// Reverse-mode derivative of one smearing step U' = exp(iQ(U)) U in FP64: rho and
+// eps beyond the bounds of the fixed-point step (mcg_smear_bwd_fx.cu), and steps
+// on links that are not near-unitary or with gradients that are not finite (only,
+// when given: null or a device count that is not zero).  Gin must be zeroed; every
+// contribution is added atomically.
 __global__ void __launch_bounds__(ST) k_smear_step_backward(const cplx<double>* __restrict__ Uall,
                                                             const cplx<double>* __restrict__ Gout_all,
                                                             double* __restrict__ Gin_all, Geom g, int nfields,
-                                                            double rho, double cp, double cr) {
+                                                            double rho, double cp, double cr,
+                                                            const unsigned* only) {
+    if (only && *only == 0) return;
     const long long n = 8LL * g.vh * nfields;
     const long long id = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (id >= n) return;
@@ -568,6 +573,11 @@ __global__ void __launch_bounds__(ST) k_smear_step_backward(const cplx<double>* 
     }
 }
 
+__global__ void __launch_bounds__(256) k_zero_if(double* __restrict__ p, long long n, const unsigned* flag) {
+    const long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (*flag && k < n) p[k] = 0.0;
+}
+
 // G = 2 tr(U) 1 per link: the matrix gradient of R = sum |tr U|^2 (FP64 out).
 template <typename T>
 __global__ void __launch_bounds__(256) k_functional_matrix_grad(const cplx<T>* __restrict__ U, double* __restrict__ G,
@@ -699,10 +709,17 @@ __global__ void __launch_bounds__(256) k_ascent_gauge(const double* __restrict__
 int run_smear_step_backward(const void* U, const double* Gout, double* Gin, const Geom& g, int nfields, double rho,
                             double eps, cudaStream_t st) {
     const double cp = (5.0 - 2.0 * eps) / 3.0, cr = -(1.0 - eps) / 12.0;
-    MCG_CK(cudaMemsetAsync(Gin, 0, 16 * link_elems(g) * (size_t)nfields, st));
     const long long n = 8LL * g.vh * nfields;
+    unsigned* only = nullptr;
+    if (smear_fx_applies(rho, eps)) {
+        int rc = run_smear_backward_fx(U, Gout, Gin, g, nfields, rho, eps, &only, st);
+        if (rc) return rc;
+        k_zero_if<<<(unsigned)((18 * n + 255) / 256), 256, 0, st>>>(Gin, 18 * n, only);
+    } else {
+        MCG_CK(cudaMemsetAsync(Gin, 0, 16 * link_elems(g) * (size_t)nfields, st));
+    }
     k_smear_step_backward<<<(int)((n + ST - 1) / ST), ST, 0, st>>>((const cplx<double>*)U, (const cplx<double>*)Gout,
-                                                                    Gin, g, nfields, rho, cp, cr);
+                                                                    Gin, g, nfields, rho, cp, cr, only);
     MCG_CK(cudaGetLastError());
     note_launches(1);
     return 0;

@@ -118,3 +118,35 @@ def test_fixed_point_plaquette_and_transforms(dims, scale):
     got = mcg.mcg_unpack_links(Ud, dims).cpu().numpy()
     for f in range(2):
         assert np.abs(got[f] - oracle.apply_gauge(dims, U, W[f])).max() < 1e-14 * max(1.0, np.abs(U).max())
+
+
+# the reverse step: lattices of extent 2 (a link in its own staples), gradients of any scale, zero but for one
+# link, and with infinities; links that are not near-unitary take the FP64 kernel.  The oracle's bar of the FP64
+# kernel (1e-11 of the gradient), for a gradient of one link relative to what it reaches
+@pytest.mark.parametrize("eps,rho", [(1.0, 0.1), (-0.25, 0.06), (1.0, 0.3)])
+@pytest.mark.parametrize("dims", [(2, 2, 2, 2), (6, 2, 4, 2), (4, 4, 2, 6)])
+def test_fixed_point_smear_backward(dims, eps, rho):
+    from paper_0807_0264_gb300 import mcg
+
+    rng = np.random.default_rng(4)
+    U, V = synth.make_field(dims, 0.7, 9), np.prod(dims)
+    dense = rng.standard_normal((V, 4, 3, 3)) + 1j * rng.standard_normal((V, 4, 3, 3))
+    point = np.zeros_like(dense)
+    point[V // 3, 1] = dense[V // 3, 1]
+
+    def step(U, G):
+        return mcg.mcg_unpack_links(mcg.mcg_smear_backward_step(_pack(mcg, [U], dims), _pack(mcg, [G], dims), dims, rho, eps),
+                                    dims)[0].cpu().numpy()
+
+    for G in (dense, point):  # the step is linear: scales by powers of ten against the scaled reference
+        ref = oracle.smear_step_backward(dims, U, G, rho, eps)
+        for scale in (1.0, 1e-200, 1e150):
+            assert np.abs(step(U, scale * G) / scale - ref).max() < 1e-11 * np.abs(ref).max()
+    assert not step(U, np.zeros_like(dense)).any()
+    Ub = U.copy()
+    Ub[0, 0] *= 1.5
+    ref = oracle.smear_step_backward(dims, Ub, dense, rho, eps)
+    assert np.abs(step(Ub, dense) - ref).max() < 1e-11 * np.abs(ref).max()
+    bad = dense.copy()
+    bad[1, 2, 0, 0] = np.inf
+    assert not np.isfinite(step(U, bad)).all()
