@@ -17,7 +17,8 @@ CSRC = os.path.join(HERE, "csrc")
 OUT_DIR = os.path.join(HERE, "_lib")
 LIB = os.path.join(OUT_DIR, "libmcg.so")
 SOURCES = ["mcg_capi.cu", "mcg_field.cu", "mcg_field_fx.cu", "mcg_observables.cu", "mcg_smear.cu", "mcg_smear_fx.cu",
-           "mcg_smear_bwd_fx.cu", "mcg_sweep.cu", "mcg_sweep_f32.cu", "mcg_sweep_fx.cu", "mcg_sweep_df.cu"]
+           "mcg_smear_bwd_fx.cu", "mcg_sweep.cu", "mcg_sweep_f32.cu", "mcg_sweep_fx.cu", "mcg_sweep_df.cu",
+           "mcg_wilson_fx.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

@@ -511,8 +511,9 @@ __global__ void k_check_su3(const cplx<T>* __restrict__ M, int nslots, size_t vh
     }
 }
 
-int validate_su3(const void* M, int prec, const Geom& g, int nslots, int nfields, const char* what,
-                 cudaStream_t st, bool finite_only) {
+// the check of nfields fields; h_out: pinned {failing matrices, the first one}
+static int check_su3(const void* M, int prec, const Geom& g, int nslots, int nfields, bool finite_only,
+                     unsigned long long** h_out, cudaStream_t st) {
     int rc = 0;
     unsigned long long* d_bad = (unsigned long long*)scratch_device("check.bad", 2 * sizeof(unsigned long long), &rc);
     if (rc) return rc;
@@ -532,6 +533,24 @@ int validate_su3(const void* M, int prec, const Geom& g, int nslots, int nfields
     note_launches(1);
     MCG_CK(cudaMemcpyAsync(h_bad, d_bad, 2 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, st));
     MCG_CK(cudaStreamSynchronize(st));
+    *h_out = h_bad;
+    return 0;
+}
+
+int count_not_su3(const void* M, int prec, const Geom& g, int nslots, int nfields, unsigned long long* count,
+                  cudaStream_t st) {
+    unsigned long long* h_bad = nullptr;
+    int rc = check_su3(M, prec, g, nslots, nfields, false, &h_bad, st);
+    if (!rc) *count = h_bad[0];
+    return rc;
+}
+
+int validate_su3(const void* M, int prec, const Geom& g, int nslots, int nfields, const char* what,
+                 cudaStream_t st, bool finite_only) {
+    unsigned long long* h_bad = nullptr;
+    int rc = check_su3(M, prec, g, nslots, nfields, finite_only, &h_bad, st);
+    if (rc) return rc;
+    const size_t vh = (size_t)g.vh;
     if (h_bad[0] == 0) return 0;
     const size_t i = (size_t)h_bad[1], per_field = (size_t)nslots * vh;
     const size_t f = i / per_field, slot = (i % per_field) / vh, s = i % vh;

@@ -290,6 +290,29 @@ int compute_wilson_loops(const void* U, int prec, const Geom& g, int nfields, in
 int compute_wilson_loops_offaxis(const void* U, int prec, const Geom& g, int nfields, const int* vecs, int nvec,
                                  int Tmax, double* W_host, cudaStream_t st);
 
+// FP64 SU(3) fields in fixed point (mcg_wilson_fx.cu).  A step of up to three
+// paths at once: the link (axis, x + from), daggered if back; first: the paths
+// begin here.  For the loops `from` is the path's displacement.  P: npath line
+// fields back to back, St: the temporal lines of length 1 .. Tmax; partial:
+// npath * Tmax * wilson_fx_blocks(g) doubles; out: Tmax sums over sites and
+// paths, times scale.
+struct PathStep {
+    int from[4];
+    int axis, back;
+};
+struct PathSteps {
+    PathStep step[3];
+    int first;
+};
+int wilson_fx_blocks(const Geom& g);
+void launch_path_step_fx(const double* U, const void* Pin, void* Pout, const Geom& g, const PathSteps& ps, int npath,
+                         cudaStream_t st);
+void launch_wilson_fx(const void* P, const void* St, const Geom& g, const PathSteps& ps, int npath, int Tmax,
+                      double* partial, double scale, double* out, cudaStream_t st);
+// number of matrices that fail the SU(3) test of validate_su3 (no message)
+int count_not_su3(const void* M, int prec, const Geom& g, int nslots, int nfields, unsigned long long* count,
+                  cudaStream_t st);
+
 // ---- smearing (mcg_smear.cu) ------------------------------------------------
 // keep_fp64: FP64 fields in FP64 (an FP32 phase starts from the result)
 int run_smear(const void* Uin, void* Uout, int prec, const Geom& g, int nfields, double rho, double eps, int n,

@@ -213,6 +213,61 @@ int wilson_impl(const cplx<T>* U, const Geom& g, int nfields, int Rmax, int Tmax
     return 0;
 }
 
+// On-axis loops of FP64 SU(3) fields in fixed point: the three axes and all T of
+// a separation per launch.
+int wilson_fx(const double* U, const Geom& g, int nfields, int Rmax, int Tmax, double* W_host, cudaStream_t st) {
+    const size_t line = (size_t)9 * 2 * g.vh;
+    int rc = 0;
+    int4* Lt = (int4*)scratch_device("wl.t", 16 * line * Tmax, &rc);
+    if (rc) return rc;
+    int4* Ls = (int4*)scratch_device("wl.s", 16 * line * 6, &rc);  // 3 axes x 2 buffers
+    if (rc) return rc;
+    double* partial = (double*)scratch_device("wl.partial", sizeof(double) * 3 * Tmax * wilson_fx_blocks(g), &rc);
+    if (rc) return rc;
+    double* d_W = (double*)scratch_device("wl.W", sizeof(double) * (size_t)nfields * Rmax * Tmax, &rc);
+    if (rc) return rc;
+    for (int f = 0; f < nfields; ++f) {
+        const double* Uf = U + 2 * (size_t)f * link_elems(g);
+        for (int T_ = 1; T_ <= Tmax; ++T_) {
+            PathSteps ps = {};
+            ps.first = T_ == 1;
+            ps.step[0].axis = 3;
+            ps.step[0].from[3] = T_ - 1;
+            launch_path_step_fx(Uf, Lt + line * (T_ < 2 ? 0 : T_ - 2), Lt + line * (T_ - 1), g, ps, 1, st);
+        }
+        for (int R = 1; R <= Rmax; ++R) {
+            int4* cur = Ls + line * 3 * (R & 1);
+            const int4* prev = Ls + line * 3 * ((R + 1) & 1);
+            PathSteps ps = {}, disp = {};
+            ps.first = R == 1;
+            for (int i = 0; i < 3; ++i) {
+                ps.step[i].axis = i;
+                ps.step[i].from[i] = R - 1;
+                disp.step[i].from[i] = R;
+            }
+            launch_path_step_fx(Uf, prev, cur, g, ps, 3, st);
+            launch_wilson_fx(cur, Lt, g, disp, 3, Tmax, partial, 1.0 / (3.0 * 2 * g.vh),
+                             d_W + ((size_t)f * Rmax + (R - 1)) * Tmax, st);
+        }
+    }
+    MCG_CK(cudaGetLastError());
+    note_launches((long long)nfields * (Tmax + 3 * Rmax));
+    MCG_CK(cudaMemcpyAsync(W_host, d_W, sizeof(double) * (size_t)nfields * Rmax * Tmax, cudaMemcpyDeviceToHost, st));
+    MCG_CK(cudaStreamSynchronize(st));
+    return 0;
+}
+
+// Whether the field can take the fixed-point loops: every link in SU(3) to the
+// 1e-6 of the input check, so that lines of any length stay near-unitary.
+int wilson_fx_applies(const void* U, int prec, const Geom& g, int nfields, bool* yes, cudaStream_t st) {
+    *yes = false;
+    if (prec != MCG_F64) return 0;
+    unsigned long long bad = 0;
+    int rc = count_not_su3(U, prec, g, 8, nfields, &bad, st);
+    if (!rc) *yes = bad == 0;
+    return rc;
+}
+
 // ---- off-axis spatial sides -------------------------------------------------
 // lexicographic index of x + (d0, d1, d2, d3), periodic, any signs
 __device__ __forceinline__ int lex_offset(const Geom& g, int x, int d0, int d1, int d2, int d3) {
@@ -328,7 +383,7 @@ void path_steps(const std::array<int, 3>& r, std::vector<int>& axis, std::vector
 
 template <typename T>
 int wilson_offaxis_impl(const cplx<T>* U, const Geom& g, int nfields, const int* vecs, int nvec, int Tmax,
-                        double* W_host, cudaStream_t st) {
+                        double* W_host, bool fx, cudaStream_t st) {
     const int V = 2 * g.vh;
     const size_t line = (size_t)9 * V;
     int rc = 0;
@@ -337,7 +392,8 @@ int wilson_offaxis_impl(const cplx<T>* U, const Geom& g, int nfields, const int*
     cplx<T>* Pb = (cplx<T>*)scratch_device("wl.s", sizeof(cplx<T>) * line * 6, &rc);  // two path buffers
     if (rc) return rc;
     const int nb = nblocks(V, OT);
-    double* partial = (double*)scratch_device("wl.partial", sizeof(double) * nb, &rc);
+    double* partial =
+        (double*)scratch_device("wl.partial", sizeof(double) * std::max(nb, fx ? Tmax * wilson_fx_blocks(g) : 0), &rc);
     if (rc) return rc;
     std::vector<std::vector<std::array<int, 3>>> imgs(nvec);
     size_t nimg_tot = 0;
@@ -353,8 +409,16 @@ int wilson_offaxis_impl(const cplx<T>* U, const Geom& g, int nfields, const int*
     for (int f = 0; f < nfields; ++f) {
         const cplx<T>* Uf = U + (size_t)f * link_elems(g);
         for (int T_ = 1; T_ <= Tmax; ++T_) {
-            k_line_extend<T><<<nb, OT, 0, st>>>(Uf, Lt + line * (T_ - 2 < 0 ? 0 : T_ - 2), Lt + line * (T_ - 1), g, 3,
-                                                T_);
+            const cplx<T>* in = Lt + line * (T_ - 2 < 0 ? 0 : T_ - 2);
+            if (fx) {
+                PathSteps ps = {};
+                ps.first = T_ == 1;
+                ps.step[0].axis = 3;
+                ps.step[0].from[3] = T_ - 1;
+                launch_path_step_fx((const double*)Uf, in, Lt + line * (T_ - 1), g, ps, 1, st);
+            } else {
+                k_line_extend<T><<<nb, OT, 0, st>>>(Uf, in, Lt + line * (T_ - 1), g, 3, T_);
+            }
             ++launches;
         }
         size_t q = 0;
@@ -364,13 +428,28 @@ int wilson_offaxis_impl(const cplx<T>* U, const Geom& g, int nfields, const int*
                 int o[3] = {0, 0, 0};
                 int cur = 0;
                 for (size_t k = 0; k < axis.size(); ++k) {
-                    k_path_step<T><<<nb, OT, 0, st>>>(Uf, Pb + line * cur, Pb + line * (1 - cur), g, o[0], o[1], o[2],
-                                                      axis[k], sign[k], k == 0 ? 1 : 0);
+                    if (fx) {
+                        PathSteps ps = {};
+                        ps.first = k == 0;
+                        ps.step[0].axis = axis[k];
+                        ps.step[0].back = sign[k] < 0;
+                        for (int j = 0; j < 3; ++j) ps.step[0].from[j] = o[j] - (sign[k] < 0 && j == axis[k] ? 1 : 0);
+                        launch_path_step_fx((const double*)Uf, Pb + line * cur, Pb + line * (1 - cur), g, ps, 1, st);
+                    } else {
+                        k_path_step<T><<<nb, OT, 0, st>>>(Uf, Pb + line * cur, Pb + line * (1 - cur), g, o[0], o[1],
+                                                          o[2], axis[k], sign[k], k == 0 ? 1 : 0);
+                    }
                     ++launches;
                     o[axis[k]] += sign[k];
                     cur = 1 - cur;
                 }
-                for (int T_ = 1; T_ <= Tmax; ++T_) {
+                if (fx) {
+                    PathSteps disp = {};
+                    for (int j = 0; j < 3; ++j) disp.step[0].from[j] = r[j];
+                    launch_wilson_fx(Pb + line * cur, Lt, g, disp, 1, Tmax, partial, 1.0 / V, d_W + q * Tmax, st);
+                    launches += 2;
+                }
+                for (int T_ = 1; T_ <= Tmax && !fx; ++T_) {
                     k_wilson_path<T><<<nb, OT, 0, st>>>(Pb + line * cur, Lt + line * (T_ - 1), g, r[0], r[1], r[2], T_,
                                                         partial);
                     k_sum_fixed<<<1, 256, 0, st>>>(partial, nb, 1.0 / V, d_W + q * Tmax + (T_ - 1));
@@ -415,15 +494,22 @@ int launch_vortex_remove(const void* U, const int8_t* Z, void* Ur, void* Zl, int
 
 int compute_wilson_loops(const void* U, int prec, const Geom& g, int nfields, int Rmax, int Tmax, double* W_host,
                          cudaStream_t st) {
+    bool fx = false;
+    int rc = wilson_fx_applies(U, prec, g, nfields, &fx, st);
+    if (rc) return rc;
+    if (fx) return wilson_fx((const double*)U, g, nfields, Rmax, Tmax, W_host, st);
     if (prec == MCG_F64) return wilson_impl<double>((const cplx<double>*)U, g, nfields, Rmax, Tmax, W_host, st);
     return wilson_impl<float>((const cplx<float>*)U, g, nfields, Rmax, Tmax, W_host, st);
 }
 
 int compute_wilson_loops_offaxis(const void* U, int prec, const Geom& g, int nfields, const int* vecs, int nvec,
                                  int Tmax, double* W_host, cudaStream_t st) {
+    bool fx = false;
+    int rc = wilson_fx_applies(U, prec, g, nfields, &fx, st);
+    if (rc) return rc;
     if (prec == MCG_F64)
-        return wilson_offaxis_impl<double>((const cplx<double>*)U, g, nfields, vecs, nvec, Tmax, W_host, st);
-    return wilson_offaxis_impl<float>((const cplx<float>*)U, g, nfields, vecs, nvec, Tmax, W_host, st);
+        return wilson_offaxis_impl<double>((const cplx<double>*)U, g, nfields, vecs, nvec, Tmax, W_host, fx, st);
+    return wilson_offaxis_impl<float>((const cplx<float>*)U, g, nfields, vecs, nvec, Tmax, W_host, false, st);
 }
 
 // index-check counter of this unit (MCG_CHECK builds)

@@ -150,3 +150,21 @@ def test_fixed_point_smear_backward(dims, eps, rho):
     bad = dense.copy()
     bad[1, 2, 0, 0] = np.inf
     assert not np.isfinite(step(U, bad)).all()
+
+
+# loops of SU(3) fields (fixed point) and of others (FP64): long lines, every T of a separation in one launch, odd
+# remainders of the 128-site blocks; ~L roundings of 1.1e-16 on a line of L links, bar 1e-15 L
+@pytest.mark.parametrize("dims", [(2, 2, 2, 2), (6, 4, 10, 6), (4, 4, 4, 14)])
+@pytest.mark.parametrize("scale", [1.0, 1.001])
+def test_fixed_point_wilson_loops(dims, scale):
+    from paper_0807_0264_gb300 import mcg
+
+    R, T = min(dims[:3]), dims[3]
+    U = [scale * synth.make_field(dims, 0.3, s, gauge=s == 1) for s in (1, 2)]
+    W = mcg.mcg_wilson_loops(_pack(mcg, U, dims), dims, R, T)
+    vec = [(1, 0, 0), (1, 1, 0)] if R == 2 else [(1, 2, 1), (0, 1, 3), (2, 2, 0)]
+    Wo = mcg.mcg_wilson_loops_offaxis(_pack(mcg, U, dims), dims, vec, T)
+    for f in range(2):
+        top = scale ** (2 * (R + T + 3))
+        assert np.abs(W[f] - oracle.wilson_loops(dims, U[f], R, T)).max() < 1e-15 * (2 * (R + T)) * top
+        assert np.abs(Wo[f] - oracle.wilson_loops_offaxis(dims, U[f], vec, T)).max() < 1e-15 * (2 * (4 + T)) * top
