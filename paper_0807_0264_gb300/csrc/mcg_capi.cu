@@ -259,8 +259,14 @@ struct FieldSpec {
     void* U;
     void* G;
     Geom g;
-    bool keep_fp64 = false;  // a later FP32 phase starts from the result: FP64 arithmetic (mcg_field_fx.cu)
+    bool keep_fp64 = false;  // later sweeps round the result to FP32: FP64 arithmetic (mcg_field_fx.cu)
 };
+
+// Whether a fix rounds its field to FP32: FP32 sweeps or fields, and the local
+// problems of the double-float and FP32-solve sweeps.
+static bool rounds_to_fp32(const mcg_params* p, int prec) {
+    return prec == MCG_F32 || p->fp32_sweeps > 0 || p->fp64_df || p->fp64_solve32;
+}
 
 // MCG relaxation of a batch of fields (all of one precision, any sizes), one
 // launch per half-sweep for the whole batch.
@@ -366,7 +372,7 @@ static int fix_fields(const std::vector<FieldSpec>& fs, int prec, const mcg_para
         // hand-off: FP64 re-unitarised transform applied to the FP64 links
         for (int f = 0; f < nf; ++f)
             if ((rc = launch_handoff(fds[f].G, nullptr, (double*)fs[f].U, (double*)fs[f].G, fs[f].g, 1,
-                                     fs[f].keep_fp64, st)))
+                                     fs[f].keep_fp64 || prm->fp64_df || prm->fp64_solve32, st)))
                 return rc;
         fresh = false;
     }
@@ -758,9 +764,8 @@ int mcg_precondition_fix(void* U, void* G, int8_t* Z, const mcg_lattice* lat, co
     int status = MCG_OK;
     const double norm = 1.0 / (9.0 * 8.0 * g.vh);
     if ((rc = launch_identity_gauge(G, prec, g, nf, stream))) return rc;
-    // the second fix starts with an FP32 phase (or is FP32): what leads to it
-    // stays in FP64 arithmetic
-    const bool keep = prec == MCG_F32 || params->fp32_sweeps > 0;
+    // what leads to a second fix that rounds to FP32 stays in FP64 arithmetic
+    const bool keep = rounds_to_fp32(params, prec);
     if (nsmear > 0) {
         // S = smear(U) in the smear precision; the smeared field is then fixed
         // in the field's precision with the caller's schedule (transform W)
@@ -957,7 +962,7 @@ int mcg_precondition_levels(const void* U, void* U_out, void* G_out, int8_t* Z_o
     for (int l = 0; l < nlevels; ++l)
         MCG_CK(cudaMemcpyAsync((char*)U_out + eb * le * l, U, eb * le, cudaMemcpyDeviceToDevice, stream));
     if ((rc = launch_identity_gauge(G_out, prec, g, nlevels, stream))) return rc;
-    const bool keep = prec == MCG_F32 || params->fp32_sweeps > 0;  // as in mcg_precondition_fix
+    const bool keep = rounds_to_fp32(params, prec);  // as in mcg_precondition_fix
     void* Sp = nullptr;  // the smeared fields, then their transforms
     void* W = nullptr;
     if (ns > 0) {
@@ -1108,7 +1113,7 @@ int mcg_gribov_search(const mcg_field* copies, int ncopies, const int* config_of
             return rc;
     // each copy starts as U^Omega0 with its own random Omega0; the fix then
     // accumulates onto Omega0, so G ends as the total transform of the copy
-    const bool keep = precision == MCG_F32 || params->fp32_sweeps > 0;  // the copies start an FP32 phase
+    const bool keep = rounds_to_fp32(params, precision);
     for (int f = 0; f < ncopies; ++f)
         if ((rc = keep ? launch_apply_gauge(fs[f].U, fs[f].G, precision, fs[f].g, 1, stream)
                        : launch_apply_gauge_fx(fs[f].U, fs[f].G, fs[f].g, 1, stream)))

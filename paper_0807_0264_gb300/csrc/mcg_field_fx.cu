@@ -3,11 +3,11 @@
 // points are not always validated: a thread that meets a matrix that is not
 // near-unitary does its link or plaquette in FP64.
 //
-// A transformed field that an FP32 phase starts from keeps the FP64 kernels of
-// mcg_field.cu: the over-relaxed FP32 sweeps of an unfixed field follow the last
-// bit of their input (one entry rounded the other way moved the links of a
-// 20^3 x 40 field by 1.4e-7 after 150 sweeps), so those results stay what they
-// were.
+// A transformed field that later sweeps round to FP32 keeps the FP64 kernels of
+// mcg_field.cu: one entry rounded the other way moved the links of an unfixed
+// 20^3 x 40 field by 1.4e-7 after 150 over-relaxed FP32 sweeps, and a link by
+// 3e-8 in the double-float sweeps, whose local problems are built from the FP32
+// parts; so those results stay what they were.
 #include <cuda_runtime.h>
 
 #include "mcg_common.cuh"

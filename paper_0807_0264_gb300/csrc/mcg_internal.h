@@ -269,8 +269,8 @@ int compute_center(const void* U, int prec, int8_t* Z, const Geom& g, int nfield
                    cudaStream_t st);
 // FP32 transform W of this call (compact form) -> FP64: W64 = reunit(W);
 // U64 <- W64 U64 W64(x+mu)^dag; G64 <- reunit(W64 G64).  W32lo (may be null):
-// lo parts of a double-float W (W = hi + lo).  keep_fp64: in FP64 (a later FP32
-// phase starts from the result), else in fixed point.
+// lo parts of a double-float W (W = hi + lo).  keep_fp64: in FP64 (later sweeps
+// round the result to FP32), else in fixed point.
 int launch_handoff(const void* W32, const void* W32lo, double* U64, double* G64, const Geom& g, int nfields,
                    bool keep_fp64, cudaStream_t st);
 int launch_handoff_fx(const void* W32, const void* W32lo, double* U64, double* G64, const Geom& g, int nfields,
@@ -314,7 +314,7 @@ int count_not_su3(const void* M, int prec, const Geom& g, int nslots, int nfield
                   cudaStream_t st);
 
 // ---- smearing (mcg_smear.cu) ------------------------------------------------
-// keep_fp64: FP64 fields in FP64 (an FP32 phase starts from the result)
+// keep_fp64: FP64 fields in FP64 (later sweeps round the result to FP32)
 int run_smear(const void* Uin, void* Uout, int prec, const Geom& g, int nfields, double rho, double eps, int n,
               cudaStream_t st, bool keep_fp64 = false);
 

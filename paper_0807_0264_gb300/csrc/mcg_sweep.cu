@@ -206,7 +206,7 @@ __device__ __forceinline__ int subgroup_step(L& lk, const int P, const int Q, co
 // Shared memory per thread: 8 links + Omega (81 complex): 41.5 KB for 64 FP32
 // threads (5 blocks per SM), 83 KB for 128 FP32 or 64 FP64 threads (2 per SM).
 // S32: the local problem in FP32.  Otherwise the exact local problem in FP64:
-// fields that an FP32 phase starts from later (see mcg_field_fx.cu), and, with
+// fields that later sweeps round to FP32 (see mcg_field_fx.cu), and, with
 // bt.bad set, only the sites that the fixed-point sweep of an unvalidated field
 // left alone (bt.bad counts them, zero for any SU(3) field), by the same test.
 template <typename T, bool ACC, int NT, bool S32>
