@@ -33,6 +33,26 @@ __device__ __forceinline__ cplx<float> unphase(cplx<float> u, double c, double s
     return mk(__fadd_rn(__fmul_rn(cf, u.x), __fmul_rn(sf, u.y)), __fsub_rn(__fmul_rn(cf, u.y), __fmul_rn(sf, u.x)));
 }
 
+// The same values with fewer FP64 operations (20^3 x 40: 152 -> 95 us against 81 us
+// for the bytes at the copy rate): for Z = 1 a finite entry is unchanged (adding zero
+// keeps the sign of a zero as 1 u + 0 v has it); otherwise the products with
+// -1/2 are exact halvings, by the exponent where that stays normal.
+__device__ __forceinline__ double minus_half(double v) {
+    const unsigned e = ((unsigned)__double2hiint(v) >> 20) & 0x7ff;
+    if (e > 1 && e < 0x7ff) return __hiloint2double((__double2hiint(v) - 0x00100000) ^ 0x80000000, __double2loint(v));
+    return __dmul_rn(-0.5, v);
+}
+__device__ __forceinline__ cplx<double> unphase_fast(cplx<double> u, int m, double c, double s) {
+    const bool finite = (__double2hiint(u.x) & 0x7ff00000) != 0x7ff00000 && (__double2hiint(u.y) & 0x7ff00000) != 0x7ff00000;
+    if (m == 0) {
+        const bool zero = ((__double2hiint(u.x) << 1) | __double2loint(u.x)) == 0 ||
+                          ((__double2hiint(u.y) << 1) | __double2loint(u.y)) == 0;
+        return finite && !zero ? u : unphase(u, c, s);
+    }
+    return mk(__dadd_rn(minus_half(u.x), __dmul_rn(s, u.y)), __dsub_rn(minus_half(u.y), __dmul_rn(s, u.x)));
+}
+__device__ __forceinline__ cplx<float> unphase_fast(cplx<float> u, int, double c, double s) { return unphase(u, c, s); }
+
 // One thread per (field, parity, site): its 4 links.  Ur (may be null, may
 // be U itself): Z^dag U; Zl (may be null): the center links Z * identity.
 template <typename T>
@@ -55,7 +75,7 @@ __global__ void __launch_bounds__(OT) k_vortex_remove(const cplx<T>* U, const in
 #pragma unroll
             for (int e = 0; e < 9; ++e) {
                 const size_t k = lo + lidx(g, mu, p, e, s);
-                Ur[k] = unphase(U[k], c, sn);
+                Ur[k] = unphase_fast(U[k], m, c, sn);
             }
         }
         if (Zl) {

@@ -168,3 +168,48 @@ def test_fixed_point_wilson_loops(dims, scale):
         top = scale ** (2 * (R + T + 3))
         assert np.abs(W[f] - oracle.wilson_loops(dims, U[f], R, T)).max() < 1e-15 * (2 * (R + T)) * top
         assert np.abs(Wo[f] - oracle.wilson_loops_offaxis(dims, U[f], vec, T)).max() < 1e-15 * (2 * (4 + T)) * top
+
+
+def test_observables_at_their_edges():
+    """The FP32 filter of the center projection and the exact halvings of the vortex removal against the oracle, bit
+    for bit: traces on and next to
+    the sector boundaries, zeros of both signs, subnormal and huge entries, infinities."""
+    from paper_0807_0264_gb300 import mcg
+
+    dims, rng = (4, 4, 2, 6), np.random.default_rng(6)
+    V = int(np.prod(dims))
+    U = (rng.standard_normal((V, 4, 3, 3)) + 1j * rng.standard_normal((V, 4, 3, 3))) * 10.0 ** rng.integers(-9, 3, (V, 4, 1, 1))
+    t = np.array([1.0, np.sqrt(3.0), np.nextafter(np.sqrt(3.0), 2), np.nextafter(np.sqrt(3.0), 1), 0.0, 1e-5, 9e-6, 1e-300])
+    for k in range(V):  # traces x + i y near the rays |y| = sqrt(3) x and y = 0, split unevenly over the diagonal
+        x, y = rng.choice(t) * rng.choice([1, -1]), rng.choice(t) * rng.choice([1, -1])
+        U[k, 1] = 0.0
+        U[k, 1, 0, 0], U[k, 1, 1, 1], U[k, 1, 2, 2] = (x + 1j * y) - 0.25, 0.5, -0.25
+    U[0, 2, 0, 1], U[1, 2, 0, 1], U[2, 2, 0, 1] = 5e-324, 1e308 + 1j * 1e308, -0.0
+    U[3, 2, 1, 1] = 2.3e-308 - 1j * 4.4e-308
+    Ud = _pack(mcg, [U], dims)
+    Z, _ = mcg.mcg_center_project(Ud, dims)
+    m = mcg.mcg_unpack_center(Z, dims)[0].cpu().numpy()
+    assert np.array_equal(m, oracle.center_project(dims, U))
+    Ur, _ = mcg.mcg_vortex_remove(Ud, Z, dims)
+    assert np.array_equal(mcg.mcg_unpack_links(Ur, dims)[0].cpu().numpy(), oracle.vortex_remove(dims, U, m))
+    W = np.where(np.abs(U) > 1e100, 0, U)
+    for scale in (1.0, 1e-3, 0.02):  # ~10 roundings of 1.1e-16
+        R = mcg.mcg_functional(_pack(mcg, [scale * W], dims), dims)[0]
+        ref = (np.abs(np.trace(scale * W, axis1=-2, axis2=-1)) ** 2).sum()
+        assert abs(R - ref) < 2e-15 * ref
+    S = synth.make_field(dims, 0.4, 2)
+    assert abs(mcg.mcg_functional(_pack(mcg, [S], dims), dims)[0] - oracle.functional_R(dims, S)) < 2e-15 * oracle.functional_R(dims, S)
+    for entry in (np.inf, -np.inf, np.nan):  # refused as before, wherever it stands
+        B = S.copy()
+        B[V - 1, 3, 2, 2] = entry
+        for call in (lambda: mcg.mcg_center_project(_pack(mcg, [B], dims), dims), lambda: mcg.mcg_smear(_pack(mcg, [B], dims), dims, 0.1, 1.0, 1)):
+            with pytest.raises(mcg.MCGError):
+                call()
+    for off, ok in ((5e-7, True), (2e-6, False)):  # the SU(3) tolerance of 1e-6
+        B = S.copy()
+        B[1, 1] *= 1 + off / 3
+        if ok:
+            mcg.mcg_smear(_pack(mcg, [B], dims), dims, 0.1, 1.0, 1)
+        else:
+            with pytest.raises(mcg.MCGError):
+                mcg.mcg_smear(_pack(mcg, [B], dims), dims, 0.1, 1.0, 1)
