@@ -178,6 +178,7 @@ int branch_streams(int n, cudaStream_t* streams, cudaEvent_t* events, cudaEvent_
 
 void release_all() {
     static_release();
+    graphs_release();
     std::lock_guard<std::mutex> lk(g_mu);
     int dev = 0;
     cudaGetDevice(&dev);

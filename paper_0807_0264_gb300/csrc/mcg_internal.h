@@ -32,6 +32,8 @@ int check_lattice(const mcg_lattice* lat, Geom* g);
 // Drops the cached device addresses of the allocation-free entry point's
 // static array (mcg_release calls it).
 void static_release();
+// Destroys the kept sweep graphs (mcg_release calls it).
+void graphs_release();
 
 // ---- launch accounting ------------------------------------------------------
 // Every kernel the library enqueues is counted (graph launches count their

@@ -213,3 +213,34 @@ def test_observables_at_their_edges():
         else:
             with pytest.raises(mcg.MCGError):
                 mcg.mcg_smear(_pack(mcg, [B], dims), dims, 0.1, 1.0, 1)
+
+
+# kept sweep graphs: calls alternating between shapes, schedules, precisions and batch sizes (more of them than are
+# kept), with other fields and other streams, before and after mcg_release, return the bits of their first call
+def test_repeated_fixes_with_kept_graphs():
+    from paper_0807_0264_gb300 import mcg
+
+    P = mcg.Params
+    kinds = [(4, P(tol=1e-9, max_sweeps=90, check_every=5)), (4, P(tol=1e-9, max_sweeps=90, check_every=7)),
+             (4, P(tol=1e-4, max_sweeps=90, check_every=5)), (4, P(tol=1e-9, max_sweeps=90, reunit_every=3)),
+             (6, P(tol=1e-9, max_sweeps=40)), (4, P(tol=1e-9, max_sweeps=90, fp32_sweeps=60)),
+             (4, P(tol=1e-9, max_sweeps=90, fp32_sweeps=60, fp64_df=1)), (4, P(tol=1e-9, max_sweeps=90, fp64_solve32=1))]
+    data = {(n, s): (synth.make_field((n, 4, 4, 6), 2.0, s)) for n in (4, 6) for s in range(3)}
+
+    def run(kind, seeds, stream):
+        n, prm = kinds[kind]
+        dims = (n, 4, 4, 6)
+        with torch.cuda.stream(stream):
+            Us = [_pack(mcg, [data[n, s]], dims) for s in seeds]
+            Gs = [mcg.identity_gauge(dims) for _ in seeds]
+            r = mcg.mcg_fix_batch(Us, Gs, [dims] * len(Us), prm)
+            return r["R"], r["sweeps"], [u.cpu().numpy().tobytes() for u in Us + Gs]
+
+    main, side = torch.cuda.current_stream(), torch.cuda.Stream()
+    calls = [(k, seeds) for k in range(len(kinds)) for seeds in ((0,), (1, 2), (1,))]
+    first = {c: run(*c, main) for c in calls}
+    for c in calls[::-1]:
+        assert run(*c, side) == first[c]
+    mcg.mcg_release()
+    for c in calls[::2]:
+        assert run(*c, main) == first[c]
