@@ -269,6 +269,17 @@ static bool rounds_to_fp32(const mcg_params* p, int prec) {
     return prec == MCG_F32 || p->fp32_sweeps > 0 || p->fp64_df || p->fp64_solve32;
 }
 
+// links and transform of each field in turn, checked by one launch
+static int validate_fields(const std::vector<FieldSpec>& fs, int prec, const char* what_U, const char* what_G,
+                           cudaStream_t st) {
+    std::vector<CheckItem> items;
+    for (const auto& f : fs) {
+        items.push_back({f.U, f.g, 8, 1, what_U});
+        items.push_back({f.G, f.g, 2, 1, what_G});
+    }
+    return validate_su3(items.data(), (int)items.size(), prec, st);
+}
+
 // MCG relaxation of a batch of fields (all of one precision, any sizes), one
 // launch per half-sweep for the whole batch.
 static int fix_fields(const std::vector<FieldSpec>& fs, int prec, const mcg_params* prm, double* R_out,
@@ -634,8 +645,8 @@ int mcg_fix(void* U, void* G, const mcg_lattice* lat, const mcg_params* params, 
     const size_t eb = elem_bytes(lat->precision);
     if (overlap(U, eb * link_elems(g) * lat->nfields, G, eb * gauge_elems(g) * lat->nfields))
         return fail(MCG_BAD_ARG, "U and G overlap");
-    if ((rc = validate_su3(U, lat->precision, g, 8, lat->nfields, "mcg_fix: U", stream))) return rc;
-    if ((rc = validate_su3(G, lat->precision, g, 2, lat->nfields, "mcg_fix: G", stream))) return rc;
+    const CheckItem items[2] = {{U, g, 8, lat->nfields, "mcg_fix: U"}, {G, g, 2, lat->nfields, "mcg_fix: G"}};
+    if ((rc = validate_su3(items, 2, lat->precision, stream))) return rc;
     return fix_impl(U, G, lat, g, params, R_out, sweeps_out, nullptr, R_hist, stream);
 }
 
@@ -1088,10 +1099,7 @@ int mcg_fix_batch(const mcg_field* fields, int nfields, int precision, const mcg
     std::vector<FieldSpec> fs(nfields);
     for (int f = 0; f < nfields; ++f)
         if ((rc = field_spec(fields[f], precision, &fs[f]))) return rc;
-    for (int f = 0; f < nfields; ++f)
-        if ((rc = validate_su3(fs[f].U, precision, fs[f].g, 8, 1, "mcg_fix_batch: U", stream)) ||
-            (rc = validate_su3(fs[f].G, precision, fs[f].g, 2, 1, "mcg_fix_batch: G", stream)))
-            return rc;
+    if ((rc = validate_fields(fs, precision, "mcg_fix_batch: U", "mcg_fix_batch: G", stream))) return rc;
     return fix_fields(fs, precision, params, R_out, sweeps_out, nullptr, nullptr, stream);
 }
 
@@ -1108,10 +1116,7 @@ int mcg_gribov_search(const mcg_field* copies, int ncopies, const int* config_of
         if ((rc = field_spec(copies[f], precision, &fs[f]))) return rc;
         if (config_of_copy[f] < 0 || config_of_copy[f] >= nconfigs) return fail(MCG_BAD_ARG, "config index out of range");
     }
-    for (int f = 0; f < ncopies; ++f)
-        if ((rc = validate_su3(fs[f].U, precision, fs[f].g, 8, 1, "mcg_gribov_search: U", stream)) ||
-            (rc = validate_su3(fs[f].G, precision, fs[f].g, 2, 1, "mcg_gribov_search: G", stream)))
-            return rc;
+    if ((rc = validate_fields(fs, precision, "mcg_gribov_search: U", "mcg_gribov_search: G", stream))) return rc;
     // each copy starts as U^Omega0 with its own random Omega0; the fix then
     // accumulates onto Omega0, so G ends as the total transform of the copy
     const bool keep = rounds_to_fp32(params, precision);

@@ -160,48 +160,44 @@ __global__ void k_identity_gauge(cplx<T>* __restrict__ G, Geom g, int nfields) {
 }
 
 // ---------------------------------------------------------------------------
-// gauge transform, in place: U_mu(x) <- Omega(x) U_mu(x) Omega(x+mu)^dag
-// thread per (field, parity, site)
+// gauge transform, in place: U_mu(x) <- Omega(x) U_mu(x) Omega(x+mu)^dag, in FP64
+// for fields of either precision.  Thread per link: the FP64 pipe bounds it (216
+// FMA per link), and a thread per site left small lattices on few SMs (60 us per
+// launch at 5 760, 8 192 and 20 736 sites alike; 24 launches of a 12-field search).
 // ---------------------------------------------------------------------------
-template <typename TU, typename TG>
-__device__ __forceinline__ void apply_site(cplx<TU>* __restrict__ U, const cplx<TG>* __restrict__ G, const Geom& g,
-                                           int p, int s) {
-    int c[4];
-    eo_coords(g, p, s, c);
-    cplx<double> Om[9];
-#pragma unroll
-    for (int e = 0; e < 9; ++e) {
-        const cplx<TG> v = G[gidx(g, p, e, s)];
-        Om[e] = mk((double)v.x, (double)v.y);
-    }
-#pragma unroll
-    for (int mu = 0; mu < 4; ++mu) {
-        const int sf = eo_neighbor(g, c, mu, +1);
-        cplx<double> u[9], on[9], t[9];
-#pragma unroll
-        for (int e = 0; e < 9; ++e) {
-            const cplx<TU> v = U[lidx(g, mu, p, e, s)];
-            u[e] = mk((double)v.x, (double)v.y);
-            const cplx<TG> w = G[gidx(g, p ^ 1, e, sf)];
-            on[e] = mk((double)w.x, (double)w.y);
-        }
-        m3_mul(Om, u, t);
-        m3_mul_nd(t, on, u);
-#pragma unroll
-        for (int e = 0; e < 9; ++e) U[lidx(g, mu, p, e, s)] = mk((TU)u[e].x, (TU)u[e].y);
-    }
-}
+constexpr int kApplyThreads = 64;
 
 template <typename T>
-__global__ void __launch_bounds__(FT) k_apply_gauge(cplx<T>* __restrict__ U, const cplx<T>* __restrict__ G, Geom g,
-                                                     int nfields) {
-    const long long n = 2LL * g.vh * nfields;
+__global__ void __launch_bounds__(kApplyThreads) k_apply_gauge(cplx<T>* __restrict__ Uall,
+                                                               const cplx<T>* __restrict__ Gall, Geom g, int nfields) {
     const long long id = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (id >= n) return;
-    const int f = (int)(id / (2LL * g.vh));
-    const int r = (int)(id - (long long)f * 2 * g.vh);
+    if (id >= 8LL * g.vh * nfields) return;
+    const int f = (int)(id / (8LL * g.vh));
+    int r = (int)(id - (long long)f * 8 * g.vh);
+    const int mu = r / (2 * g.vh);
+    r -= mu * 2 * g.vh;
     const int p = r / g.vh, s = r - p * g.vh;
-    apply_site<T, T>(U + (size_t)f * link_elems(g), G + (size_t)f * gauge_elems(g), g, p, s);
+    cplx<T>* U = Uall + (size_t)f * link_elems(g);
+    const cplx<T>* G = Gall + (size_t)f * gauge_elems(g);
+    int c[4];
+    eo_coords(g, p, s, c);
+    const int sf = eo_neighbor(g, c, mu, +1);
+    cplx<double> u[9], om[9], t[9];
+#pragma unroll
+    for (int e = 0; e < 9; ++e) {
+        const cplx<T> v = U[lidx(g, mu, p, e, s)], w = G[gidx(g, p, e, s)];
+        u[e] = mk((double)v.x, (double)v.y);
+        om[e] = mk((double)w.x, (double)w.y);
+    }
+    m3_mul(om, u, t);
+#pragma unroll
+    for (int e = 0; e < 9; ++e) {
+        const cplx<T> w = G[gidx(g, p ^ 1, e, sf)];
+        om[e] = mk((double)w.x, (double)w.y);
+    }
+    m3_mul_nd(t, om, u);
+#pragma unroll
+    for (int e = 0; e < 9; ++e) U[lidx(g, mu, p, e, s)] = mk((T)u[e].x, (T)u[e].y);
 }
 
 template <typename T>
@@ -227,9 +223,10 @@ __global__ void __launch_bounds__(FT) k_reunit_all(cplx<T>* __restrict__ M, int 
 // Mixed-precision hand-off, pass 1: W64 = reunit(W) written to scratch (W in
 // the compact FP32 form: rows 0 and 1; the FP64 re-unitarisation rebuilds row
 // 2 from them), G64 <- reunit(W64 G64).
-__global__ void __launch_bounds__(FT) k_handoff_gauge(const float4* __restrict__ W, const float4* __restrict__ Wlo,
-                                                      cplx<double>* __restrict__ W64, cplx<double>* __restrict__ G,
-                                                      Geom g, int nfields) {
+__global__ void __launch_bounds__(kApplyThreads) k_handoff_gauge(const float4* __restrict__ W,
+                                                                 const float4* __restrict__ Wlo,
+                                                                 cplx<double>* __restrict__ W64,
+                                                                 cplx<double>* __restrict__ G, Geom g, int nfields) {
     const long long n = 2LL * g.vh * nfields;
     const long long id = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (id >= n) return;
@@ -499,11 +496,27 @@ int launch_unpack_center(const int8_t* Z, int8_t* canon, const Geom& g, int nfie
 // if max_ij |(M M^dag - 1)_ij| > tol or if |det M - 1| > tol (FP32 arithmetic:
 // its rounding, ~1e-7, is far below the tolerances used).  bad[0]: number of
 // failing matrices; bad[1]: smallest failing global matrix index.
+// One launch checks the fields of a table (bad: two numbers per field): a search
+// over 12 fields made 24 launches with a read-back each.
+struct CheckTable {
+    static constexpr int kMax = 32;  // by value, within the 4 KB of kernel arguments
+    const void* M[kMax];
+    size_t vh[kMax], nmat[kMax];
+    int nslots[kMax];
+    unsigned blk0[kMax + 1];
+    int n;
+};
 template <typename T>
-__global__ void k_check_su3(const cplx<T>* __restrict__ M, int nslots, size_t vh, size_t nmat, float tol,
-                            bool finite_only, unsigned long long* __restrict__ bad) {
-    const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= nmat) return;
+__global__ void __launch_bounds__(FT) k_check_su3(const __grid_constant__ CheckTable tab, float tol, bool finite_only,
+                                                  unsigned long long* __restrict__ bad) {
+    int item = 0;
+    while (blockIdx.x >= tab.blk0[item + 1]) ++item;
+    const size_t i = (size_t)(blockIdx.x - tab.blk0[item]) * blockDim.x + threadIdx.x;
+    if (i >= tab.nmat[item]) return;
+    const cplx<T>* __restrict__ M = (const cplx<T>*)tab.M[item];
+    const int nslots = tab.nslots[item];
+    const size_t vh = tab.vh[item];
+    bad += 2 * item;
     const size_t per_field = (size_t)nslots * vh;
     const size_t f = i / per_field, m = i % per_field;
     const cplx<T>* base = M + f * per_field * 9 + (m / vh) * 9 * vh + m % vh;
@@ -541,27 +554,42 @@ __global__ void k_check_su3(const cplx<T>* __restrict__ M, int nslots, size_t vh
     }
 }
 
-// the check of nfields fields; h_out: pinned {failing matrices, the first one}
-static int check_su3(const void* M, int prec, const Geom& g, int nslots, int nfields, bool finite_only,
-                     unsigned long long** h_out, cudaStream_t st) {
+// the check of n fields (or arrays of fields); h_out: pinned {failing matrices,
+// the first one} per item
+static int check_su3(const CheckItem* items, int n, int prec, bool finite_only, unsigned long long** h_out,
+                     cudaStream_t st) {
     int rc = 0;
-    unsigned long long* d_bad = (unsigned long long*)scratch_device("check.bad", 2 * sizeof(unsigned long long), &rc);
+    const size_t bytes = 2 * sizeof(unsigned long long) * n;
+    unsigned long long* d_bad = (unsigned long long*)scratch_device("check.bad", bytes, &rc);
     if (rc) return rc;
-    unsigned long long* h_bad = (unsigned long long*)scratch_host("check.bad", 2 * sizeof(unsigned long long), &rc);
+    unsigned long long* h_bad = (unsigned long long*)scratch_host("check.bad", bytes, &rc);
     if (rc) return rc;
-    MCG_CK(cudaMemsetAsync(d_bad, 0, sizeof(unsigned long long), st));
-    MCG_CK(cudaMemsetAsync(d_bad + 1, 0xff, sizeof(unsigned long long), st));
-    const size_t vh = (size_t)g.vh, nmat = (size_t)nslots * vh * nfields;
-    const unsigned nb = (unsigned)((nmat + FT - 1) / FT);
-    if (prec == MCG_F64)
-        k_check_su3<double><<<nb, FT, 0, st>>>((const cplx<double>*)M, nslots, vh, nmat, kSU3TolF64, finite_only,
-                                               d_bad);
-    else
-        k_check_su3<float><<<nb, FT, 0, st>>>((const cplx<float>*)M, nslots, vh, nmat, kSU3TolF32, finite_only,
-                                              d_bad);
-    MCG_CK(cudaGetLastError());
-    note_launches(1);
-    MCG_CK(cudaMemcpyAsync(h_bad, d_bad, 2 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, st));
+    for (int k = 0; k < n; ++k) {
+        h_bad[2 * k] = 0;
+        h_bad[2 * k + 1] = ~0ull;
+    }
+    MCG_CK(cudaMemcpyAsync(d_bad, h_bad, bytes, cudaMemcpyHostToDevice, st));
+    for (int k0 = 0; k0 < n; k0 += CheckTable::kMax) {
+        CheckTable tab;
+        tab.n = std::min(n - k0, CheckTable::kMax);
+        tab.blk0[0] = 0;
+        for (int k = 0; k < tab.n; ++k) {
+            const CheckItem& it = items[k0 + k];
+            tab.M[k] = it.M;
+            tab.vh[k] = (size_t)it.g.vh;
+            tab.nmat[k] = (size_t)it.nslots * it.g.vh * it.nfields;
+            tab.nslots[k] = it.nslots;
+            tab.blk0[k + 1] = tab.blk0[k] + (unsigned)((tab.nmat[k] + FT - 1) / FT);
+        }
+        const unsigned nb = tab.blk0[tab.n];
+        if (prec == MCG_F64)
+            k_check_su3<double><<<nb, FT, 0, st>>>(tab, kSU3TolF64, finite_only, d_bad + 2 * k0);
+        else
+            k_check_su3<float><<<nb, FT, 0, st>>>(tab, kSU3TolF32, finite_only, d_bad + 2 * k0);
+        MCG_CK(cudaGetLastError());
+        note_launches(1);
+    }
+    MCG_CK(cudaMemcpyAsync(h_bad, d_bad, bytes, cudaMemcpyDeviceToHost, st));
     MCG_CK(cudaStreamSynchronize(st));
     *h_out = h_bad;
     return 0;
@@ -570,16 +598,16 @@ static int check_su3(const void* M, int prec, const Geom& g, int nslots, int nfi
 int count_not_su3(const void* M, int prec, const Geom& g, int nslots, int nfields, unsigned long long* count,
                   cudaStream_t st) {
     unsigned long long* h_bad = nullptr;
-    int rc = check_su3(M, prec, g, nslots, nfields, false, &h_bad, st);
+    const CheckItem it{M, g, nslots, nfields, ""};
+    int rc = check_su3(&it, 1, prec, false, &h_bad, st);
     if (!rc) *count = h_bad[0];
     return rc;
 }
 
-int validate_su3(const void* M, int prec, const Geom& g, int nslots, int nfields, const char* what,
-                 cudaStream_t st, bool finite_only) {
-    unsigned long long* h_bad = nullptr;
-    int rc = check_su3(M, prec, g, nslots, nfields, finite_only, &h_bad, st);
-    if (rc) return rc;
+static int report_not_su3(const CheckItem& it, int prec, const unsigned long long* h_bad, bool finite_only) {
+    const Geom& g = it.g;
+    const int nslots = it.nslots;
+    const char* what = it.what;
     const size_t vh = (size_t)g.vh;
     if (h_bad[0] == 0) return 0;
     const size_t i = (size_t)h_bad[1], per_field = (size_t)nslots * vh;
@@ -599,6 +627,19 @@ int validate_su3(const void* M, int prec, const Geom& g, int nslots, int nfields
                  "in-parity site %zu)",
                  what, h_bad[0], prec == MCG_F64 ? kSU3TolF64 : kSU3TolF32, f, slot, s);
     return fail(MCG_BAD_INPUT, buf);
+}
+
+int validate_su3(const CheckItem* items, int n, int prec, cudaStream_t st, bool finite_only) {
+    unsigned long long* h_bad = nullptr;
+    int rc = check_su3(items, n, prec, finite_only, &h_bad, st);
+    for (int k = 0; k < n && !rc; ++k) rc = report_not_su3(items[k], prec, h_bad + 2 * k, finite_only);
+    return rc;
+}
+
+int validate_su3(const void* M, int prec, const Geom& g, int nslots, int nfields, const char* what,
+                 cudaStream_t st, bool finite_only) {
+    const CheckItem it{M, g, nslots, nfields, what};
+    return validate_su3(&it, 1, prec, st, finite_only);
 }
 
 // ---------------------------------------------------------------------------
@@ -692,11 +733,11 @@ int launch_identity_gauge(void* G, int prec, const Geom& g, int nfields, cudaStr
 }
 
 int launch_apply_gauge(void* U, const void* G, int prec, const Geom& g, int nfields, cudaStream_t st) {
-    const long long n = 2LL * g.vh * nfields;
+    const int nb = blocks_for(8LL * g.vh * nfields, kApplyThreads);
     if (prec == MCG_F64)
-        k_apply_gauge<double><<<blocks_for(n, FT), FT, 0, st>>>((cplx<double>*)U, (const cplx<double>*)G, g, nfields);
+        k_apply_gauge<double><<<nb, kApplyThreads, 0, st>>>((cplx<double>*)U, (const cplx<double>*)G, g, nfields);
     else
-        k_apply_gauge<float><<<blocks_for(n, FT), FT, 0, st>>>((cplx<float>*)U, (const cplx<float>*)G, g, nfields);
+        k_apply_gauge<float><<<nb, kApplyThreads, 0, st>>>((cplx<float>*)U, (const cplx<float>*)G, g, nfields);
     MCG_CK(cudaGetLastError());
     note_launches(1);
     return 0;
@@ -783,13 +824,10 @@ int launch_handoff(const void* W32, const void* W32lo, double* U64, double* G64,
     cplx<double>* W64 =
         (cplx<double>*)scratch_device("handoff.W64", sizeof(cplx<double>) * gauge_elems(g) * nfields, &rc);
     if (rc) return rc;
-    const long long n = 2LL * g.vh * nfields;
-    k_handoff_gauge<<<blocks_for(n, FT), FT, 0, st>>>((const float4*)W32, (const float4*)W32lo, W64,
-                                                      (cplx<double>*)G64, g, nfields);
-    k_apply_gauge<double><<<blocks_for(n, FT), FT, 0, st>>>((cplx<double>*)U64, W64, g, nfields);
-    MCG_CK(cudaGetLastError());
-    note_launches(2);
-    return 0;
+    k_handoff_gauge<<<blocks_for(2LL * g.vh * nfields, kApplyThreads), kApplyThreads, 0, st>>>(
+        (const float4*)W32, (const float4*)W32lo, W64, (cplx<double>*)G64, g, nfields);
+    note_launches(1);
+    return launch_apply_gauge(U64, W64, MCG_F64, g, nfields, st);
 }
 
 int launch_to_c12(const void* src, int src_prec, void* dst, const Geom& g, int nmat, int nfields, cudaStream_t st) {

@@ -249,6 +249,15 @@ constexpr float kSU3TolF32 = 1e-4f;
 // Synchronises the stream.
 int validate_su3(const void* M, int prec, const Geom& g, int nslots, int nfields, const char* what,
                  cudaStream_t st, bool finite_only = false);
+// The same for n arrays of fields with one synchronisation: the message is that
+// of the first item that fails.
+struct CheckItem {
+    const void* M;
+    Geom g;
+    int nslots, nfields;
+    const char* what;
+};
+int validate_su3(const CheckItem* items, int n, int prec, cudaStream_t st, bool finite_only = false);
 
 // Arithmetic throughput probes: tflops[0..2] = FP64 FMA, FP32 FMA, packed FP32
 // FMA (TFLOP/s, 2 flop per FMA lane), measured on the current device.

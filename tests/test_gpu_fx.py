@@ -244,3 +244,25 @@ def test_repeated_fixes_with_kept_graphs():
     mcg.mcg_release()
     for c in calls[::2]:
         assert run(*c, main) == first[c]
+
+
+# the input check of a batch in one launch per 32 arrays: the message is that of the first bad array in the order
+# U_0, G_0, U_1, ..., wherever its blocks lie, and no field is touched
+@pytest.mark.parametrize("prec", ["F64", "F32"])
+@pytest.mark.parametrize("bad,which", [(0, "U"), (15, "G"), (16, "U"), (19, "G")])
+def test_batched_input_check(prec, bad, which):
+    from paper_0807_0264_gb300 import mcg
+
+    prec = getattr(mcg, prec)
+    dl = [(2, 2, 2, 2), (6, 2, 10, 4), (4, 14, 2, 6)] * 6 + [(8, 8, 4, 4), (2, 4, 2, 2)]
+    Us = [mcg.mcg_pack_links(torch.from_numpy(synth.make_field(d, 1.0, i)).unsqueeze(0).cuda(), d, prec)
+          for i, d in enumerate(dl)]
+    Gs = [mcg.identity_gauge(d, 1, prec) for d in dl]
+    (Us if which == "U" else Gs)[bad].view(-1)[-1] += 0.5
+    Us[19].view(-1)[0] = float("nan")
+    before = [x.clone() for x in Us + Gs]
+    name = which if bad < 19 else "U"
+    with pytest.raises(RuntimeError, match=f"mcg_fix_batch: {name}: 1 matrices are not finite"):
+        mcg.mcg_fix_batch(Us, Gs, dl, mcg.Params(max_sweeps=2))
+    for x, y in zip(Us + Gs, before):
+        assert torch.equal(torch.nan_to_num(x, nan=9.0), torch.nan_to_num(y, nan=9.0))
