@@ -116,6 +116,27 @@ void* scratch_device(const char* name, size_t bytes, int* rc) {
     return b.p;
 }
 
+void* scratch_device_optional(const char* name, size_t bytes) {
+    std::lock_guard<std::mutex> lk(g_mu);
+    int rc = 0;
+    DeviceScratch& ds = cur(&rc);
+    if (rc) return nullptr;
+    Buf& b = ds.dev[name];
+    if (b.bytes >= bytes) return b.p;
+    void* p = nullptr;
+    if (cudaMalloc(&p, bytes) != cudaSuccess) {
+        cudaGetLastError();  // not the caller's error
+        return nullptr;
+    }
+    if (b.p) {
+        cudaDeviceSynchronize();
+        cudaFree(b.p);
+    }
+    b.p = p;
+    b.bytes = bytes;
+    return p;
+}
+
 void* scratch_host(const char* name, size_t bytes, int* rc) {
     std::lock_guard<std::mutex> lk(g_mu);
     DeviceScratch& ds = cur(rc);

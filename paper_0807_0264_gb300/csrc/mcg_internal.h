@@ -47,6 +47,9 @@ void note_phase(int prec, double ms, long long site_updates);
 // Named, grow-only device and pinned-host buffers cached per device; freed by
 // mcg_release().
 void* scratch_device(const char* name, size_t bytes, int* rc);
+// The same for memory that the caller can do without: null, and no error, when
+// there is none (the old buffer, if any, is kept).
+void* scratch_device_optional(const char* name, size_t bytes);
 void* scratch_host(const char* name, size_t bytes, int* rc);
 cudaStream_t capture_stream(int* rc);
 // n branch streams (and an event per stream, plus a fork event) for the

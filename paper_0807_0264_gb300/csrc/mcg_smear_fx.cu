@@ -2,6 +2,7 @@
 // mcg_smear.cu on fields held as 64-bit integers of unit 2^-60.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 
 #include "mcg_common.cuh"
@@ -10,6 +11,155 @@
 #include "mcg_smear_fx.cuh"
 
 namespace mcg {
+
+// ---------------------------------------------------------------------------
+// Over-improved steps: the rectangle staples of neighbouring links share their
+// three-link parts.  A first pass computes, per ordered pair of directions (a, b)
+// and site y, the corner K_ab(y) = U_a(y) U_b(y+a) and the two plaquette staples
+// that it closes, P_ab(y) = K_ab(y) U_a(y+b)^dag (from y to y + b) and
+// D_ab(y) = U_b(y)^dag K_ab(y) (from y + b to y + b + a): 9 products per link.
+// With them a link's plaquette staples are loads and its 18 rectangles take 30
+// products, 41 with the step's own two against 86 when every path is multiplied
+// out.  (Storing the other two corners of a plaquette as well would make 38, for
+// a third more memory.)  36 matrices per site: 5 184 bytes.  Measured, ms per
+// step, 12 x 10 x 14 x 22: 0.63 and 0.38, this pass included.
+// ---------------------------------------------------------------------------
+constexpr int kFxAux = 36;  // the 12 K, then the P, then the D
+__device__ __forceinline__ int fx_pair(int a, int b) { return 3 * a + (b < a ? b : b - 1); }
+
+__device__ __forceinline__ size_t fx_aux_idx(const Geom& g, int slot, int p, int s) {
+#ifdef MCG_CHECK
+    if (mcg_bad((unsigned)slot >= (unsigned)kFxAux || (unsigned)p >= 2u || (unsigned)s >= (unsigned)g.vh)) return 0;
+#endif
+    return ((size_t)(2 * slot + p) * 9) * g.vh + s;
+}
+
+// A factor of a path: kind 0 / 1: the link of direction mu / nu, 2 / 3: K_numu /
+// K_munu, 4 / 5: P, 6 / 7: D; displacement (dm, dn) of its site from x, daggered
+// or not
+struct FxAuxFactor {
+    signed char kind, dm, dn, dag;
+};
+// the shapes of c_fx_paths in their order
+__constant__ FxAuxFactor c_fx_aux_paths[8][3] = {
+    {{4, 0, 0, 0}, {0, 0, 0, 0}, {0, 0, 0, 0}},
+    {{7, 0, -1, 0}, {0, 0, 0, 0}, {0, 0, 0, 0}},
+    {{1, 0, 0, 0}, {4, 0, 1, 0}, {1, 1, 0, 1}},
+    {{1, 0, -1, 1}, {7, 0, -2, 0}, {1, 1, -1, 0}},
+    {{2, 0, 0, 0}, {5, 1, 0, 1}, {0, 0, 0, 0}},
+    {{1, 0, -1, 1}, {0, 0, -1, 0}, {5, 1, -1, 0}},
+    {{6, -1, 0, 0}, {0, 0, 1, 0}, {1, 1, 0, 1}},
+    {{6, -1, -1, 1}, {3, 0, -1, 0}, {0, 0, 0, 0}},
+};
+__constant__ signed char c_fx_aux_len[8] = {1, 1, 3, 3, 2, 3, 3, 2};
+
+// nine entries at base (stride vh), daggered or not
+__device__ __forceinline__ void fx_load_entries(const int4* __restrict__ base, size_t vh, bool dag, cfx* m) {
+    const size_t sr = vh * (dag ? 1 : 3), sc = vh * (dag ? 3 : 1);
+    const int sg = dag ? -1 : 1;
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            cfx v = fx_load(base + i * sr + j * sc);
+            v.im.h *= sg;
+            v.im.l *= sg;
+            m[3 * i + j] = v;
+        }
+}
+
+__device__ __forceinline__ void fx_aux_factor(const int4* __restrict__ U, const int4* __restrict__ A, const Geom& g,
+                                              const int c[4], int mu, int nu, FxAuxFactor f, cfx* m) {
+    int q[4];
+#pragma unroll
+    for (int d = 0; d < 4; ++d) {
+        const int v = c[d] + (d == mu ? f.dm : 0) + (d == nu ? f.dn : 0);
+        q[d] = v < 0 ? v + g.n[d] : (v >= g.n[d] ? v - g.n[d] : v);
+    }
+    const int p = (q[0] + q[1] + q[2] + q[3]) & 1;
+    const int s = eo_index(g, q);
+    const int4* base = f.kind < 2 ? U + lidx(g, f.kind ? nu : mu, p, 0, s)
+                                  : A + fx_aux_idx(g, 12 * ((f.kind >> 1) - 1) +
+                                                          ((f.kind & 1) ? fx_pair(mu, nu) : fx_pair(nu, mu)), p, s);
+    fx_load_entries(base, (size_t)g.vh, f.dag, m);
+}
+
+// fx_staple_sum of an over-improved step from the first pass's products
+__device__ __forceinline__ void fx_staple_sum_aux(const int4* __restrict__ U, const int4* __restrict__ A,
+                                                  const Geom& g, const int c[4], int mu, const FxSmear& P, cfx* a,
+                                                  cfx* b) {
+    long long C[18];
+#pragma unroll
+    for (int e = 0; e < 18; ++e) C[e] = 0;
+#pragma unroll 1
+    for (int k = 7; k >= 0; --k) {
+        const int nf = c_fx_aux_len[k];
+        if (k == 1) {
+#pragma unroll
+            for (int e = 0; e < 18; ++e) C[e] = fx_mul(fx_split(C[e]), P.wr);
+        }
+#pragma unroll 1
+        for (int nu = 0; nu < 4; ++nu) {
+            if (nu == mu) continue;
+            fx_aux_factor(U, A, g, c, mu, nu, c_fx_aux_paths[k][0], a);
+#pragma unroll 1
+            for (int j = 1; j < nf; ++j) {
+                fx_aux_factor(U, A, g, c, mu, nu, c_fx_aux_paths[k][j], b);
+                m3fx_mul_inplace<false>(a, b);
+            }
+#pragma unroll
+            for (int e = 0; e < 9; ++e) {
+                if (k < 2) {
+                    C[2 * e] += fx_mul(a[e].re, P.wp);
+                    C[2 * e + 1] += fx_mul(a[e].im, P.wp);
+                } else {
+                    C[2 * e] += fx_join(a[e].re) >> 3;
+                    C[2 * e + 1] += fx_join(a[e].im) >> 3;
+                }
+            }
+        }
+    }
+#pragma unroll
+    for (int e = 0; e < 9; ++e) {
+        a[e].re = fx_split(C[2 * e]);
+        a[e].im = fx_split(C[2 * e + 1]);
+    }
+}
+
+// the first pass: thread per (field, pair, parity, site)
+__global__ void __launch_bounds__(128, 3) k_smear_products_fx(const int4* __restrict__ Uin, int4* __restrict__ Aux,
+                                                              Geom g, int nfields) {
+    const long long id = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (id >= 24LL * g.vh * nfields) return;
+    const int f = (int)(id / (24LL * g.vh));
+    int r = (int)(id - (long long)f * 24 * g.vh);
+    const int pair = r / (2 * g.vh), da = pair / 3, pb = pair - 3 * da, db = pb < da ? pb : pb + 1;
+    r -= pair * 2 * g.vh;
+    const int p = r / g.vh, s = r - p * g.vh;
+    const size_t vh = (size_t)g.vh;
+    const int4* U = Uin + (size_t)f * link_elems(g);
+    int4* out = Aux + (size_t)f * (kFxAux / 4) * link_elems(g) + fx_aux_idx(g, pair, p, s);
+    const size_t kind = 12 * 18 * vh;  // from one kind of product to the next
+    int c[4];
+    eo_coords(g, p, s, c);
+    const int sa = eo_neighbor(g, c, da, +1), sb = eo_neighbor(g, c, db, +1);
+    cfx K[9], a[9], b[9];
+    fx_load_entries(U + lidx(g, da, p, 0, s), vh, false, K);
+    fx_load_entries(U + lidx(g, db, p ^ 1, 0, sa), vh, false, b);
+    m3fx_mul_inplace<false>(K, b);
+#pragma unroll
+    for (int e = 0; e < 9; ++e) out[e * vh] = fx_pack(K[e]);
+    fx_load_entries(U + lidx(g, da, p ^ 1, 0, sb), vh, true, b);
+#pragma unroll
+    for (int e = 0; e < 9; ++e) a[e] = K[e];
+    m3fx_mul_inplace<false>(a, b);
+#pragma unroll
+    for (int e = 0; e < 9; ++e) out[kind + e * vh] = fx_pack(a[e]);
+    fx_load_entries(U + lidx(g, db, p, 0, s), vh, true, a);
+    m3fx_mul_inplace<false>(a, K);
+#pragma unroll
+    for (int e = 0; e < 9; ++e) out[2 * kind + e * vh] = fx_pack(a[e]);
+}
 
 // exp(iQ) with Q = 2 x, x traceless Hermitian of spectral radius at most 0.67.
 // Powers of x reduce by Cayley-Hamilton, x^3 = c1 x + c0:
@@ -56,12 +206,14 @@ __device__ __forceinline__ void fx_exp(const fx (&d)[3], const cfx (&x)[3], cons
 // the last step).
 // Bound by the integer multiplier.  Measured on 20^3 x 40: 0.96 ms per stout
 // step (the FP64 kernel: 4.88 ms, FP64 pipe 93 % busy); over-improved steps on
-// 12 x 10 x 14 x 22: 0.63 ms (2.70 ms).  3 blocks of 128 per SM: 2 blocks take
+// 12 x 10 x 14 x 22: 0.38 ms (2.70 ms; without the first pass's products 0.63).  3 blocks of 128 per SM: 2 blocks take
 // 12 %, 4 (spilling) 4 % longer.  Deviation from a 128-bit reference (4^4, ten
 // stout steps): 7.5e-17 rms, the FP64 kernel's 2.2e-16.
-template <bool RECT, bool OUT64>
-__global__ void __launch_bounds__(128, 3) k_smear_step_fx(const int4* __restrict__ Uin, int4* __restrict__ Uout,
-                                                          Geom g, int nfields, const __grid_constant__ FxSmear P) {
+enum { kPlaquettes, kRectangles, kRectanglesFromProducts };
+template <int MODE, bool OUT64>
+__global__ void __launch_bounds__(128, 3) k_smear_step_fx(const int4* __restrict__ Uin, const int4* __restrict__ Aux,
+                                                          int4* __restrict__ Uout, Geom g, int nfields,
+                                                          const __grid_constant__ FxSmear P) {
     const long long n = 8LL * g.vh * nfields;
     const long long id = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (id >= n) return;
@@ -75,7 +227,10 @@ __global__ void __launch_bounds__(128, 3) k_smear_step_fx(const int4* __restrict
     eo_coords(g, p, s, c);
 
     cfx a[9], b[9];
-    fx_staple_sum<RECT>(U, g, c, mu, P, a, b);
+    if (MODE == kRectanglesFromProducts)
+        fx_staple_sum_aux(U, Aux + (size_t)f * (kFxAux / 4) * link_elems(g), g, c, mu, P, a, b);
+    else
+        fx_staple_sum<MODE == kRectangles>(U, g, c, mu, P, a, b);
     const int4* ul = U + lidx(g, mu, p, 0, s);
 #pragma unroll
     for (int e = 0; e < 9; ++e) b[e] = fx_load(ul + (size_t)e * g.vh);
@@ -144,6 +299,11 @@ FxSmear fx_smear_params(double rho, double eps, double slack) {
     return P;
 }
 
+// Scratch of the over-improved step's products at most: 3.3 million sites at a
+// time.  A field beyond it, or with no memory for it, takes the step that
+// multiplies every path out.
+constexpr size_t kFxAuxBytes = (size_t)16 << 30;
+
 int run_smear_fx(const void* Uin, void* Uout, const Geom& g, int nfields, double rho, double eps, int n,
                  cudaStream_t st) {
     const size_t elems = link_elems(g) * (size_t)nfields;
@@ -155,25 +315,36 @@ int run_smear_fx(const void* Uin, void* Uout, const Geom& g, int nfields, double
     // step k's source: tmp or Uout in turn, so that the last step reads tmp
     auto buf = [&](int k) { return (n - 1 - k) % 2 == 0 ? tmp : Uout; };
     launch_to_fx(Uin, buf(0), elems, st);
-    const unsigned nb = (unsigned)((8LL * g.vh * nfields + 127) / 128);
+    // fields per pass: all, or as many as the products' scratch has room for
+    int chunk = nfields;
+    int4* aux = nullptr;
+    if (rect) {
+        const size_t per_field = 16 * (kFxAux / 4) * link_elems(g);
+        chunk = (int)std::min<size_t>(nfields, kFxAuxBytes / per_field);
+        if (chunk > 0) aux = (int4*)scratch_device_optional("smear.products", per_field * chunk);
+        if (!aux) chunk = nfields;
+    }
     for (int k = 0; k < n; ++k) {
-        const int4* src = (const int4*)buf(k);
         const bool last = k + 1 == n;
-        int4* dst = (int4*)(last ? Uout : buf(k + 1));
-        if (rect) {
-            if (last)
-                k_smear_step_fx<true, true><<<nb, 128, 0, st>>>(src, dst, g, nfields, P);
-            else
-                k_smear_step_fx<true, false><<<nb, 128, 0, st>>>(src, dst, g, nfields, P);
-        } else {
-            if (last)
-                k_smear_step_fx<false, true><<<nb, 128, 0, st>>>(src, dst, g, nfields, P);
-            else
-                k_smear_step_fx<false, false><<<nb, 128, 0, st>>>(src, dst, g, nfields, P);
+        for (int f0 = 0; f0 < nfields; f0 += chunk) {
+            const int nf = std::min(chunk, nfields - f0);
+            const size_t off = (size_t)f0 * link_elems(g);
+            const int4* src = (const int4*)buf(k) + off;
+            int4* dst = (int4*)(last ? Uout : buf(k + 1)) + off;
+            if (aux) {
+                k_smear_products_fx<<<(unsigned)((24LL * g.vh * nf + 127) / 128), 128, 0, st>>>(src, aux, g, nf);
+                note_launches(1);
+            }
+            const auto step = !rect ? (last ? k_smear_step_fx<kPlaquettes, true> : k_smear_step_fx<kPlaquettes, false>)
+                              : aux ? (last ? k_smear_step_fx<kRectanglesFromProducts, true>
+                                            : k_smear_step_fx<kRectanglesFromProducts, false>)
+                                    : (last ? k_smear_step_fx<kRectangles, true> : k_smear_step_fx<kRectangles, false>);
+            step<<<(unsigned)((8LL * g.vh * nf + 127) / 128), 128, 0, st>>>(src, aux, dst, g, nf, P);
+            note_launches(1);
         }
     }
     MCG_CK(cudaGetLastError());
-    note_launches(n + 1);
+    note_launches(1);
     return 0;
 }
 
