@@ -244,6 +244,13 @@ int mcg_reunitarise(void* M, int which, const mcg_lattice* lat, cudaStream_t str
  * U_in and U_out are fields of lat (U_out must not overlap U_in); n = 0 copies.
  * U_in is validated first (see "Input validation"; synchronises), then the
  * steps run asynchronously on `stream`.
+ * FP64 fields with |rho| (6 |5-2eps| / 3 + 18 |1-eps| / 12) <= 1 take the steps
+ * in 64-bit fixed point of unit 2^-60 (errors below the FP64 arithmetic's), on
+ * a scratch copy of the field and, for eps != 1, up to 16 GiB of scratch for
+ * products that neighbouring links share; without memory for the one or the
+ * other they run in FP64 (one step needs no scratch then) or without the
+ * sharing.  Calls on several streams are ordered on the GPU where they share
+ * scratch.
  */
 int mcg_smear(const void* U_in, void* U_out, const mcg_lattice* lat, double rho, double eps, int n,
               cudaStream_t stream);
@@ -284,7 +291,9 @@ int mcg_fix(void* U, void* G, const mcg_lattice* lat, const mcg_params* params, 
  * precision MCG_F32: the solve of the FP32 and double-float sweeps (A and b
  * rounded to FP32, Newton from a = e0 on the KKT system with its certificate
  * that the multiplier lies above lambda_max(A), else FP32 Jacobi + secular);
- * MCG_F64: the solve of the exact FP64 sweep.  In the hard case (b orthogonal
+ * MCG_F64: the solve of the exact sweep in FP64 arithmetic (the plain FP64
+ * sweep of validated fields solves the same problem in fixed point, with this
+ * solve where its own does not settle).  In the hard case (b orthogonal
  * to the top eigenspace, a maximum that is not unique) any maximiser may be
  * returned.  n = 0 does nothing; n < 0, a null array (n > 0) or another
  * precision return MCG_BAD_ARG.  Asynchronous on `stream`.
@@ -510,8 +519,12 @@ int mcg_gribov_search(const mcg_field* copies, int ncopies, const int* config_of
  * mcg_smear, Sec. II.B): Gin = gradient w.r.t. U given Gout w.r.t. U'.
  * Chain rule per link: Gin += exp(iQ)^dag Gout; the adjoint of exp's Frechet
  * derivative B = L(iQ, U Gout^dag); its traceless anti-Hermitian part K; then
- * Gin += K C on the link and rho U^dag K scattered over every factor of every
- * staple (atomic FP64 adds: summation order, hence the last bits, vary).
+ * Gin += K C on the link and rho U^dag K carried to every factor of every
+ * staple.  In 64-bit fixed point, each link gathering its terms (reproducible
+ * bits), under the rule of mcg_smear and for links that are near-unitary;
+ * otherwise, while `stream` is being captured and where there is no memory for
+ * the scratch (two fields), in FP64 with atomic adds (summation order, hence
+ * the last bits, vary).
  * U: the step's input field (FP64); Gout, Gin: FP64, link layout, distinct. */
 int mcg_smear_backward_step(const void* U, const double* Gout, double* Gin, const mcg_lattice* lat, double rho,
                             double eps, cudaStream_t stream);
@@ -564,8 +577,10 @@ int mcg_time_halfsweep(void* U, void* G, const mcg_lattice* lat, int parity, int
 int mcg_plaquette_static(const void* U, double* out, const mcg_lattice* lat, cudaStream_t stream);
 
 /* Threads per block of the half-sweep kernel for one precision, one thread
- * per site: FP64 64 or 128, FP32 64, 128 or 256; 128 by default.  A process-wide tuning setting (not part of the paper's
- * method): Python's autotune_sweep_block() times the choices with
+ * per site: FP64 64 or 128, FP32 64, 128 or 256; 128 by default.  (The plain
+ * FP64 sweep chooses its own shape by the number of sites; the setting applies
+ * to FP64 sweeps with the FP32 local solve.)  A process-wide tuning setting
+ * (not part of the paper's method): Python's autotune_sweep_block() times the choices with
  * mcg_time_halfsweep and keeps the fastest.  Returns MCG_BAD_ARG otherwise. */
 int mcg_set_sweep_block(int precision, int threads);
 int mcg_get_sweep_block(int precision);

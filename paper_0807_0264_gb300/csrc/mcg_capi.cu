@@ -83,6 +83,7 @@ struct DeviceScratch {
     std::vector<cudaStream_t> side;  // branch streams of captured per-field chains
     std::vector<cudaEvent_t> side_ev;
     cudaEvent_t fork_ev = nullptr;
+    std::map<std::string, cudaEvent_t> used;  // end of the last use of a group of buffers
 };
 static std::mutex g_mu;
 static std::map<int, DeviceScratch> g_scratch;
@@ -135,6 +136,27 @@ void* scratch_device_optional(const char* name, size_t bytes) {
     b.p = p;
     b.bytes = bytes;
     return p;
+}
+
+int scratch_wait(const char* group, cudaStream_t st) {
+    std::lock_guard<std::mutex> lk(g_mu);
+    int rc = 0;
+    DeviceScratch& ds = cur(&rc);
+    if (rc) return rc;
+    const auto it = ds.used.find(group);
+    if (it != ds.used.end()) MCG_CK(cudaStreamWaitEvent(st, it->second, 0));
+    return 0;
+}
+
+int scratch_mark(const char* group, cudaStream_t st) {
+    std::lock_guard<std::mutex> lk(g_mu);
+    int rc = 0;
+    DeviceScratch& ds = cur(&rc);
+    if (rc) return rc;
+    cudaEvent_t& ev = ds.used[group];
+    if (!ev) MCG_CK(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
+    MCG_CK(cudaEventRecord(ev, st));
+    return 0;
 }
 
 void* scratch_host(const char* name, size_t bytes, int* rc) {
@@ -214,6 +236,8 @@ void release_all() {
         for (auto s : kv.second.side) cudaStreamDestroy(s);
         for (auto ev : kv.second.side_ev) cudaEventDestroy(ev);
         if (kv.second.fork_ev) cudaEventDestroy(kv.second.fork_ev);
+        for (auto& ev : kv.second.used)
+            if (ev.second) cudaEventDestroy(ev.second);
     }
     g_scratch.clear();
     cudaSetDevice(dev);

@@ -50,6 +50,11 @@ void* scratch_device(const char* name, size_t bytes, int* rc);
 // The same for memory that the caller can do without: null, and no error, when
 // there is none (the old buffer, if any, is kept).
 void* scratch_device_optional(const char* name, size_t bytes);
+// Around an asynchronous use of a group of scratch buffers: the stream waits for
+// the group's last use, which may have been on another stream; the end of this
+// one.  Not for streams that are being captured.
+int scratch_wait(const char* group, cudaStream_t st);
+int scratch_mark(const char* group, cudaStream_t st);
 void* scratch_host(const char* name, size_t bytes, int* rc);
 cudaStream_t capture_stream(int* rc);
 // n branch streams (and an event per stream, plus a fork event) for the
@@ -335,7 +340,7 @@ int run_smear(const void* Uin, void* Uout, int prec, const Geom& g, int nfields,
 // FP64 smearing in fixed point (mcg_smear_fx.cu), n >= 1 steps of a validated
 // field: whether rho, eps meet its operand bounds, and the steps.
 bool smear_fx_applies(double rho, double eps);
-int run_smear_fx(const void* Uin, void* Uout, const Geom& g, int nfields, double rho, double eps, int n,
+int run_smear_fx(const void* Uin, void* Uout, const Geom& g, int nfields, double rho, double eps, int n, bool* ran,
                  cudaStream_t st);
 
 // ---- differentiation (mcg_smear.cu) -----------------------------------------

@@ -285,14 +285,19 @@ int run_smear(const void* Uin, void* Uout, int prec, const Geom& g, int nfields,
         return 0;
     }
     // FP64 fields in fixed point where its operand bounds hold (the paper's
-    // parameters: 0.6 and 0.77 of the limit); other rho, eps in FP64
-    if (prec == MCG_F64 && !keep_fp64 && smear_fx_applies(rho, eps))
-        return run_smear_fx(Uin, Uout, g, nfields, rho, eps, n, st);
+    // parameters: 0.6 and 0.77 of the limit); other rho, eps in FP64, as where
+    // there is no memory for the fixed-point copy (one step in FP64 needs none)
     int rc = 0;
+    if (prec == MCG_F64 && !keep_fp64 && smear_fx_applies(rho, eps)) {
+        bool ran = false;
+        rc = run_smear_fx(Uin, Uout, g, nfields, rho, eps, n, &ran, st);
+        if (rc || ran) return rc;
+    }
     void* tmp = nullptr;
     if (n >= 2) {
         tmp = scratch_device("smear.tmp", bytes, &rc);
         if (rc) return rc;
+        if ((rc = scratch_wait("smear", st))) return rc;
     }
     const double cp = (5.0 - 2.0 * eps) / 3.0, cr = -(1.0 - eps) / 12.0;
     const bool rect = cr != 0.0;
@@ -320,7 +325,7 @@ int run_smear(const void* Uin, void* Uout, int prec, const Geom& g, int nfields,
         note_launches(1);
         src = dst;
     }
-    return 0;
+    return n >= 2 ? scratch_mark("smear", st) : 0;
 }
 
 }  // namespace mcg
@@ -711,9 +716,16 @@ int run_smear_step_backward(const void* U, const double* Gout, double* Gin, cons
     const double cp = (5.0 - 2.0 * eps) / 3.0, cr = -(1.0 - eps) / 12.0;
     const long long n = 8LL * g.vh * nfields;
     unsigned* only = nullptr;
-    if (smear_fx_applies(rho, eps)) {
+    // The FP64 kernel alone while a graph is captured (the fixed-point kernels
+    // need scratch, which a graph that is launched later would share unordered
+    // with other calls) and where there is no memory for that scratch.
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    MCG_CK(cudaStreamIsCapturing(st, &cap));
+    if (cap == cudaStreamCaptureStatusNone && smear_fx_applies(rho, eps)) {
         int rc = run_smear_backward_fx(U, Gout, Gin, g, nfields, rho, eps, &only, st);
         if (rc) return rc;
+    }
+    if (only) {
         k_zero_if<<<(unsigned)((18 * n + 255) / 256), 256, 0, st>>>(Gin, 18 * n, only);
     } else {
         MCG_CK(cudaMemsetAsync(Gin, 0, 16 * link_elems(g) * (size_t)nfields, st));
@@ -722,7 +734,7 @@ int run_smear_step_backward(const void* U, const double* Gout, double* Gin, cons
                                                                     Gin, g, nfields, rho, cp, cr, only);
     MCG_CK(cudaGetLastError());
     note_launches(1);
-    return 0;
+    return only ? scratch_mark("bwd", st) : 0;
 }
 
 int run_functional_matrix_grad(const void* U, int prec, double* G, const Geom& g, int nfields, cudaStream_t st) {

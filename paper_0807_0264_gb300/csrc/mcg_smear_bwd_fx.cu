@@ -478,15 +478,12 @@ int run_smear_backward_fx(const void* U, const double* Gout, double* Gin, const 
                           double eps, unsigned** bad_out, cudaStream_t st) {
     const size_t elems = link_elems(g) * (size_t)nfields;
     const long long nlinks = 8LL * g.vh * nfields;
-    int rc = 0;
-    int4* Ufx = (int4*)scratch_device("bwd.U", 16 * elems, &rc);
-    if (rc) return rc;
-    int4* Y = (int4*)scratch_device("bwd.Y", 16 * elems, &rc);
-    if (rc) return rc;
-    int* ex = (int*)scratch_device("bwd.exp", sizeof(int) * nlinks, &rc);
-    if (rc) return rc;
-    unsigned* bad = (unsigned*)scratch_device("bwd.bad", sizeof(unsigned), &rc);
-    if (rc) return rc;
+    int4* Ufx = (int4*)scratch_device_optional("bwd.U", 16 * elems);
+    int4* Y = (int4*)scratch_device_optional("bwd.Y", 16 * elems);
+    int* ex = (int*)scratch_device_optional("bwd.exp", sizeof(int) * nlinks);
+    unsigned* bad = (unsigned*)scratch_device_optional("bwd.bad", sizeof(unsigned));
+    if (!Ufx || !Y || !ex || !bad) return 0;  // *bad_out stays null
+    if (int rc = scratch_wait("bwd", st)) return rc;
     *bad_out = bad;
     const FxSmear P = fx_smear_params(rho, eps, 1.2);
     MCG_CK(cudaMemsetAsync(bad, 0, sizeof(unsigned), st));

@@ -304,12 +304,13 @@ FxSmear fx_smear_params(double rho, double eps, double slack) {
 // multiplies every path out.
 constexpr size_t kFxAuxBytes = (size_t)16 << 30;
 
-int run_smear_fx(const void* Uin, void* Uout, const Geom& g, int nfields, double rho, double eps, int n,
+int run_smear_fx(const void* Uin, void* Uout, const Geom& g, int nfields, double rho, double eps, int n, bool* ran,
                  cudaStream_t st) {
     const size_t elems = link_elems(g) * (size_t)nfields;
-    int rc = 0;
-    void* tmp = scratch_device("smear.tmp", 16 * elems, &rc);
-    if (rc) return rc;
+    void* tmp = scratch_device_optional("smear.tmp", 16 * elems);
+    *ran = tmp != nullptr;
+    if (!tmp) return 0;
+    if (int rc = scratch_wait("smear", st)) return rc;
     const bool rect = eps != 1.0;
     const FxSmear P = fx_smear_params(rho, eps, 1.0);
     // step k's source: tmp or Uout in turn, so that the last step reads tmp
@@ -345,7 +346,7 @@ int run_smear_fx(const void* Uin, void* Uout, const Geom& g, int nfields, double
     }
     MCG_CK(cudaGetLastError());
     note_launches(1);
-    return 0;
+    return scratch_mark("smear", st);
 }
 
 // index-check counter of this unit (MCG_CHECK builds)

@@ -266,3 +266,35 @@ def test_batched_input_check(prec, bad, which):
         mcg.mcg_fix_batch(Us, Gs, dl, mcg.Params(max_sweeps=2))
     for x, y in zip(Us + Gs, before):
         assert torch.equal(torch.nan_to_num(x, nan=9.0), torch.nan_to_num(y, nan=9.0))
+
+
+# calls enqueued on several streams without a wait between them share the smearing scratch: each returns the bits of
+# its own call made alone.  In a captured graph (with no scratch allocated) the backward step runs the FP64 kernel:
+# both round ~300 times per link relative to the gradient's size, 1e-13
+def test_smear_calls_on_several_streams_and_captured():
+    from paper_0807_0264_gb300 import mcg
+
+    dims, gen = (8, 8, 8, 16), torch.Generator(device="cuda").manual_seed(5)
+    Us = [_pack(mcg, [synth.make_field(dims, 1.0, s)], dims) for s in range(4)]
+    Gs = [torch.randn(U.shape, dtype=U.dtype, device="cuda", generator=gen) for U in Us]
+    for eps, rho in ((1.0, 0.1), (-0.25, 0.06)):
+        alone = []
+        for U, G in zip(Us, Gs):
+            alone.append((mcg.mcg_smear(U, dims, rho, eps, 1), mcg.mcg_smear_backward_step(U, G, dims, rho, eps)))
+            torch.cuda.synchronize()
+        streams = [torch.cuda.Stream() for _ in Us]
+        outs = [[] for _ in Us]
+        for _ in range(3):
+            for st, U, G, o in zip(streams, Us, Gs, outs):
+                with torch.cuda.stream(st):
+                    o.append((mcg.mcg_smear(U, dims, rho, eps, 1), mcg.mcg_smear_backward_step(U, G, dims, rho, eps)))
+        torch.cuda.synchronize()
+        for o, (s, b) in zip(outs, alone):
+            assert all(torch.equal(x, s) and torch.equal(y, b) for x, y in o)
+        mcg.mcg_release()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            out = mcg.mcg_smear_backward_step(Us[0], Gs[0], dims, rho, eps)
+        graph.replay()
+        torch.cuda.synchronize()
+        assert float((out - alone[0][1]).abs().max()) < 1e-13 * float(alone[0][1].abs().max())
