@@ -148,8 +148,47 @@ __device__ __forceinline__ void exp_iQ(const cplx<T>* Q, cplx<T>* E) {
     }
 }
 
+// Sites x + a mu + b nu around a link's site x: lexicographic index, parity and
+// what the two directions need.  (The directions are runtime values: with the
+// coordinates in an array that they index, the array lay in local memory, and a
+// neighbour's index took four wraps.)
+struct Walk {
+    int lex, p, cm, nm, sm, cn, nn, sn;
+    __device__ __forceinline__ static void pick(const Geom& g, const int c[4], int d, int& cd, int& nd, int& sd) {
+        cd = c[0];
+        nd = g.n[0];
+        sd = 1;
+        int stride = g.n[0];
+#pragma unroll
+        for (int k = 1; k < 4; ++k) {
+            if (d == k) {
+                cd = c[k];
+                nd = g.n[k];
+                sd = stride;
+            }
+            stride *= g.n[k];
+        }
+    }
+    __device__ __forceinline__ Walk(const Geom& g, const int c[4], int parity, int mu) {
+        lex = c[0] + g.n[0] * (c[1] + g.n[1] * (c[2] + g.n[2] * c[3]));
+        p = parity;
+        pick(g, c, mu, cm, nm, sm);
+    }
+    __device__ __forceinline__ void set_nu(const Geom& g, const int c[4], int nu) { pick(g, c, nu, cn, nn, sn); }
+};
+
+template <typename T>
+__device__ __forceinline__ void ld(const cplx<T>* U, const Geom& g, int dir, const Walk& w, int a, int b, cplx<T>* m) {
+    const int q = w.lex + (wrapc(w.cm + a, w.nm) - w.cm) * w.sm + (wrapc(w.cn + b, w.nn) - w.cn) * w.sn;
+    load_link(U, g, dir, w.p ^ ((a + b) & 1), q >> 1, m);
+}
+
+// FP32 stout steps are bound by latency: 5 blocks of 128 per SM (96 registers; 3
+// at the 133 that the coordinate array took) and indices by Walk took the step on
+// 16^3 x 32 from 94 to 70 us (six blocks spill).  The rectangle steps keep their
+// indices: by Walk the compiler holds so many links that it spills.
 template <typename T, bool RECT>
-__global__ void __launch_bounds__(ST) k_smear_step(const cplx<T>* __restrict__ Uin, cplx<T>* __restrict__ Uout, Geom g,
+__global__ void __launch_bounds__(ST, sizeof(T) == 4 && !RECT ? 5 : 1) k_smear_step(const cplx<T>* __restrict__ Uin, cplx<T>* __restrict__ Uout, Geom g,
                                                    int nfields, T rho, T cp, T cr) {
     const long long n = 8LL * g.vh * nfields;
     const long long id = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -163,91 +202,100 @@ __global__ void __launch_bounds__(ST) k_smear_step(const cplx<T>* __restrict__ U
     int c[4];
     eo_coords(g, p, s, c);
 
+    Walk w(g, c, p, mu);
+
     cplx<T> C[9];
 #pragma unroll
     for (int e = 0; e < 9; ++e) C[e] = mk(T(0), T(0));
     cplx<T> a[9], b[9], t[9], t2[9];
     for (int nu = 0; nu < 4; ++nu) {
         if (nu == mu) continue;
+        if (!RECT) w.set_nu(g, c, nu);
+        auto at = [&](int dir, int a, int b, cplx<T>* m) {
+            if (RECT)
+                ld(U, g, dir, c, dsp(mu, a, nu, b), m);
+            else
+                ld(U, g, dir, w, a, b, m);
+        };
         // upper: U_nu(x) U_mu(x+nu) U_nu(x+mu)^dag
-        ld(U, g, nu, c, dsp(mu, 0, nu, 0), a);
-        ld(U, g, mu, c, dsp(mu, 0, nu, 1), b);
+        at(nu, 0, 0, a);
+        at(mu, 0, 1, b);
         m3_mul(a, b, t);
-        ld(U, g, nu, c, dsp(mu, 1, nu, 0), a);
+        at(nu, 1, 0, a);
         m3_mul_nd(t, a, t2);
         acc(C, t2, cp);
         // lower: U_nu(x-nu)^dag U_mu(x-nu) U_nu(x-nu+mu)
-        ld(U, g, nu, c, dsp(mu, 0, nu, -1), a);
-        ld(U, g, mu, c, dsp(mu, 0, nu, -1), b);
+        at(nu, 0, -1, a);
+        at(mu, 0, -1, b);
         m3_mul_dn(a, b, t);
-        ld(U, g, nu, c, dsp(mu, 1, nu, -1), a);
+        at(nu, 1, -1, a);
         m3_mul(t, a, t2);
         acc(C, t2, cp);
         if (RECT) {
             // 1x2, up: U_nu(x) U_nu(x+nu) U_mu(x+2nu) U_nu(x+mu+nu)^dag U_nu(x+mu)^dag
-            ld(U, g, nu, c, dsp(mu, 0, nu, 0), a);
-            ld(U, g, nu, c, dsp(mu, 0, nu, 1), b);
+            at(nu, 0, 0, a);
+            at(nu, 0, 1, b);
             m3_mul(a, b, t);
-            ld(U, g, mu, c, dsp(mu, 0, nu, 2), a);
+            at(mu, 0, 2, a);
             m3_mul(t, a, t2);
-            ld(U, g, nu, c, dsp(mu, 1, nu, 1), a);
+            at(nu, 1, 1, a);
             m3_mul_nd(t2, a, t);
-            ld(U, g, nu, c, dsp(mu, 1, nu, 0), a);
+            at(nu, 1, 0, a);
             m3_mul_nd(t, a, t2);
             acc(C, t2, cr);
             // 1x2, down: U_nu(x-nu)^dag U_nu(x-2nu)^dag U_mu(x-2nu) U_nu(x-2nu+mu) U_nu(x-nu+mu)
-            ld(U, g, nu, c, dsp(mu, 0, nu, -2), a);
-            ld(U, g, nu, c, dsp(mu, 0, nu, -1), b);
+            at(nu, 0, -2, a);
+            at(nu, 0, -1, b);
             m3_mul(a, b, t);  // U_nu(x-2nu) U_nu(x-nu)
-            ld(U, g, mu, c, dsp(mu, 0, nu, -2), a);
+            at(mu, 0, -2, a);
             m3_mul_dn(t, a, t2);  // (..)^dag U_mu(x-2nu)
-            ld(U, g, nu, c, dsp(mu, 1, nu, -2), a);
+            at(nu, 1, -2, a);
             m3_mul(t2, a, t);
-            ld(U, g, nu, c, dsp(mu, 1, nu, -1), a);
+            at(nu, 1, -1, a);
             m3_mul(t, a, t2);
             acc(C, t2, cr);
             // 2x1 forward, up: U_nu(x) U_mu(x+nu) U_mu(x+mu+nu) U_nu(x+2mu)^dag U_mu(x+mu)^dag
-            ld(U, g, nu, c, dsp(mu, 0, nu, 0), a);
-            ld(U, g, mu, c, dsp(mu, 0, nu, 1), b);
+            at(nu, 0, 0, a);
+            at(mu, 0, 1, b);
             m3_mul(a, b, t);
-            ld(U, g, mu, c, dsp(mu, 1, nu, 1), a);
+            at(mu, 1, 1, a);
             m3_mul(t, a, t2);
-            ld(U, g, nu, c, dsp(mu, 2, nu, 0), a);
+            at(nu, 2, 0, a);
             m3_mul_nd(t2, a, t);
-            ld(U, g, mu, c, dsp(mu, 1, nu, 0), a);
+            at(mu, 1, 0, a);
             m3_mul_nd(t, a, t2);
             acc(C, t2, cr);
             // 2x1 forward, down: U_nu(x-nu)^dag U_mu(x-nu) U_mu(x-nu+mu) U_nu(x-nu+2mu) U_mu(x+mu)^dag
-            ld(U, g, nu, c, dsp(mu, 0, nu, -1), a);
-            ld(U, g, mu, c, dsp(mu, 0, nu, -1), b);
+            at(nu, 0, -1, a);
+            at(mu, 0, -1, b);
             m3_mul_dn(a, b, t);
-            ld(U, g, mu, c, dsp(mu, 1, nu, -1), a);
+            at(mu, 1, -1, a);
             m3_mul(t, a, t2);
-            ld(U, g, nu, c, dsp(mu, 2, nu, -1), a);
+            at(nu, 2, -1, a);
             m3_mul(t2, a, t);
-            ld(U, g, mu, c, dsp(mu, 1, nu, 0), a);
+            at(mu, 1, 0, a);
             m3_mul_nd(t, a, t2);
             acc(C, t2, cr);
             // 2x1 backward, up: U_mu(x-mu)^dag U_nu(x-mu) U_mu(x-mu+nu) U_mu(x+nu) U_nu(x+mu)^dag
-            ld(U, g, mu, c, dsp(mu, -1, nu, 0), a);
-            ld(U, g, nu, c, dsp(mu, -1, nu, 0), b);
+            at(mu, -1, 0, a);
+            at(nu, -1, 0, b);
             m3_mul_dn(a, b, t);
-            ld(U, g, mu, c, dsp(mu, -1, nu, 1), a);
+            at(mu, -1, 1, a);
             m3_mul(t, a, t2);
-            ld(U, g, mu, c, dsp(mu, 0, nu, 1), a);
+            at(mu, 0, 1, a);
             m3_mul(t2, a, t);
-            ld(U, g, nu, c, dsp(mu, 1, nu, 0), a);
+            at(nu, 1, 0, a);
             m3_mul_nd(t, a, t2);
             acc(C, t2, cr);
             // 2x1 backward, down: U_mu(x-mu)^dag U_nu(x-mu-nu)^dag U_mu(x-mu-nu) U_mu(x-nu) U_nu(x-nu+mu)
-            ld(U, g, nu, c, dsp(mu, -1, nu, -1), a);
-            ld(U, g, mu, c, dsp(mu, -1, nu, 0), b);
+            at(nu, -1, -1, a);
+            at(mu, -1, 0, b);
             m3_mul(a, b, t);  // U_nu(x-mu-nu) U_mu(x-mu)
-            ld(U, g, mu, c, dsp(mu, -1, nu, -1), a);
+            at(mu, -1, -1, a);
             m3_mul_dn(t, a, t2);
-            ld(U, g, mu, c, dsp(mu, 0, nu, -1), a);
+            at(mu, 0, -1, a);
             m3_mul(t2, a, t);
-            ld(U, g, nu, c, dsp(mu, 1, nu, -1), a);
+            at(nu, 1, -1, a);
             m3_mul(t, a, t2);
             acc(C, t2, cr);
         }
