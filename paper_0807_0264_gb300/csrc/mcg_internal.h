@@ -120,6 +120,7 @@ struct SweepBatch {
     int reunit_every;
     double omega;  // over-relaxation parameter (1: plain relaxation)
     int solve32;   // FP64 sweeps: local problem built and solved in FP32
+    int spb = 0;              // sites per block
     int tps = 0;              // threads per site of the fixed-point FP64 sweep (0: another kernel)
     unsigned* bad = nullptr;  // unvalidated fields: sites left to the FP64 kernel
 };

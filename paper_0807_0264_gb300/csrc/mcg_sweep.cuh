@@ -701,6 +701,14 @@ __device__ __forceinline__ void warp_partial(double v, double* __restrict__ part
     if ((threadIdx.x & 31) == 0) partial[blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)] = v;
 }
 
+// At the entry of an FP64 odd half-sweep: whether its sweep is one after which
+// the field is re-unitarised (never when the field was done before it).
+__device__ __forceinline__ void reunit_due(const SweepBatch& bt, int f) {
+    if (bt.reunit_every <= 0 || threadIdx.x != 0 || blockIdx.x != bt.desc[f].blk0) return;
+    FieldState* st = &bt.state[f];
+    st->reunit_pending = !st->done && (st->sweep + 1) % bt.reunit_every == 0;
+}
+
 __device__ __forceinline__ int field_of_block(const FieldDesc* __restrict__ d, int nf, int b) {
     int lo = 0, hi = nf - 1;
     while (lo < hi) {

@@ -315,6 +315,7 @@ __global__ void __launch_bounds__(NT, MINB) k_halfsweep_fx(SweepBatch bt, int pa
     const double2 zero2 = make_double2(0.0, 0.0);
     extern __shared__ int4 fx_smem[];
     const int f = field_of_block(bt.desc, bt.nf, blockIdx.x);
+    if (ACC) reunit_due(bt, f);
     if (bt.state[f].done) return;  // block-uniform
     const FieldDesc fd = bt.desc[f];
     const Geom g = fd.geo;

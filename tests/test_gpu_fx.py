@@ -298,3 +298,22 @@ def test_smear_calls_on_several_streams_and_captured():
         graph.replay()
         torch.cuda.synchronize()
         assert float((out - alone[0][1]).abs().max()) < 1e-13 * float(alone[0][1].abs().max())
+
+
+# re-unitarisation in the kernel that ends the sweep: after every sweep, every third, and only past the last one; fields
+# of several sizes as chains and in one launch; the sweep test's bar of 1e-11 per link for fields near a maximum
+@pytest.mark.parametrize("every", [1, 3, 4])
+@pytest.mark.parametrize("copies", [1, 6])
+def test_reunitarise_at_the_end_of_a_sweep(every, copies):
+    from paper_0807_0264_gb300 import mcg
+
+    dl = [(2, 2, 2, 2), (4, 6, 2, 4), (6, 2, 10, 14)]
+    Uh = [synth.make_field(d, 0.4, i, gauge=False) for i, d in enumerate(dl)]
+    Us = [_pack(mcg, [U], d) for _ in range(copies) for U, d in zip(Uh, dl)]
+    Gs = [mcg.identity_gauge(d) for _ in range(copies) for d in dl]
+    mcg.mcg_fix_batch(Us, Gs, dl * copies, mcg.Params(tol=-1e300, max_sweeps=3, reunit_every=every, check_every=2))
+    refs = [oracle.fix(d, U, tol=-1e300, max_sweeps=3, reunit_every=every) for U, d in zip(Uh, dl)]
+    for k, (U, G) in enumerate(zip(Us, Gs)):
+        d, ref = dl[k % 3], refs[k % 3]
+        assert np.abs(mcg.mcg_unpack_links(U, d)[0].cpu().numpy() - ref["U"]).max() < 1e-11
+        assert np.abs(mcg.mcg_unpack_gauge(G, d)[0].cpu().numpy() - ref["G"]).max() < 1e-11
