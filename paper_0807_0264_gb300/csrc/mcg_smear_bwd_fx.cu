@@ -419,17 +419,7 @@ __global__ void __launch_bounds__(128, 3)
                         const FxPathFactor ft = c_fx_paths[k][m < nf ? m : m - nf - 1];
                         const int4* q =
                             U + link_at(g, c, ft.dir ? nu : mu, mu, ft.dm - fj.dm, nu, ft.dn - fj.dn);
-                        const size_t sr = vh * (ft.dag ? 1 : 3), sc = vh * (ft.dag ? 3 : 1);
-                        const int sg = ft.dag ? -1 : 1;
-#pragma unroll
-                        for (int i = 0; i < 3; ++i)
-#pragma unroll
-                            for (int h = 0; h < 3; ++h) {
-                                cfx v = fx_load(q + i * sr + h * sc);
-                                v.im.h *= sg;
-                                v.im.l *= sg;
-                                b[3 * i + h] = v;
-                            }
+                        fx_load_entries(q, vh, ft.dag, b);
                     }
                     if (t == 0) {
 #pragma unroll

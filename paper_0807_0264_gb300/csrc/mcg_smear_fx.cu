@@ -22,7 +22,7 @@ namespace mcg {
 // products, 41 with the step's own two against 86 when every path is multiplied
 // out.  (Storing the other two corners of a plaquette as well would make 38, for
 // a third more memory.)  36 matrices per site: 5 184 bytes.  Measured, ms per
-// step, 12 x 10 x 14 x 22: 0.63 and 0.38, this pass included.
+// step, 12 x 10 x 14 x 22: 0.63 and 0.37, this pass included.
 // ---------------------------------------------------------------------------
 constexpr int kFxAux = 36;  // the 12 K, then the P, then the D
 __device__ __forceinline__ int fx_pair(int a, int b) { return 3 * a + (b < a ? b : b - 1); }
@@ -52,21 +52,6 @@ __constant__ FxAuxFactor c_fx_aux_paths[8][3] = {
     {{6, -1, -1, 1}, {3, 0, -1, 0}, {0, 0, 0, 0}},
 };
 __constant__ signed char c_fx_aux_len[8] = {1, 1, 3, 3, 2, 3, 3, 2};
-
-// nine entries at base (stride vh), daggered or not
-__device__ __forceinline__ void fx_load_entries(const int4* __restrict__ base, size_t vh, bool dag, cfx* m) {
-    const size_t sr = vh * (dag ? 1 : 3), sc = vh * (dag ? 3 : 1);
-    const int sg = dag ? -1 : 1;
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int j = 0; j < 3; ++j) {
-            cfx v = fx_load(base + i * sr + j * sc);
-            v.im.h *= sg;
-            v.im.l *= sg;
-            m[3 * i + j] = v;
-        }
-}
 
 __device__ __forceinline__ void fx_aux_factor(const int4* __restrict__ U, const int4* __restrict__ A, const Geom& g,
                                               const int c[4], int mu, int nu, FxAuxFactor f, cfx* m) {
@@ -204,9 +189,9 @@ __device__ __forceinline__ void fx_exp(const fx (&d)[3], const cfx (&x)[3], cons
 
 // One thread per link, old field in, new field out (fixed point, or FP64 after
 // the last step).
-// Bound by the integer multiplier.  Measured on 20^3 x 40: 0.96 ms per stout
+// Bound by the integer multiplier.  Measured on 20^3 x 40: 0.93 ms per stout
 // step (the FP64 kernel: 4.88 ms, FP64 pipe 93 % busy); over-improved steps on
-// 12 x 10 x 14 x 22: 0.38 ms (2.70 ms; without the first pass's products 0.63).  3 blocks of 128 per SM: 2 blocks take
+// 12 x 10 x 14 x 22: 0.37 ms (2.70 ms; without the first pass's products 0.63).  3 blocks of 128 per SM: 2 blocks take
 // 12 %, 4 (spilling) 4 % longer.  Deviation from a 128-bit reference (4^4, ten
 // stout steps): 7.5e-17 rms, the FP64 kernel's 2.2e-16.
 enum { kPlaquettes, kRectangles, kRectanglesFromProducts };

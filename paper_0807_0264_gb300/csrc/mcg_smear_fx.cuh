@@ -41,6 +41,29 @@ struct FxSmear {
     int nterms;          // even
 };
 
+// The nine entries at base (stride vh); dag: of the adjoint, a transposed read
+// with the imaginary parts negated.  Addresses and signs by additions: products
+// for them go to the multiplier, which bounds the callers (3.5 % of a smearing
+// step).
+__device__ __forceinline__ void fx_load_entries(const int4* __restrict__ base, size_t vh, bool dag, cfx* m) {
+    const size_t sr = vh * (dag ? 16 : 48), sc = vh * (dag ? 48 : 16);
+    const int sg = dag ? -1 : 0;
+    const char* row = reinterpret_cast<const char*>(base);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        const char* q = row;
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            cfx v = fx_load(reinterpret_cast<const int4*>(q));
+            v.im.h = (v.im.h ^ sg) - sg;
+            v.im.l = (v.im.l ^ sg) - sg;
+            m[3 * i + j] = v;
+            q += sc;
+        }
+        row += sr;
+    }
+}
+
 // factor f of a staple path of the link (mu, c): its matrix, daggered (a
 // transposed read with the imaginary parts negated) where the path asks for it
 __device__ __forceinline__ void fx_factor(const int4* __restrict__ U, const Geom& g, const int c[4], int mu, int nu,
@@ -52,18 +75,7 @@ __device__ __forceinline__ void fx_factor(const int4* __restrict__ U, const Geom
         q[d] = v < 0 ? v + g.n[d] : (v >= g.n[d] ? v - g.n[d] : v);
     }
     const int p = (q[0] + q[1] + q[2] + q[3]) & 1;
-    const int4* base = U + lidx(g, f.dir ? nu : mu, p, 0, eo_index(g, q));
-    const size_t sr = (size_t)g.vh * (f.dag ? 1 : 3), sc = (size_t)g.vh * (f.dag ? 3 : 1);
-    const int sg = f.dag ? -1 : 1;
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int j = 0; j < 3; ++j) {
-            cfx v = fx_load(base + i * sr + j * sc);
-            v.im.h *= sg;
-            v.im.l *= sg;
-            m[3 * i + j] = v;
-        }
+    fx_load_entries(U + lidx(g, f.dir ? nu : mu, p, 0, eo_index(g, q)), (size_t)g.vh, f.dag, m);
 }
 
 __device__ __forceinline__ long long fx_abs2(cfx a) {
