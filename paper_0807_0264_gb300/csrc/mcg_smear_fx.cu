@@ -13,23 +13,27 @@
 namespace mcg {
 
 // ---------------------------------------------------------------------------
-// Over-improved steps: the rectangle staples of neighbouring links share their
-// three-link parts.  A first pass computes, per ordered pair of directions (a, b)
-// and site y, the corner K_ab(y) = U_a(y) U_b(y+a) and the two plaquette staples
-// that it closes, P_ab(y) = K_ab(y) U_a(y+b)^dag (from y to y + b) and
-// D_ab(y) = U_b(y)^dag K_ab(y) (from y + b to y + b + a): 9 products per link.
-// With them a link's plaquette staples are loads and its 18 rectangles take 30
-// products, 41 with the step's own two against 86 when every path is multiplied
-// out.  (Storing the other two corners of a plaquette as well would make 38, for
-// a third more memory.)  36 matrices per site: 5 184 bytes.  Measured, ms per
-// step, 12 x 10 x 14 x 22: 0.63 and 0.37, this pass included.
+// Products that neighbouring links share, from a first pass over ordered pairs of
+// directions (a, b) and sites y: the corner K_ab(y) = U_a(y) U_b(y+a) and, for
+// over-improved steps, the two plaquette staples that it closes,
+// P_ab(y) = K_ab(y) U_a(y+b)^dag (from y to y + b) and D_ab(y) = U_b(y)^dag K_ab(y)
+// (from y + b to y + b + a).
+// Stout: 3 products per link for the corners, then one per staple: 11 with the
+// step's own two instead of 14.  Over-improved: 9 per link, then the plaquette
+// staples are loads and the 18 rectangles take 30 products: 41 instead of 86.
+// (Storing the other two corners of a plaquette as well would make 38, for a
+// third more memory.)  12 or 36 matrices per site: 1 728 or 5 184 bytes.
+// Measured, ms per step with this pass, without and with the products: stout on
+// 20^3 x 40 0.93 and 0.89, on 16^4 0.198 and 0.191; over-improved on
+// 12 x 10 x 14 x 22 0.63 and 0.37.
 // ---------------------------------------------------------------------------
-constexpr int kFxAux = 36;  // the 12 K, then the P, then the D
+template <bool RECT>
+constexpr int kFxAux = RECT ? 36 : 12;  // matrices per site: the 12 K, then the P, then the D
 __device__ __forceinline__ int fx_pair(int a, int b) { return 3 * a + (b < a ? b : b - 1); }
 
 __device__ __forceinline__ size_t fx_aux_idx(const Geom& g, int slot, int p, int s) {
 #ifdef MCG_CHECK
-    if (mcg_bad((unsigned)slot >= (unsigned)kFxAux || (unsigned)p >= 2u || (unsigned)s >= (unsigned)g.vh)) return 0;
+    if (mcg_bad((unsigned)slot >= (unsigned)kFxAux<true> || (unsigned)p >= 2u || (unsigned)s >= (unsigned)g.vh)) return 0;
 #endif
     return ((size_t)(2 * slot + p) * 9) * g.vh + s;
 }
@@ -41,7 +45,7 @@ struct FxAuxFactor {
     signed char kind, dm, dn, dag;
 };
 // the shapes of c_fx_paths in their order
-__constant__ FxAuxFactor c_fx_aux_paths[8][3] = {
+__constant__ FxAuxFactor c_fx_aux_paths[10][3] = {
     {{4, 0, 0, 0}, {0, 0, 0, 0}, {0, 0, 0, 0}},
     {{7, 0, -1, 0}, {0, 0, 0, 0}, {0, 0, 0, 0}},
     {{1, 0, 0, 0}, {4, 0, 1, 0}, {1, 1, 0, 1}},
@@ -50,8 +54,11 @@ __constant__ FxAuxFactor c_fx_aux_paths[8][3] = {
     {{1, 0, -1, 1}, {0, 0, -1, 0}, {5, 1, -1, 0}},
     {{6, -1, 0, 0}, {0, 0, 1, 0}, {1, 1, 0, 1}},
     {{6, -1, -1, 1}, {3, 0, -1, 0}, {0, 0, 0, 0}},
+    // plaquettes from the corners alone
+    {{2, 0, 0, 0}, {1, 1, 0, 1}, {0, 0, 0, 0}},
+    {{1, 0, -1, 1}, {3, 0, -1, 0}, {0, 0, 0, 0}},
 };
-__constant__ signed char c_fx_aux_len[8] = {1, 1, 3, 3, 2, 3, 3, 2};
+__constant__ signed char c_fx_aux_len[10] = {1, 1, 3, 3, 2, 3, 3, 2, 2, 2};
 
 __device__ __forceinline__ void fx_aux_factor(const int4* __restrict__ U, const int4* __restrict__ A, const Geom& g,
                                               const int c[4], int mu, int nu, FxAuxFactor f, cfx* m) {
@@ -69,17 +76,18 @@ __device__ __forceinline__ void fx_aux_factor(const int4* __restrict__ U, const 
     fx_load_entries(base, (size_t)g.vh, f.dag, m);
 }
 
-// fx_staple_sum of an over-improved step from the first pass's products
-__device__ __forceinline__ void fx_staple_sum_aux(const int4* __restrict__ U, const int4* __restrict__ A,
+// fx_staple_sum from the first pass's products
+template <bool RECT>
+__device__ __forceinline__ void fx_staple_sum_shared(const int4* __restrict__ U, const int4* __restrict__ A,
                                                   const Geom& g, const int c[4], int mu, const FxSmear& P, cfx* a,
                                                   cfx* b) {
     long long C[18];
 #pragma unroll
     for (int e = 0; e < 18; ++e) C[e] = 0;
 #pragma unroll 1
-    for (int k = 7; k >= 0; --k) {
-        const int nf = c_fx_aux_len[k];
-        if (k == 1) {
+    for (int k = RECT ? 7 : 9; k >= (RECT ? 0 : 8); --k) {
+        const int nf = RECT ? c_fx_aux_len[k] : 2;
+        if (RECT && k == 1) {
 #pragma unroll
             for (int e = 0; e < 18; ++e) C[e] = fx_mul(fx_split(C[e]), P.wr);
         }
@@ -94,7 +102,10 @@ __device__ __forceinline__ void fx_staple_sum_aux(const int4* __restrict__ U, co
             }
 #pragma unroll
             for (int e = 0; e < 9; ++e) {
-                if (k < 2) {
+                if (!RECT) {
+                    C[2 * e] += fx_join(a[e].re);
+                    C[2 * e + 1] += fx_join(a[e].im);
+                } else if (k < 2) {
                     C[2 * e] += fx_mul(a[e].re, P.wp);
                     C[2 * e + 1] += fx_mul(a[e].im, P.wp);
                 } else {
@@ -106,12 +117,13 @@ __device__ __forceinline__ void fx_staple_sum_aux(const int4* __restrict__ U, co
     }
 #pragma unroll
     for (int e = 0; e < 9; ++e) {
-        a[e].re = fx_split(C[2 * e]);
-        a[e].im = fx_split(C[2 * e + 1]);
+        a[e].re = fx_split(RECT ? C[2 * e] : fx_mul(fx_split(C[2 * e]), P.wp));
+        a[e].im = fx_split(RECT ? C[2 * e + 1] : fx_mul(fx_split(C[2 * e + 1]), P.wp));
     }
 }
 
 // the first pass: thread per (field, pair, parity, site)
+template <bool RECT>
 __global__ void __launch_bounds__(128, 3) k_smear_products_fx(const int4* __restrict__ Uin, int4* __restrict__ Aux,
                                                               Geom g, int nfields) {
     const long long id = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -123,7 +135,7 @@ __global__ void __launch_bounds__(128, 3) k_smear_products_fx(const int4* __rest
     const int p = r / g.vh, s = r - p * g.vh;
     const size_t vh = (size_t)g.vh;
     const int4* U = Uin + (size_t)f * link_elems(g);
-    int4* out = Aux + (size_t)f * (kFxAux / 4) * link_elems(g) + fx_aux_idx(g, pair, p, s);
+    int4* out = Aux + (size_t)f * (kFxAux<RECT> / 4) * link_elems(g) + fx_aux_idx(g, pair, p, s);
     const size_t kind = 12 * 18 * vh;  // from one kind of product to the next
     int c[4];
     eo_coords(g, p, s, c);
@@ -134,6 +146,7 @@ __global__ void __launch_bounds__(128, 3) k_smear_products_fx(const int4* __rest
     m3fx_mul_inplace<false>(K, b);
 #pragma unroll
     for (int e = 0; e < 9; ++e) out[e * vh] = fx_pack(K[e]);
+    if (!RECT) return;
     fx_load_entries(U + lidx(g, da, p ^ 1, 0, sb), vh, true, b);
 #pragma unroll
     for (int e = 0; e < 9; ++e) a[e] = K[e];
@@ -189,13 +202,12 @@ __device__ __forceinline__ void fx_exp(const fx (&d)[3], const cfx (&x)[3], cons
 
 // One thread per link, old field in, new field out (fixed point, or FP64 after
 // the last step).
-// Bound by the integer multiplier.  Measured on 20^3 x 40: 0.93 ms per stout
-// step (the FP64 kernel: 4.88 ms, FP64 pipe 93 % busy); over-improved steps on
-// 12 x 10 x 14 x 22: 0.37 ms (2.70 ms; without the first pass's products 0.63).  3 blocks of 128 per SM: 2 blocks take
-// 12 %, 4 (spilling) 4 % longer.  Deviation from a 128-bit reference (4^4, ten
-// stout steps): 7.5e-17 rms, the FP64 kernel's 2.2e-16.
-enum { kPlaquettes, kRectangles, kRectanglesFromProducts };
-template <int MODE, bool OUT64>
+// Bound by the integer multiplier.  Measured on 20^3 x 40, first pass included:
+// 0.89 ms per stout step (the FP64 kernel: 4.88 ms, FP64 pipe 93 % busy);
+// over-improved steps on 12 x 10 x 14 x 22: 0.37 ms (2.70 ms).  3 blocks of 128
+// per SM: 2 blocks take 12 %, 4 (spilling) 4 % longer.  Deviation from a 128-bit reference (4^4, ten
+// stout steps): 8.5e-17 rms, the FP64 kernel's 2.2e-16.
+template <bool RECT, bool SHARED, bool OUT64>
 __global__ void __launch_bounds__(128, 3) k_smear_step_fx(const int4* __restrict__ Uin, const int4* __restrict__ Aux,
                                                           int4* __restrict__ Uout, Geom g, int nfields,
                                                           const __grid_constant__ FxSmear P) {
@@ -212,10 +224,10 @@ __global__ void __launch_bounds__(128, 3) k_smear_step_fx(const int4* __restrict
     eo_coords(g, p, s, c);
 
     cfx a[9], b[9];
-    if (MODE == kRectanglesFromProducts)
-        fx_staple_sum_aux(U, Aux + (size_t)f * (kFxAux / 4) * link_elems(g), g, c, mu, P, a, b);
+    if (SHARED)
+        fx_staple_sum_shared<RECT>(U, Aux + (size_t)f * (kFxAux<RECT> / 4) * link_elems(g), g, c, mu, P, a, b);
     else
-        fx_staple_sum<MODE == kRectangles>(U, g, c, mu, P, a, b);
+        fx_staple_sum<RECT>(U, g, c, mu, P, a, b);
     const int4* ul = U + lidx(g, mu, p, 0, s);
 #pragma unroll
     for (int e = 0; e < 9; ++e) b[e] = fx_load(ul + (size_t)e * g.vh);
@@ -284,9 +296,18 @@ FxSmear fx_smear_params(double rho, double eps, double slack) {
     return P;
 }
 
-// Scratch of the over-improved step's products at most: 3.3 million sites at a
-// time.  A field beyond it, or with no memory for it, takes the step that
-// multiplies every path out.
+template <bool RECT, bool SHARED>
+static auto step_kernel(bool out64) {
+    return out64 ? k_smear_step_fx<RECT, SHARED, true> : k_smear_step_fx<RECT, SHARED, false>;
+}
+static auto step_kernel(bool rect, bool shared, bool out64) {
+    return rect ? (shared ? step_kernel<true, true>(out64) : step_kernel<true, false>(out64))
+                : (shared ? step_kernel<false, true>(out64) : step_kernel<false, false>(out64));
+}
+
+// Scratch of the products at most: 9.9 million sites of a stout step, 3.3 million
+// of an over-improved one at a time.  A field beyond it, or with no memory for it,
+// takes the step that multiplies every path out.
 constexpr size_t kFxAuxBytes = (size_t)16 << 30;
 
 int run_smear_fx(const void* Uin, void* Uout, const Geom& g, int nfields, double rho, double eps, int n, bool* ran,
@@ -304,12 +325,10 @@ int run_smear_fx(const void* Uin, void* Uout, const Geom& g, int nfields, double
     // fields per pass: all, or as many as the products' scratch has room for
     int chunk = nfields;
     int4* aux = nullptr;
-    if (rect) {
-        const size_t per_field = 16 * (kFxAux / 4) * link_elems(g);
-        chunk = (int)std::min<size_t>(nfields, kFxAuxBytes / per_field);
-        if (chunk > 0) aux = (int4*)scratch_device_optional("smear.products", per_field * chunk);
-        if (!aux) chunk = nfields;
-    }
+    const size_t per_field = 16 * ((rect ? kFxAux<true> : kFxAux<false>) / 4) * link_elems(g);
+    chunk = (int)std::min<size_t>(nfields, kFxAuxBytes / per_field);
+    if (chunk > 0) aux = (int4*)scratch_device_optional("smear.products", per_field * chunk);
+    if (!aux) chunk = nfields;
     for (int k = 0; k < n; ++k) {
         const bool last = k + 1 == n;
         for (int f0 = 0; f0 < nfields; f0 += chunk) {
@@ -318,13 +337,11 @@ int run_smear_fx(const void* Uin, void* Uout, const Geom& g, int nfields, double
             const int4* src = (const int4*)buf(k) + off;
             int4* dst = (int4*)(last ? Uout : buf(k + 1)) + off;
             if (aux) {
-                k_smear_products_fx<<<(unsigned)((24LL * g.vh * nf + 127) / 128), 128, 0, st>>>(src, aux, g, nf);
+                (rect ? k_smear_products_fx<true> : k_smear_products_fx<false>)
+                    <<<(unsigned)((24LL * g.vh * nf + 127) / 128), 128, 0, st>>>(src, aux, g, nf);
                 note_launches(1);
             }
-            const auto step = !rect ? (last ? k_smear_step_fx<kPlaquettes, true> : k_smear_step_fx<kPlaquettes, false>)
-                              : aux ? (last ? k_smear_step_fx<kRectanglesFromProducts, true>
-                                            : k_smear_step_fx<kRectanglesFromProducts, false>)
-                                    : (last ? k_smear_step_fx<kRectangles, true> : k_smear_step_fx<kRectangles, false>);
+            const auto step = step_kernel(rect, aux != nullptr, last);
             step<<<(unsigned)((8LL * g.vh * nf + 127) / 128), 128, 0, st>>>(src, aux, dst, g, nf, P);
             note_launches(1);
         }
