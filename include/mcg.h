@@ -561,7 +561,7 @@ int mcg_time_halfsweep(void* U, void* G, const mcg_lattice* lat, int parity, int
  * Mean plaquette per field, like mcg_plaquette, for callers that cannot let
  * the library allocate device memory (the paper has no counterpart: this is
  * an interface variant).  Its only scratch, the per-block partial sums, is a
- * fixed 512 KiB array compiled into the library (65 536 doubles), so a call
+ * fixed 1 MiB array compiled into the library (131 072 doubles), so a call
  * needs nfields * ceil(V / 256) <= 65 536; larger requests return
  * MCG_BAD_ARG without touching the GPU.  out: DEVICE pointer to nfields
  * doubles, written asynchronously on `stream` (no synchronisation, no host

@@ -759,7 +759,8 @@ static int reduce_per_field(int which, const void* U, int prec, const Geom& g, i
                             cudaStream_t st) {
     const int bpf = blocks_for(2LL * g.vh, FT);
     int rc = 0;
-    double* partial = (double*)scratch_device("obs.partial", sizeof(double) * (size_t)bpf * nfields, &rc);
+    const int per_block = which == 0 ? 2 : 1;  // partial sums per block of FT sites
+    double* partial = (double*)scratch_device("obs.partial", sizeof(double) * per_block * (size_t)bpf * nfields, &rc);
     if (rc) return rc;
     double* d_out = (double*)scratch_device("obs.out", sizeof(double) * nfields, &rc);
     if (rc) return rc;
@@ -772,7 +773,7 @@ static int reduce_per_field(int which, const void* U, int prec, const Geom& g, i
         else
             k_functional_all<float><<<nb, FT, 0, st>>>((const cplx<float>*)U, g, bpf, partial);
     }
-    k_sum_partials<<<nfields, 256, 0, st>>>(partial, bpf, d_out);
+    k_sum_partials<<<nfields, 256, 0, st>>>(partial, per_block * bpf, d_out);
     MCG_CK(cudaGetLastError());
     note_launches(2);
     MCG_CK(cudaMemcpyAsync(out_host, d_out, sizeof(double) * nfields, cudaMemcpyDeviceToHost, st));
@@ -885,8 +886,8 @@ __global__ void k_static_finish(const double* __restrict__ partial, int bpf, dou
 // the process exits.
 namespace mcg {
 
-constexpr int kStaticPartials = 1 << 16;  // 65 536 doubles = 512 KiB
-static __device__ __align__(256) double g_static_partials[kStaticPartials];
+constexpr int kStaticPartials = 1 << 16;  // blocks of 256 sites, two partial sums each: 1 MiB
+static __device__ __align__(256) double g_static_partials[2 * kStaticPartials];
 
 static std::mutex g_static_mu;
 static double* g_static_addr[64];  // symbol address per device, resolved once
@@ -934,7 +935,7 @@ extern "C" int mcg_plaquette_static(const void* U, double* out, const mcg_lattic
     // every partial slot read below is written by its block first: nothing in
     // the shared array has to start at zero
     launch_plaquette_partials(U, lat->precision, g, (int)bpf, lat->nfields, partial, stream);
-    k_static_finish<<<lat->nfields, 256, 0, stream>>>(partial, (int)bpf, 1.0 / (6.0 * (double)V), out);
+    k_static_finish<<<lat->nfields, 256, 0, stream>>>(partial, 2 * (int)bpf, 1.0 / (6.0 * (double)V), out);
     MCG_CK(cudaGetLastError());
     note_launches(2);
     return MCG_OK;

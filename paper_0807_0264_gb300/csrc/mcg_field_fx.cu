@@ -160,24 +160,27 @@ __device__ __noinline__ double plaquette_f64(const V* a, const V* b, const V* c,
 
 // Per-block partial of the sum over sites of (1/3) Re tr of the six plaquettes:
 // X = U_mu(x) U_nu(x+mu) and Y = U_nu(x) U_mu(x+nu) row by row, sum Re X Y^*.
-// bpf blocks of 256 sites per field.  Measured on 20^3 x 40: 353 us (the FP64
-// kernel 917 us, FP64 pipe 93 %); one block per SM instead of two: 412 us.
+// Two threads per site, three planes each (mu = 0; mu = 1 and 2), 2 bpf blocks of
+// 128 sites per field: the six planes of a site are a serial chain, and whole
+// sites per thread made four full waves and a nearly empty one on 20^3 x 40.
+// Measured, us, with whole sites and so (2^4, 8^4, 16^4, 16^3 x 32, 20^3 x 40): 36
+// 52 89 163 361 and 29 31 87 148 349 (the FP64 kernel 917 on the last).
 template <typename T>
 __global__ void __launch_bounds__(256, 2) k_plaquette_fx(const void* Uall, Geom g, int bpf,
                                                          double* __restrict__ partial) {
     typedef typename Vec2<T>::type V;
-    const int f = blockIdx.x / bpf;
-    const int s2 = (blockIdx.x - f * bpf) * 256 + threadIdx.x;  // 0 .. 2*vh-1
+    const int f = blockIdx.x / (2 * bpf), half = threadIdx.x >> 7;
+    const int s2 = (blockIdx.x - f * 2 * bpf) * 128 + (threadIdx.x & 127);  // 0 .. 2*vh-1
     const V* U = reinterpret_cast<const V*>(Uall) + (size_t)f * link_elems(g);
     const size_t vh = (size_t)g.vh;
     double slow = 0.0;
-    long long acc = 0;  // units of 2^-57: at most 6 * 3.2
+    long long acc = 0;  // units of 2^-57: at most 3 * 3.2
     if (s2 < 2 * g.vh) {
         const int p = s2 / g.vh, s = s2 - p * g.vh;
         int c[4];
         eo_coords(g, p, s, c);
 #pragma unroll 1
-        for (int mu = 0; mu < 3; ++mu) {
+        for (int mu = half; mu < 1 + 2 * half; ++mu) {
             const int smu = eo_neighbor(g, c, mu, +1);
 #pragma unroll 1
             for (int nu = mu + 1; nu < 4; ++nu) {
@@ -252,7 +255,7 @@ int launch_handoff_fx(const void* W32, const void* W32lo, double* U64, double* G
 
 void launch_plaquette_partials(const void* U, int prec, const Geom& g, int bpf, int nfields, double* partial,
                                cudaStream_t st) {
-    const unsigned nb = (unsigned)bpf * nfields;
+    const unsigned nb = 2u * (unsigned)bpf * nfields;
     if (prec == MCG_F64)
         k_plaquette_fx<double><<<nb, 256, 0, st>>>(U, g, bpf, partial);
     else

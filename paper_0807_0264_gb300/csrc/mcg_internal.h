@@ -279,8 +279,8 @@ int launch_apply_gauge(void* U, const void* G, int prec, const Geom& g, int nfie
 int launch_reunitarise(void* M, int which, int prec, const Geom& g, int nfields, cudaStream_t st);
 // the same for FP64 fields in fixed point (mcg_field_fx.cu)
 int launch_apply_gauge_fx(void* U, const void* G, const Geom& g, int nfields, cudaStream_t st);
-// sums over sites of (1/3) Re tr of the six plaquettes, one per block of 256
-// sites, bpf blocks per field
+// sums over sites of (1/3) Re tr of the six plaquettes, one per 128 sites: 2 bpf
+// per field, bpf the blocks of 256 sites of a field
 void launch_plaquette_partials(const void* U, int prec, const Geom& g, int bpf, int nfields, double* partial,
                                cudaStream_t st);
 int compute_plaquette(const void* U, int prec, const Geom& g, int nfields, double* out_host, cudaStream_t st);
