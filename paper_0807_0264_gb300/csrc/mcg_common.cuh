@@ -271,6 +271,42 @@ __device__ __forceinline__ int eo_neighbor(const Geom& g, const int c[4], int mu
     return eo_index(g, d);
 }
 
+// Blocks of 128 threads over the links of fields (or other per-site items of ndir
+// kinds).  Tiled: 64 in-parity indices of both parities and one kind per block,
+// the kinds in turn.  All links of a site then run close together, and the
+// staples they share are read from DRAM once: with the direction as the slowest
+// index a field beyond L2 was streamed once per direction (stout steps, tiled and
+// not: FP64 20^3 x 40 0.81 and 0.89 ms, FP32 16^3 x 32 68 and 71 us).  Steps with
+// rectangles reach two sites far and go by the direction first (over-improved
+// FP64, 12 x 10 x 14 x 22: 0.40 ms tiled, 0.37).
+struct LinkItem {
+    int f, kind, p, s;
+};
+template <bool TILED>
+__device__ __forceinline__ bool link_item(const Geom& g, int ndir, int nfields, LinkItem& r) {
+    if (TILED) {
+        const unsigned tiles = ((unsigned)g.vh + 63) / 64, b = blockIdx.x / ndir;
+        r.kind = (int)(blockIdx.x - b * ndir);
+        r.f = (int)(b / tiles);
+        r.s = (int)(b - r.f * tiles) * 64 + (int)(threadIdx.x & 63);
+        r.p = (int)(threadIdx.x >> 6);
+        return r.s < g.vh;
+    }
+    const long long per = 2LL * ndir * g.vh, id = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (id >= per * nfields) return false;
+    r.f = (int)(id / per);
+    int k = (int)(id - r.f * per);
+    r.kind = k / (2 * g.vh);
+    k -= r.kind * 2 * g.vh;
+    r.p = k / g.vh;
+    r.s = k - r.p * g.vh;
+    return true;
+}
+static inline unsigned link_blocks(bool tiled, const Geom& g, int ndir, int nfields) {
+    return tiled ? (unsigned)ndir * (((unsigned)g.vh + 63) / 64) * (unsigned)nfields
+                 : (unsigned)((2LL * ndir * g.vh * nfields + 127) / 128);
+}
+
 template <typename T>
 __device__ __forceinline__ void load_link(const cplx<T>* __restrict__ U, const Geom& g, int mu, int p, int s,
                                           cplx<T>* m) {

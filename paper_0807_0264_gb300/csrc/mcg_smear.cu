@@ -185,19 +185,14 @@ __device__ __forceinline__ void ld(const cplx<T>* U, const Geom& g, int dir, con
 
 // FP32 stout steps are bound by latency: 5 blocks of 128 per SM (96 registers; 3
 // at the 133 that the coordinate array took) and indices by Walk took the step on
-// 16^3 x 32 from 94 to 70 us (six blocks spill).  The rectangle steps keep their
+// 16^3 x 32 from 94 to 71 us (six blocks spill).  The rectangle steps keep their
 // indices: by Walk the compiler holds so many links that it spills.
 template <typename T, bool RECT>
 __global__ void __launch_bounds__(ST, sizeof(T) == 4 && !RECT ? 5 : 1) k_smear_step(const cplx<T>* __restrict__ Uin, cplx<T>* __restrict__ Uout, Geom g,
                                                    int nfields, T rho, T cp, T cr) {
-    const long long n = 8LL * g.vh * nfields;
-    const long long id = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (id >= n) return;
-    const int f = (int)(id / (8LL * g.vh));
-    int r = (int)(id - (long long)f * 8 * g.vh);
-    const int mu = r / (2 * g.vh);
-    r -= mu * 2 * g.vh;
-    const int p = r / g.vh, s = r - p * g.vh;
+    LinkItem it;
+    if (!link_item<!RECT>(g, 4, nfields, it)) return;
+    const int f = it.f, mu = it.kind, p = it.p, s = it.s;
     const cplx<T>* U = Uin + (size_t)f * link_elems(g);
     int c[4];
     eo_coords(g, p, s, c);
@@ -349,25 +344,17 @@ int run_smear(const void* Uin, void* Uout, int prec, const Geom& g, int nfields,
     }
     const double cp = (5.0 - 2.0 * eps) / 3.0, cr = -(1.0 - eps) / 12.0;
     const bool rect = cr != 0.0;
-    const long long nthreads = 8LL * g.vh * nfields;
-    const int nb = (int)((nthreads + ST - 1) / ST);
+    static_assert(ST == 128, "link_item");
+    const unsigned nb = link_blocks(!rect, g, 4, nfields);
     const void* src = Uin;
     for (int k = 0; k < n; ++k) {
         void* dst = ((n - 1 - k) % 2 == 0) ? Uout : tmp;
         if (prec == MCG_F64) {
-            if (rect)
-                k_smear_step<double, true><<<nb, ST, 0, st>>>((const cplx<double>*)src, (cplx<double>*)dst, g, nfields,
-                                                              rho, cp, cr);
-            else
-                k_smear_step<double, false><<<nb, ST, 0, st>>>((const cplx<double>*)src, (cplx<double>*)dst, g,
-                                                               nfields, rho, cp, cr);
+            (rect ? k_smear_step<double, true> : k_smear_step<double, false>)<<<nb, ST, 0, st>>>(
+                (const cplx<double>*)src, (cplx<double>*)dst, g, nfields, rho, cp, cr);
         } else {
-            if (rect)
-                k_smear_step<float, true><<<nb, ST, 0, st>>>((const cplx<float>*)src, (cplx<float>*)dst, g, nfields,
-                                                             (float)rho, (float)cp, (float)cr);
-            else
-                k_smear_step<float, false><<<nb, ST, 0, st>>>((const cplx<float>*)src, (cplx<float>*)dst, g, nfields,
-                                                              (float)rho, (float)cp, (float)cr);
+            (rect ? k_smear_step<float, true> : k_smear_step<float, false>)<<<nb, ST, 0, st>>>(
+                (const cplx<float>*)src, (cplx<float>*)dst, g, nfields, (float)rho, (float)cp, (float)cr);
         }
         MCG_CK(cudaGetLastError());
         note_launches(1);

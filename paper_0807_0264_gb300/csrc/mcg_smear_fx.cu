@@ -24,7 +24,7 @@ namespace mcg {
 // (Storing the other two corners of a plaquette as well would make 38, for a
 // third more memory.)  12 or 36 matrices per site: 1 728 or 5 184 bytes.
 // Measured, ms per step with this pass, without and with the products: stout on
-// 20^3 x 40 0.93 and 0.89, on 16^4 0.198 and 0.191; over-improved on
+// 20^3 x 40 0.93 and 0.89 (0.81 tiled), on 16^4 0.198 and 0.191; over-improved on
 // 12 x 10 x 14 x 22 0.63 and 0.37.
 // ---------------------------------------------------------------------------
 template <bool RECT>
@@ -122,17 +122,14 @@ __device__ __forceinline__ void fx_staple_sum_shared(const int4* __restrict__ U,
     }
 }
 
-// the first pass: thread per (field, pair, parity, site)
+// the first pass: thread per (field, site, parity, pair)
 template <bool RECT>
 __global__ void __launch_bounds__(128, 3) k_smear_products_fx(const int4* __restrict__ Uin, int4* __restrict__ Aux,
                                                               Geom g, int nfields) {
-    const long long id = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (id >= 24LL * g.vh * nfields) return;
-    const int f = (int)(id / (24LL * g.vh));
-    int r = (int)(id - (long long)f * 24 * g.vh);
-    const int pair = r / (2 * g.vh), da = pair / 3, pb = pair - 3 * da, db = pb < da ? pb : pb + 1;
-    r -= pair * 2 * g.vh;
-    const int p = r / g.vh, s = r - p * g.vh;
+    LinkItem it;
+    if (!link_item<!RECT>(g, 12, nfields, it)) return;
+    const int f = it.f, p = it.p, s = it.s, pair = it.kind;
+    const int da = pair / 3, pb = pair - 3 * da, db = pb < da ? pb : pb + 1;
     const size_t vh = (size_t)g.vh;
     const int4* U = Uin + (size_t)f * link_elems(g);
     int4* out = Aux + (size_t)f * (kFxAux<RECT> / 4) * link_elems(g) + fx_aux_idx(g, pair, p, s);
@@ -203,7 +200,7 @@ __device__ __forceinline__ void fx_exp(const fx (&d)[3], const cfx (&x)[3], cons
 // One thread per link, old field in, new field out (fixed point, or FP64 after
 // the last step).
 // Bound by the integer multiplier.  Measured on 20^3 x 40, first pass included:
-// 0.89 ms per stout step (the FP64 kernel: 4.88 ms, FP64 pipe 93 % busy);
+// 0.81 ms per stout step (the FP64 kernel: 4.88 ms, FP64 pipe 93 % busy);
 // over-improved steps on 12 x 10 x 14 x 22: 0.37 ms (2.70 ms).  3 blocks of 128
 // per SM: 2 blocks take 12 %, 4 (spilling) 4 % longer.  Deviation from a 128-bit reference (4^4, ten
 // stout steps): 8.5e-17 rms, the FP64 kernel's 2.2e-16.
@@ -211,14 +208,25 @@ template <bool RECT, bool SHARED, bool OUT64>
 __global__ void __launch_bounds__(128, 3) k_smear_step_fx(const int4* __restrict__ Uin, const int4* __restrict__ Aux,
                                                           int4* __restrict__ Uout, Geom g, int nfields,
                                                           const __grid_constant__ FxSmear P) {
-    const long long n = 8LL * g.vh * nfields;
-    const long long id = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (id >= n) return;
-    const int f = (int)(id / (8LL * g.vh));
-    int r = (int)(id - (long long)f * 8 * g.vh);
-    const int mu = r / (2 * g.vh);
-    r -= mu * 2 * g.vh;
-    const int p = r / g.vh, s = r - p * g.vh;
+    int f, mu, p, s;
+    if (RECT) {  // link_item<false>, which the step took 0.8 % longer with
+        const long long n = 8LL * g.vh * nfields;
+        const long long id = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+        if (id >= n) return;
+        f = (int)(id / (8LL * g.vh));
+        int r = (int)(id - (long long)f * 8 * g.vh);
+        mu = r / (2 * g.vh);
+        r -= mu * 2 * g.vh;
+        p = r / g.vh;
+        s = r - p * g.vh;
+    } else {
+        LinkItem it;
+        if (!link_item<true>(g, 4, nfields, it)) return;
+        f = it.f;
+        mu = it.kind;
+        p = it.p;
+        s = it.s;
+    }
     const int4* U = Uin + (size_t)f * link_elems(g);
     int c[4];
     eo_coords(g, p, s, c);
@@ -338,11 +346,11 @@ int run_smear_fx(const void* Uin, void* Uout, const Geom& g, int nfields, double
             int4* dst = (int4*)(last ? Uout : buf(k + 1)) + off;
             if (aux) {
                 (rect ? k_smear_products_fx<true> : k_smear_products_fx<false>)
-                    <<<(unsigned)((24LL * g.vh * nf + 127) / 128), 128, 0, st>>>(src, aux, g, nf);
+                    <<<link_blocks(!rect, g, 12, nf), 128, 0, st>>>(src, aux, g, nf);
                 note_launches(1);
             }
             const auto step = step_kernel(rect, aux != nullptr, last);
-            step<<<(unsigned)((8LL * g.vh * nf + 127) / 128), 128, 0, st>>>(src, aux, dst, g, nf, P);
+            step<<<link_blocks(!rect, g, 4, nf), 128, 0, st>>>(src, aux, dst, g, nf, P);
             note_launches(1);
         }
     }
