@@ -1,7 +1,7 @@
 // Field kernels in fixed-point arithmetic (mcg_fx.cuh): gauge transforms of FP64
 // fields, the mixed-precision hand-off and the plaquette.  Fields of these entry
-// points are not always validated: a thread that meets a matrix that is not
-// near-unitary does its link or plaquette in FP64.
+// points are not always validated: a thread that meets a matrix with an entry or a
+// row norm out of range does its link or plaquette in FP64.
 //
 // A transformed field that later sweeps round to FP32 keeps the FP64 kernels of
 // mcg_field.cu: one entry rounded the other way moved the links of an unfixed
@@ -165,6 +165,10 @@ __device__ __noinline__ double plaquette_f64(const V* a, const V* b, const V* c,
 // sites per thread made four full waves and a nearly empty one on 20^3 x 40.
 // Measured, us, with whole sites and so (2^4, 8^4, 16^4, 16^3 x 32, 20^3 x 40): 36
 // 52 89 163 361 and 29 31 87 148 349 (the FP64 kernel 917 on the last).
+// Bounds, for any matrices that pass the row test (not only unitary ones): rows of
+// norm 1.025 give rows of X and Y of norm up to sqrt(3) 1.025^2 = 1.82, so a row's
+// share of the trace is below 3.4 and is widened before the next one's (the trace
+// itself may be 9.9, more than one accumulator holds).
 template <typename T>
 __global__ void __launch_bounds__(256, 2) k_plaquette_fx(const void* Uall, Geom g, int bpf,
                                                          double* __restrict__ partial) {
@@ -174,7 +178,7 @@ __global__ void __launch_bounds__(256, 2) k_plaquette_fx(const void* Uall, Geom 
     const V* U = reinterpret_cast<const V*>(Uall) + (size_t)f * link_elems(g);
     const size_t vh = (size_t)g.vh;
     double slow = 0.0;
-    long long acc = 0;  // units of 2^-57: at most 3 * 3.2
+    long long acc = 0;  // units of 2^-57: at most 3 * 9.9
     if (s2 < 2 * g.vh) {
         const int p = s2 / g.vh, s = s2 - p * g.vh;
         int c[4];
@@ -191,7 +195,7 @@ __global__ void __launch_bounds__(256, 2) k_plaquette_fx(const void* Uall, Geom 
                 cfx b[9], m[9];
                 bool bad = fx_load_matrix(ub, 3 * vh, vh, b);
                 bad = fx_load_matrix(uc, 3 * vh, vh, m) || bad;
-                facc t = facc_zero();
+                long long tr = 0;
 #pragma unroll 1
                 for (int i = 0; i < 3; ++i) {
                     cfx ra[3], rd[3], x[3], y[3];
@@ -213,16 +217,18 @@ __global__ void __launch_bounds__(256, 2) k_plaquette_fx(const void* Uall, Geom 
                           !(fabsf(nd * 0x1p-56f - 1.f) < 0.05f);
                     m3fx_row<false>(ra, b, x);
                     m3fx_row<false>(rd, m, y);
+                    facc t = facc_zero();
 #pragma unroll
                     for (int k = 0; k < 3; ++k) {
                         fx_mac(t, x[k].re, y[k].re);
                         fx_mac(t, x[k].im, y[k].im);
                     }
+                    tr += facc_get(t) >> 3;
                 }
                 if (bad)
                     slow += plaquette_f64(ua, ub, uc, ud, vh);
                 else
-                    acc += facc_get(t) >> 3;
+                    acc += tr;
             }
         }
     }

@@ -1,0 +1,40 @@
+"""FP64 entry points at the limits of their fixed-point kernels: links that are not unitary though their rows are
+of unit norm."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_0807_0264_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+
+def _pack(mcg, Us, dims):
+    return mcg.mcg_pack_links(torch.from_numpy(np.ascontiguousarray(np.stack(Us))).cuda(), dims)
+
+
+def _unit_rows(dims, diagonal, scale=1.0):
+    """Every link the all-ones matrix plus `diagonal` times the identity, its rows normalised to `scale`."""
+    m = np.ones((3, 3)) + diagonal * np.eye(3)
+    m *= scale / np.linalg.norm(m[0])
+    return np.broadcast_to(m.astype(complex), (int(np.prod(dims)), 4, 3, 3)).copy()
+
+
+# rows of norm 1 that are not orthogonal: a plaquette of 9, beyond the 8 that one sum of the fixed point holds (row norms
+# to 1.02 pass the kernel's test; the last case fills the low halves too).  ~30 roundings of 1.1e-16 relative to 9 / 3
+@pytest.mark.parametrize("diagonal,scale", [(0.0, 1.0), (0.1, 1.0), (0.2, 1.0), (-0.5, 1.0), (0.0, 1.02), (0.0, 1.0199999)])
+def test_plaquette_of_rows_that_are_not_orthogonal(diagonal, scale):
+    from paper_0807_0264_gb300 import mcg
+
+    dims = (4, 2, 6, 4)
+    U = _unit_rows(dims, diagonal, scale)
+    ref = oracle.plaquette(dims, U)
+    Ud = _pack(mcg, [U, U], dims)
+    out = torch.empty(2, dtype=torch.float64, device="cuda")
+    assert np.abs(np.array(mcg.mcg_plaquette(Ud, dims)) - ref).max() < 2e-14
+    assert np.abs(mcg.mcg_plaquette_static(Ud, dims, out).cpu().numpy() - ref).max() < 2e-14
+    U32 = mcg.mcg_convert(Ud, mcg.F32)
+    ref32 = oracle.plaquette(dims, mcg.mcg_unpack_links(U32, dims)[0].cpu().numpy())
+    assert np.abs(np.array(mcg.mcg_plaquette(U32, dims)) - ref32).max() < 2e-14
