@@ -233,7 +233,12 @@ MCG_HD bool m3fx_reunitarise(cfx* m) {
 // ---- loads of FP64 and FP32 matrices ---------------------------------------------
 // Matrices the fixed-point kernels do not take (callers' unvalidated fields): an
 // entry above 1.03 in magnitude or not finite, or a row whose squared norm is
-// off 1 by 5 % (tiny rows would lose relative precision).
+// off 1 by 5 % (tiny rows would lose relative precision).  Unit rows need not be
+// orthogonal: a matrix that passes has a spectral norm of up to 1.78.  Kernels
+// whose sums need more than that allows take fx_bad_gram (fx_load_unitary) as
+// well: squared row norms within 2 % of 1 and row inner products of components
+// below 1 %, which bounds the spectral norm by 1.024 (the Gram matrix less 1 has
+// a norm below 0.02 + 2 sqrt(2) 0.01).
 __device__ __forceinline__ unsigned fx_magnitude(double d) { return __double2hiint(d) & 0x7fffffff; }
 __device__ __forceinline__ unsigned fx_magnitude(float f) {  // as the high word of the same double, roughly
     return ((__float_as_uint(f) & 0x7fffffff) >> 3) + 0x38000000u;
@@ -258,7 +263,26 @@ __device__ __forceinline__ bool fx_bad_rows(const cfx* m) {
     }
     return bad;
 }
-// entry (r, k) at src[r sr + k sc] to m; true: not near-unitary
+__device__ __forceinline__ bool fx_bad_gram(const cfx* m) {
+    bool bad = false;
+#pragma unroll
+    for (int r = 0; r < 3; ++r)
+#pragma unroll
+        for (int q = r; q < 3; ++q) {
+            float re = 0.f, im = 0.f;  // conj(row r) . row q, unit 2^-56
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                const float ax = (float)m[3 * r + k].re.h, ay = (float)m[3 * r + k].im.h;
+                const float bx = (float)m[3 * q + k].re.h, by = (float)m[3 * q + k].im.h;
+                re = fmaf(ax, bx, fmaf(ay, by, re));
+                im = fmaf(ax, by, fmaf(-ay, bx, im));
+            }
+            bad = bad || (q == r ? !(fabsf(re * 0x1p-56f - 1.f) < 0.02f)
+                                 : !(fmaxf(fabsf(re), fabsf(im)) * 0x1p-56f < 0.01f));
+        }
+    return bad;
+}
+// entry (r, k) at src[r sr + k sc] to m; true: an entry or a row norm out of range
 template <typename C>
 __device__ __forceinline__ bool fx_load_matrix(const C* __restrict__ src, size_t sr, size_t sc, cfx* m) {
     unsigned big = 0;
@@ -273,9 +297,14 @@ __device__ __forceinline__ bool fx_load_matrix(const C* __restrict__ src, size_t
         }
     return big > kFxMagnitude || fx_bad_rows(m);
 }
+// the same; true: not near-unitary
+__device__ __forceinline__ bool fx_load_unitary(const double2* __restrict__ src, size_t sr, size_t sc, cfx* m) {
+    const bool bad = fx_load_matrix(src, sr, sc, m);
+    return fx_bad_gram(m) || bad;
+}
 __device__ __forceinline__ bool fx_bad_matrix(const double2* src, size_t sr, size_t sc) {
     cfx m[9];
-    return fx_load_matrix(src, sr, sc, m);
+    return fx_load_unitary(src, sr, sc, m);
 }
 // X 2^-60 rounded to FP32 (ties away from zero)
 __device__ __forceinline__ float fx_single(long long X) {

@@ -50,7 +50,7 @@ __global__ void __launch_bounds__(128) k_links_to_fx(const double2* __restrict__
     if (id >= nmat) return;
     const size_t o = (size_t)(id / (long long)vh) * 9 * vh + (size_t)(id % (long long)vh);
     cfx m[9];
-    if (fx_load_matrix(src + o, 3 * vh, vh, m)) atomicAdd(bad, 1u);
+    if (fx_load_unitary(src + o, 3 * vh, vh, m)) atomicAdd(bad, 1u);
 #pragma unroll
     for (int e = 0; e < 9; ++e) dst[o + e * vh] = fx_pack(m[e]);
 }
@@ -344,7 +344,7 @@ __device__ __forceinline__ size_t link_at(const Geom& g, const int c[4], int dir
 // adjoint where the factor is not daggered), times the staple's weight.  One
 // rolled product body over the table of paths, as in the staple sum.  Matrices Y
 // are shifted to the largest exponent of all that the link meets.  Their entries
-// are at most 2.1 there, so the 18 plaquette terms are summed 3 bits lower and
+// are at most 2.5 there, so the 18 plaquette terms are summed 3 bits lower and
 // weighted at the end; with rectangles (90 more terms) each term is weighted
 // before it is added, 1 bit lower (18 |wr| + 6 |wp| <= 1: the sums stay below 8).
 // In place: D's entries are replaced by the FP64 gradient of the same link.

@@ -91,7 +91,8 @@ __device__ __forceinline__ long long fx_abs2(cfx a) {
 // instruction fetch out of the way; a daggered factor is a transposed read; with
 // a second body for it the stout step took 12 % longer).  Rectangles first, then
 // (weighted) plaquettes: one sum in registers.  Links have entries and row norms
-// at most 1 (a few percent more for unvalidated ones), so has every path; the
+// at most 1 (spectral norms of 1.024 for unvalidated ones, fx_bad_gram, and 1.13
+// for a path of five), so has every path; the
 // plaquette sum of six paths stays below 8, the sum of 18 rectangles is kept in
 // units of 8.
 template <bool RECT>

@@ -302,8 +302,8 @@ __device__ __forceinline__ long long fx_site_sum(facc v) {
 // of Omega(x) per thread stays in registers.
 // Shared memory: 1152 / TPS bytes per thread, entry-major.
 // CHECK (callers' fields that were not validated): a site whose matrices are
-// not near-unitary (a row norm off 1 by 2.5 %, or not finite) is left alone and
-// counted in bt.bad.
+// not near-unitary (fx_bad_gram, or not finite) is left alone and counted in
+// bt.bad.
 // Bound by issue and the integer multiplier (52 % of the issue slots, of them a
 // third multiply-adds), for small lattices by the latency of the three solves.
 // Measured on 20^3 x 40: 285 us per half-sweep near a maximum (the FP64 kernel

@@ -38,3 +38,23 @@ def test_plaquette_of_rows_that_are_not_orthogonal(diagonal, scale):
     U32 = mcg.mcg_convert(Ud, mcg.F32)
     ref32 = oracle.plaquette(dims, mcg.mcg_unpack_links(U32, dims)[0].cpu().numpy())
     assert np.abs(np.array(mcg.mcg_plaquette(U32, dims)) - ref32).max() < 2e-14
+
+
+# the reverse step of such links (staple sums of 10 before the weight), and of links just inside the test (None: inner
+# products of rows below 0.01, squared row norms 1.014): the bar of the FP64 kernel, 1e-11 of the gradient
+@pytest.mark.parametrize("diagonal", [0.0, 0.1, 1.0, None])
+@pytest.mark.parametrize("eps,rho", [(1.0, 1 / 6), (-0.25, 0.06)])
+def test_smear_backward_of_rows_that_are_not_orthogonal(diagonal, eps, rho):
+    from paper_0807_0264_gb300 import mcg
+
+    dims, rng = (4, 2, 6, 4), np.random.default_rng(3)
+    if diagonal is None:
+        U = synth.make_field(dims, 0.7, 3)
+        U[..., 0, :] += 0.009 * U[..., 1, :]
+        U *= 1.007 / np.linalg.norm(U, axis=-1, keepdims=True)
+    else:
+        U = _unit_rows(dims, diagonal)
+    G = rng.standard_normal(U.shape) + 1j * rng.standard_normal(U.shape)
+    got = mcg.mcg_smear_backward_step(_pack(mcg, [U], dims), _pack(mcg, [G], dims), dims, rho, eps)
+    ref = oracle.smear_step_backward(dims, U, G, rho, eps)
+    assert np.abs(mcg.mcg_unpack_links(got, dims)[0].cpu().numpy() - ref).max() < 1e-11 * np.abs(ref).max()
