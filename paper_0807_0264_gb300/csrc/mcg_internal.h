@@ -106,6 +106,13 @@ struct FieldState {
     double ring[kRing];  // R after sweep k stored at k % kRing
 };
 
+// Sites of a half-sweep that the fixed-point kernel left to the FP64 kernel: their
+// number, and a mark per site of the parity (written for every site swept).
+struct LeftSites {
+    unsigned count;
+    unsigned char site[1];  // vh of them
+};
+
 struct SweepBatch {
     const FieldDesc* desc;
     int nf;
@@ -122,7 +129,7 @@ struct SweepBatch {
     int solve32;   // FP64 sweeps: local problem built and solved in FP32
     int spb = 0;              // sites per block
     int tps = 0;              // threads per site of the fixed-point FP64 sweep (0: another kernel)
-    unsigned* bad = nullptr;  // unvalidated fields: sites left to the FP64 kernel
+    LeftSites* left = nullptr;  // one unvalidated field: the sites left to the FP64 kernel
 };
 
 // Haar-random SU(3) transforms (FP64 gauge layout, the same in each of the
@@ -226,8 +233,8 @@ int launch_identity_df(void* hi, void* lo, const Geom& g, int nfields, cudaStrea
 // The exact FP64 half-sweep in fixed point (mcg_sweep_fx.cu): threads per site
 // and per block for a number of sites of one parity, shared-memory set-up on
 // the current device, launch (nblocks of shape.nt / shape.tps sites).  With
-// bt.bad set (shape {2, 128}) sites with matrices that are not near-unitary
-// are left alone and counted there.
+// bt.left set (shape {2, 128}, one field) sites with matrices that are not
+// near-unitary are left alone and marked there.
 struct FxShape {
     int tps, nt;
 };

@@ -31,7 +31,6 @@
 #include <vector>
 
 #include "mcg_common.cuh"
-#include "mcg_fx.cuh"
 #include "mcg_internal.h"
 #include "mcg_sweep.cuh"
 
@@ -209,11 +208,11 @@ __device__ __forceinline__ int subgroup_step(L& lk, const int P, const int Q, co
 // threads (5 blocks per SM), 83 KB for 128 FP32 or 64 FP64 threads (2 per SM).
 // S32: the local problem in FP32.  Otherwise the exact local problem in FP64:
 // fields that later sweeps round to FP32 (see mcg_field_fx.cu), and, with
-// bt.bad set, only the sites that the fixed-point sweep of an unvalidated field
-// left alone (bt.bad counts them, zero for any SU(3) field), by the same test.
+// bt.left set, only the sites that the fixed-point sweep of an unvalidated field
+// left alone and marked there (none for any SU(3) field).
 template <typename T, bool ACC, int NT, bool S32>
 __global__ void __launch_bounds__(NT, 2) k_halfsweep(SweepBatch bt, int parity) {
-    if (!S32 && bt.bad && *bt.bad == 0) return;
+    if (!S32 && bt.left && bt.left->count == 0) return;
     const int f = field_of_block(bt.desc, bt.nf, blockIdx.x);
     if (ACC) reunit_due(bt, f);
     if (bt.state[f].done) return;  // block-uniform
@@ -235,22 +234,11 @@ __global__ void __launch_bounds__(NT, 2) k_halfsweep(SweepBatch bt, int parity) 
 
     double rsum = 0.0;
     int fb = 0;
-    int sb[4] = {0, 0, 0, 0};
+    if (!S32 && active && bt.left) active = bt.left->site[s] != 0;
     if (active) {
+        int sb[4];
 #pragma unroll
         for (int mu = 0; mu < 4; ++mu) sb[mu] = eo_neighbor(g, c, mu, -1);
-        if (!S32 && bt.bad) {
-            const double2* Ud = reinterpret_cast<const double2*>(fd.U);
-            const size_t vh = (size_t)g.vh;
-            bool bad = fx_bad_matrix(reinterpret_cast<const double2*>(fd.G) + gidx(g, parity, 0, s), 3 * vh, vh);
-#pragma unroll 1
-            for (int mu = 0; mu < 4; ++mu)
-                bad = bad || fx_bad_matrix(Ud + lidx(g, mu, parity, 0, s), 3 * vh, vh) ||
-                      fx_bad_matrix(Ud + lidx(g, mu, parity ^ 1, 0, sb[mu]), vh, 3 * vh);
-            active = bad;
-        }
-    }
-    if (active) {
         // stage the 8 links and Omega in shared memory without passing
         // through registers
 #pragma unroll
@@ -819,7 +807,7 @@ static int prepare_unvalidated() {
 }
 constexpr int kUnvalidatedSites = 64, kUnvalidatedPartials = 6;  // per block
 static int launch_unvalidated(bool acc, SweepBatch bt, int parity, int nblocks, cudaStream_t st) {
-    MCG_CK(cudaMemsetAsync(bt.bad, 0, sizeof(unsigned), st));
+    MCG_CK(cudaMemsetAsync(bt.left, 0, sizeof(unsigned), st));  // the count; the first kernel writes its sites
     double* rest = bt.partial + (size_t)nblocks * 4;
     if (acc) MCG_CK(cudaMemsetAsync(rest, 0, sizeof(double) * 2 * nblocks, st));
     launch_halfsweep_fx(FxShape{2, 128}, acc, bt, parity, nblocks, st);
@@ -901,7 +889,7 @@ struct GraphKey {
         add(b.omega);
         add(b.solve32);
         add(b.tps);
-        add(b.bad);
+        add(b.left);
     }
 };
 
@@ -1294,7 +1282,7 @@ int time_halfsweep(void* U, void* G, const Geom& g, int parity, int nreps, int f
     double* d_partial =
         (double*)scratch_device("time.partial", sizeof(double) * fd.nblk * (F64 ? kUnvalidatedPartials : NT / 32), &rc);
     if (rc) return rc;
-    unsigned* d_bad = (unsigned*)scratch_device("time.bad", sizeof(unsigned), &rc);
+    LeftSites* d_left = (LeftSites*)scratch_device("time.left", sizeof(unsigned) + (size_t)g.vh, &rc);
     if (rc) return rc;
     void* flush = nullptr;
     const size_t flush_bytes = (size_t)256 << 20;
@@ -1311,7 +1299,7 @@ int time_halfsweep(void* U, void* G, const Geom& g, int parity, int nreps, int f
     bt.state = d_state;
     bt.partial = d_partial;
     bt.ppb = NT / 32;
-    bt.bad = d_bad;
+    bt.left = d_left;
     bt.R_hist = nullptr;
     bt.hist_len = 0;
     bt.tol = 0;
@@ -1409,7 +1397,7 @@ int run_halfsweep_slab(void* U, void* G, const Geom& g, int parity, int t_lo, in
     if (rc) return rc;
     double* d_partial = (double*)scratch_device("slab.partial", sizeof(double) * fd.nblk * kUnvalidatedPartials, &rc);
     if (rc) return rc;
-    unsigned* d_bad = (unsigned*)scratch_device("slab.bad", sizeof(unsigned), &rc);
+    LeftSites* d_left = (LeftSites*)scratch_device("slab.left", sizeof(unsigned) + (size_t)g.vh, &rc);
     if (rc) return rc;
     double* d_R = (double*)scratch_device("slab.R", sizeof(double), &rc);
     if (rc) return rc;
@@ -1426,7 +1414,7 @@ int run_halfsweep_slab(void* U, void* G, const Geom& g, int parity, int t_lo, in
     bt.state = d_state;
     bt.partial = d_partial;
     bt.ppb = 4;
-    bt.bad = d_bad;
+    bt.left = d_left;
     bt.R_hist = nullptr;
     bt.hist_len = 0;
     bt.tol = 0;

@@ -302,8 +302,9 @@ __device__ __forceinline__ long long fx_site_sum(facc v) {
 // of Omega(x) per thread stays in registers.
 // Shared memory: 1152 / TPS bytes per thread, entry-major.
 // CHECK (callers' fields that were not validated): a site whose matrices are
-// not near-unitary (fx_bad_gram, or not finite) is left alone and counted in
-// bt.bad.
+// not near-unitary (fx_bad_gram, or not finite) is left alone and marked in
+// bt.left, which the FP64 kernel reads (by then the moved links' rows may have
+// other norms).
 // Bound by issue and the integer multiplier (52 % of the issue slots, of them a
 // third multiply-adds), for small lattices by the latency of the three solves.
 // Measured on 20^3 x 40: 285 us per half-sweep near a maximum (the FP64 kernel
@@ -380,7 +381,10 @@ __global__ void __launch_bounds__(NT, MINB) k_halfsweep_fx(SweepBatch bt, int pa
         int b = bad;
 #pragma unroll
         for (int o = SPW; o < 32; o *= 2) b |= __shfl_xor_sync(0xffffffffu, b, o);
-        if (b && active && q == 0) atomicAdd(bt.bad, 1u);
+        if (active && q == 0) {
+            bt.left->site[s] = b != 0;
+            if (b) atomicAdd(&bt.left->count, 1u);
+        }
         active = active && !b;
     }
 
@@ -558,7 +562,7 @@ static void launch_shape(bool acc, const SweepBatch& bt, int parity, int nblocks
         k_halfsweep_fx<TPS, NT, MINB, false, false><<<nblocks, NT, smem, st>>>(bt, parity);
 }
 void launch_halfsweep_fx(FxShape sh, bool acc, const SweepBatch& bt, int parity, int nblocks, cudaStream_t st) {
-    if (bt.bad) {  // unvalidated fields: shape (2, 128)
+    if (bt.left) {  // unvalidated fields: shape (2, 128)
         const size_t smem = 1152 / 2 * 128;
         if (acc)
             k_halfsweep_fx<2, 128, 3, true, true><<<nblocks, 128, smem, st>>>(bt, parity);

@@ -58,3 +58,27 @@ def test_smear_backward_of_rows_that_are_not_orthogonal(diagonal, eps, rho):
     got = mcg.mcg_smear_backward_step(_pack(mcg, [U], dims), _pack(mcg, [G], dims), dims, rho, eps)
     ref = oracle.smear_step_backward(dims, U, G, rho, eps)
     assert np.abs(mcg.mcg_unpack_links(got, dims)[0].cpu().numpy() - ref).max() < 1e-11 * np.abs(ref).max()
+
+
+# a half-sweep of links a few percent or less off unitarity, with one link far off: a site moves once, whatever the
+# norms of its rows after the move, and counts once in R.  The FP64 sweep's bar of 1e-11 per link near a maximum,
+# 9 times that for the link scaled by 3
+@pytest.mark.parametrize("overlap,scale", [(0.1, 1.0), (0.1, 1.02), (0.009, 1.007), (0.007, 0.994)])
+def test_halfsweep_of_links_off_unitarity(overlap, scale):
+    from paper_0807_0264_gb300 import mcg
+
+    dims = (4, 6, 4, 6)
+    U, G = synth.make_field(dims, 0.4, 5, gauge=False), synth.identity_gauge(dims)
+    U[..., 0, :] += overlap * U[..., 1, :]
+    U *= scale / np.linalg.norm(U, axis=-1, keepdims=True)
+    U[7, 2] *= 3.0
+    Ud, Gd = _pack(mcg, [U], dims), mcg.mcg_pack_gauge(torch.from_numpy(G).unsqueeze(0).cuda(), dims)
+    Uo, Go = U.copy(), G.copy()
+    for sweep in range(2):
+        for parity in (0, 1):
+            R = mcg.mcg_halfsweep_slab(Ud, Gd, dims, parity, 0, dims[3], want_R=parity == 1)
+            oracle.halfsweep_slab(dims, Uo, Go, parity, 0, dims[3])
+    assert np.abs(mcg.mcg_unpack_links(Ud, dims)[0].cpu().numpy() - Uo).max() < 9e-11
+    assert np.abs(mcg.mcg_unpack_gauge(Gd, dims)[0].cpu().numpy() - Go).max() < 9e-11
+    ref = (np.abs(np.trace(Uo, axis1=-2, axis2=-1)) ** 2).sum()
+    assert abs(R - ref) < 1e-11 * ref
