@@ -860,6 +860,7 @@ int mcg_precondition_fix(void* U, void* G, int8_t* Z, const mcg_lattice* lat, co
     if (rc != MCG_OK && rc != MCG_NOT_CONVERGED) return rc;
     if (rc == MCG_NOT_CONVERGED) status = MCG_NOT_CONVERGED;
     int8_t* Zb = Z;
+    rc = 0;  // a fix that did not converge is no error here
     if (!Zb) {
         Zb = (int8_t*)scratch_device("pre.Z", 8 * (size_t)g.vh * nf, &rc);
         if (rc) return rc;
@@ -1106,6 +1107,7 @@ int mcg_precondition_levels(const void* U, void* U_out, void* G_out, int8_t* Z_o
         }
     }
     int8_t* Zb = Z_out;
+    rc = 0;  // a fix that did not converge is no error here
     if (!Zb) {
         Zb = (int8_t*)scratch_device("lev.Z", 8 * (size_t)g.vh * nlevels, &rc);
         if (rc) return rc;

@@ -1,5 +1,5 @@
 """FP64 entry points at the limits of their fixed-point kernels: links that are not unitary though their rows are
-of unit norm."""
+of unit norm, schedules and batches."""
 import numpy as np
 import pytest
 
@@ -82,3 +82,19 @@ def test_halfsweep_of_links_off_unitarity(overlap, scale):
     assert np.abs(mcg.mcg_unpack_gauge(Gd, dims)[0].cpu().numpy() - Go).max() < 9e-11
     ref = (np.abs(np.trace(Uo, axis1=-2, axis2=-1)) ** 2).sum()
     assert abs(R - ref) < 1e-11 * ref
+
+
+# a preconditioned fix that ends at its sweep cap fills its results whether or not the caller asks for the sectors
+def test_results_of_a_fix_at_its_cap_without_sectors():
+    from paper_0807_0264_gb300 import mcg
+
+    dims, prm = (4, 2, 6, 4), mcg.Params(tol=1e-12, max_sweeps=3)
+    U = _pack(mcg, [synth.make_field(dims, 1.5, 4)], dims)
+    Z = torch.empty((1, 4, 2, int(np.prod(dims)) // 2), dtype=torch.int8, device="cuda")
+    runs = [mcg.mcg_precondition_fix(U.clone(), mcg.identity_gauge(dims), dims, prm, nsmear=2, Z=z)[0] for z in (Z, None)]
+    assert runs[0] == runs[1] and runs[0]["status"] == 1 and runs[0]["sweeps_fixed"] == 3 and runs[0]["V_fixed"] > 0
+    res = (mcg.mcg_precond_result * 1)()
+    cp, ns, out, G = prm.c(), (mcg.ctypes.c_int * 1)(2), torch.empty_like(U), mcg.identity_gauge(dims)
+    rc = mcg.library().mcg_precondition_levels(U.data_ptr(), out.data_ptr(), G.data_ptr(), None, mcg.lattice(dims, 1, mcg.F64),
+                                               mcg.ctypes.byref(cp), 0.1, 1.0, ns, 1, mcg.F64, res, None)
+    assert rc == 1 and res[0].as_dict() == runs[0]
