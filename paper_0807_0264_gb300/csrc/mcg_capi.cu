@@ -481,9 +481,16 @@ static int fix_fields(const std::vector<FieldSpec>& fs, int prec, const mcg_para
             fds[f].geo = fs[f].g;
             fds[f].norm = 1.0 / (9.0 * 8.0 * fs[f].g.vh);
         }
-        rc = run_fix_phase<double>(fds, d_state, h_state, d_hist, hist_len, prm->tol, 1, 1.0, prm->reunit_every,
-                                   prm->max_sweeps, prm->check_every, fresh, st, prm->fp64_solve32 != 0, nullptr,
-                                   std::any_of(fs.begin(), fs.end(), [](const FieldSpec& f) { return f.keep_fp64; }));
+        // fields that stay in FP64 arithmetic and the others apart: which kernel a
+        // field runs does not depend on its batch
+        auto keeps = [&](int f) { return fs[f].keep_fp64 && !prm->fp64_solve32; };
+        for (int a = 0, b = 0; a < nf && !rc; a = b) {
+            while (b < nf && keeps(b) == keeps(a)) ++b;
+            rc = run_fix_phase<double>(std::vector<FieldDesc>(fds.begin() + a, fds.begin() + b), d_state + a,
+                                       h_state + a, d_hist ? d_hist + (size_t)hist_len * a : nullptr, hist_len,
+                                       prm->tol, 1, 1.0, prm->reunit_every, prm->max_sweeps, prm->check_every, fresh,
+                                       st, prm->fp64_solve32 != 0, nullptr, keeps(a));
+        }
     } else {
         // FP32 fields: compact copies in, full layout (row 2 rebuilt) out
         std::vector<FieldDesc> fds;

@@ -98,3 +98,22 @@ def test_results_of_a_fix_at_its_cap_without_sectors():
     rc = mcg.library().mcg_precondition_levels(U.data_ptr(), out.data_ptr(), G.data_ptr(), None, mcg.lattice(dims, 1, mcg.F64),
                                                mcg.ctypes.byref(cp), 0.1, 1.0, ns, 1, mcg.F64, res, None)
     assert rc == 1 and res[0].as_dict() == runs[0]
+
+
+# a level without smearing beside smeared ones, on schedules that keep some fields in FP64 arithmetic and not others:
+# the bits of the level alone
+@pytest.mark.parametrize("schedule", [dict(fp32_sweeps=60), dict(fp32_sweeps=60, fp64_df=1),
+                                      dict(fp32_sweeps=60, fp64_solve32=1), dict()])
+def test_unsmeared_level_beside_smeared_ones(schedule):
+    from paper_0807_0264_gb300 import mcg
+
+    dims = (6, 4, 4, 6)
+    prm = mcg.Params(tol=1e-9, max_sweeps=120, check_every=10, **schedule)
+    U = _pack(mcg, [synth.make_field(dims, 2.0, 4)], dims)
+    Ua, Ga, _, ra = mcg.mcg_precondition_levels(U, dims, [0], prm)
+    Ub, Gb, _, rb = mcg.mcg_precondition_levels(U, dims, [0, 2, 5], prm)
+    Uc, Gc = U.clone(), mcg.identity_gauge(dims)
+    rc = mcg.mcg_precondition_fix(Uc, Gc, dims, prm)
+    for Ux, Gx, rx in ((Ub, Gb, rb), (Uc, Gc, rc)):
+        assert torch.equal(Ux[:1], Ua) and torch.equal(Gx[:1], Ga)
+        assert rx[0]["V_fixed"] == ra[0]["V_fixed"] and rx[0]["sweeps_fixed"] == ra[0]["sweeps_fixed"]
