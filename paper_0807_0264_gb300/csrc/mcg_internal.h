@@ -118,7 +118,7 @@ struct SweepBatch {
     int nf;
     int total_blocks;
     FieldState* state;
-    double* partial;  // one per warp: ppb per block
+    double* partial;  // one per warp: ppb per block (of a fixed-point half-sweep: integers of unit 2^-50)
     int ppb;          // partials per block (threads per block / 32)
     double* R_hist;   // nf x hist_len (may be null)
     int hist_len;

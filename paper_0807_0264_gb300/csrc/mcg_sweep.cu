@@ -617,31 +617,73 @@ __global__ void __launch_bounds__(256) k_functional(SweepBatch bt) {
     warp_partial(r, bt.partial);
 }
 
+// Sum of the integer partials (units of 2^-50) of a fixed-point half-sweep, in the
+// first thread of a block of 256: exact in two words, rounded once.
+__device__ __forceinline__ double sum_partials_fx(const long long* __restrict__ part, size_t n) {
+    long long hi = 0, lo = 0;
+    for (size_t k = threadIdx.x; k < n; k += 8 * (size_t)blockDim.x) {
+        long long x[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const size_t kk = k + (size_t)j * blockDim.x;
+            x[j] = kk < n ? part[kk] : 0;
+        }
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            hi += x[j] >> 32;
+            lo += x[j] & 0xffffffffLL;
+        }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        hi += __shfl_xor_sync(0xffffffffu, hi, o);
+        lo += __shfl_xor_sync(0xffffffffu, lo, o);
+    }
+    __shared__ long long red[16];
+    if ((threadIdx.x & 31) == 0) {
+        red[threadIdx.x >> 5] = hi;
+        red[8 + (threadIdx.x >> 5)] = lo;
+    }
+    __syncthreads();
+    if (threadIdx.x != 0) return 0.0;
+    for (int k = 1; k < 8; ++k) {
+        hi += red[k];
+        lo += red[8 + k];
+    }
+    hi += lo >> 32;
+    return ((double)hi * 4294967296.0 + (double)(lo & 0xffffffffLL)) * 0x1p-50;
+}
+
 // mode 0: end of a sweep; 1: fresh start (sweep = 0); 2: continue (new phase)
 __device__ __forceinline__ void finalize_field(const SweepBatch& bt, int f, int mode) {
     FieldState* st = &bt.state[f];
     if (mode == 0 && st->done) return;
     const FieldDesc fd = bt.desc[f];
-    double v = 0.0;
     const size_t n = (size_t)fd.nblk * bt.ppb;
     const double* __restrict__ part = bt.partial + (size_t)fd.blk0 * bt.ppb;
-    // each thread adds its strided partials k, k + blockDim, ... in that
-    // order; eight are loaded before they are added (zeros past the end come
-    // after the last partial, so the sum is unchanged), which takes the
-    // dependent load latency off this kernel: it sits on the critical path of
-    // every sweep (measured: a lone-field fix 4 % faster, same bits)
-    for (size_t k = threadIdx.x; k < n; k += 8 * (size_t)blockDim.x) {
-        double x[8];
+    double R;
+    if (mode == 0 && bt.tps > 0) {
+        R = sum_partials_fx(reinterpret_cast<const long long*>(part), n);
+    } else {
+        double v = 0.0;
+        // each thread adds its strided partials k, k + blockDim, ... in that
+        // order; eight are loaded before they are added (zeros past the end come
+        // after the last partial, so the sum is unchanged), which takes the
+        // dependent load latency off this kernel: it sits on the critical path of
+        // every sweep (measured: a lone-field fix 4 % faster, same bits)
+        for (size_t k = threadIdx.x; k < n; k += 8 * (size_t)blockDim.x) {
+            double x[8];
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            const size_t kk = k + (size_t)j * blockDim.x;
-            x[j] = kk < n ? part[kk] : 0.0;
+            for (int j = 0; j < 8; ++j) {
+                const size_t kk = k + (size_t)j * blockDim.x;
+                x[j] = kk < n ? part[kk] : 0.0;
+            }
+#pragma unroll
+            for (int j = 0; j < 8; ++j) v += x[j];
         }
-#pragma unroll
-        for (int j = 0; j < 8; ++j) v += x[j];
+        __shared__ double red[8];
+        R = block_sum(v, red);
     }
-    __shared__ double red[8];
-    const double R = block_sum(v, red);
     if (threadIdx.x != 0) return;
     if (mode != 0) {
         if (mode == 1) {

@@ -474,9 +474,8 @@ __global__ void __launch_bounds__(NT, MINB) k_halfsweep_fx(SweepBatch bt, int pa
         }
     }
 
-    long long racc = 0;
+    facc tr2 = facc_zero();
     if (active) {
-        facc tr2 = facc_zero();
 #pragma unroll 1
         for (int i = 0; i < NM; ++i) {
             size_t sr, sc;
@@ -501,7 +500,6 @@ __global__ void __launch_bounds__(NT, MINB) k_halfsweep_fx(SweepBatch bt, int pa
                 fx_mac(tr2, sy, sy);
             }
         }
-        racc = facc_get(tr2);  // unit 2^-56, at most 72 (1.03)^2
 #pragma unroll
         for (int n = 0; n < NC; ++n)
             if (q + n * TPS < 3) {
@@ -512,11 +510,19 @@ __global__ void __launch_bounds__(NT, MINB) k_halfsweep_fx(SweepBatch bt, int pa
             }
     }
     if (ACC) {
-        // the warp's sites in units of 2^-50 (at most 32 76 2^50 < 2^62), widened once
-        racc >>= 6;
+        // a site's share (unit 2^-56, at most 72 (1.03)^2), cut to units of 2^-50, and
+        // the sum over the warp's sites (below 2^61), as an integer: with the integer
+        // sum of the partials R has the same bits for every number of threads per site
+        long long r = fx_site_sum<SPW>(tr2) >> 6;
 #pragma unroll
-        for (int o = 1; o < 32; o *= 2) racc += __shfl_xor_sync(0xffffffffu, racc, o);
-        if (lane == 0) bt.partial[blockIdx.x * (NT / 32) + (threadIdx.x >> 5)] = fx_double(racc) * 0x1p10;
+        for (int o = 1; o < SPW; o *= 2) r += __shfl_xor_sync(0xffffffffu, r, o);
+        const int k = blockIdx.x * (NT / 32) + (threadIdx.x >> 5);
+        if (lane == 0) {
+            if (CHECK)
+                bt.partial[k] = fx_double(r) * 0x1p10;
+            else
+                reinterpret_cast<long long*>(bt.partial)[k] = r;
+        }
     }
     {
         const int w = __reduce_add_sync(0xffffffffu, fb);

@@ -117,3 +117,26 @@ def test_unsmeared_level_beside_smeared_ones(schedule):
     for Ux, Gx, rx in ((Ub, Gb, rb), (Uc, Gc, rc)):
         assert torch.equal(Ux[:1], Ua) and torch.equal(Gx[:1], Ga)
         assert rx[0]["V_fixed"] == ra[0]["V_fixed"] and rx[0]["sweeps_fixed"] == ra[0]["sweeps_fixed"]
+
+
+# plain FP64 sweeps: links, transform, R of every sweep and the stop sweep are those of the field alone, in batches for
+# which the sweep takes 8, 4 and 2 threads per site, as chains and in one launch
+@pytest.mark.parametrize("copies", [2, 4, 10, 17])
+def test_fp64_batch_equals_the_field_alone(copies):
+    from paper_0807_0264_gb300 import mcg
+
+    dims = (8, 6, 10, 8)
+    prm = mcg.Params(tol=1e-5, max_sweeps=25, reunit_every=10, check_every=5)
+    fields = [synth.make_field(dims, 1.5, s) for s in (1, 2)]
+    alone = []
+    for U in fields:
+        Ud, Gd = _pack(mcg, [U], dims), mcg.identity_gauge(dims)
+        r = mcg.mcg_fix(Ud, Gd, dims, prm, history=True)
+        alone.append((Ud, Gd, r["R"][0], r["sweeps"][0], np.asarray(r["R_hist"]).reshape(-1)))
+    Ud, Gd = _pack(mcg, [fields[k % 2] for k in range(copies)], dims), mcg.identity_gauge(dims, copies)
+    r = mcg.mcg_fix(Ud, Gd, dims, prm, history=True)
+    hist = np.asarray(r["R_hist"]).reshape(copies, -1)
+    for k in range(copies):
+        U1, G1, R1, s1, h1 = alone[k % 2]
+        assert r["sweeps"][k] == s1 and r["R"][k] == R1 and np.array_equal(hist[k], h1)
+        assert torch.equal(Ud[k], U1[0]) and torch.equal(Gd[k], G1[0])
