@@ -898,6 +898,12 @@ def main():
     t32 = mcg.mcg_time_halfsweep(U32, G32, dims, parity=1, nreps=20, flush_l2=True)
     t32_even = mcg.mcg_time_halfsweep(U32, G32, dims, parity=0, nreps=20, flush_l2=True)
     t64 = mcg.mcg_time_halfsweep(Uc, Gc, dims, parity=1, nreps=5, flush_l2=True)
+    # the plain FP64 sweep (fixed point): sweep-graph time of a short fix of the same field
+    for _ in range(2):
+        mcg.mcg_phase_stats(reset=True)
+        mcg.mcg_fix(U_warm.clone(), mcg.identity_gauge(dims, 1, mcg.F64, dev), dims,
+                    mcg.Params(tol=-1e300, max_sweeps=10, check_every=10, reunit_every=0))
+        plain64 = mcg.mcg_phase_stats(reset=True)["f64"]
     del Uc, Gc, U32, G32
     vh = V // 2
     bytes32 = vh * (8 * 48 * 2 + 48 * 2)  # 8 links + W read and written, FP32 rows 0 and 1
@@ -927,7 +933,8 @@ def main():
                          "frac": bytes32 / ((t32 + t32_even) / 2 / 1e3) / 1e9 / peak,
                          "method": "one 20^3 x 40 field, mean of the odd and even half-sweep, L2 flushed by a "
                                    "256 MB memset before each launch"}}
-    roof["kernel_ms"] = {"fp32_odd": t32, "fp32_even": t32_even, "fp64_odd_exact_solve": t64}
+    roof["kernel_ms"] = {"fp32_odd": t32, "fp32_even": t32_even, "fp64_odd_exact_solve": t64,
+                         "fp64_fixed_point_half": plain64["ms"] * vh / max(1, plain64["site_updates"])}
     # the same kernel inside a fix (no flush: each half-sweep's 138 MB working
     # set exceeds the 129 MB L2): FP32-phase time of N2 - N1 sweeps on a copy
     # of the warm field, both half-sweeps and the end-of-sweep kernel per sweep

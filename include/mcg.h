@@ -548,10 +548,12 @@ int mcg_ascent_step(void* U, void* G, const double* grad, double alpha, const mc
  * parity 1: odd sites with the fused R reduction) on one field, over nreps
  * launches each bracketed by CUDA events on `stream`; with flush_l2 != 0 a
  * 256 MB buffer is overwritten between launches, outside the timed interval,
- * so every launch reads its links from HBM.  FP64: the sweeps are applied to
- * U and G.  FP32: the FP32 kernel works on the library's compact storage
- * (rows 0 and 1 of each matrix, row 2 implied by unitarity); U and G are
- * converted to it once, before the timed launches, and left unchanged.
+ * so every launch reads its links from HBM.  FP64: the exact half-sweep in FP64
+ * arithmetic, whose block size mcg_set_sweep_block sets (mcg_phase_stats times
+ * the sweeps of a fix, in fixed point or not); the sweeps are applied to U and
+ * G.  FP32: the FP32 kernel works on the library's compact storage (rows 0 and 1
+ * of each matrix, row 2 implied by unitarity); U and G are converted to it once,
+ * before the timed launches, and left unchanged.
  * ms_out: host float.  Synchronises.  (Instrumentation; not part of the
  * paper's method.) */
 int mcg_time_halfsweep(void* U, void* G, const mcg_lattice* lat, int parity, int nreps, int flush_l2, float* ms_out,
@@ -579,7 +581,8 @@ int mcg_plaquette_static(const void* U, double* out, const mcg_lattice* lat, cud
 /* Threads per block of the half-sweep kernel for one precision, one thread
  * per site: FP64 64 or 128, FP32 64, 128 or 256; 128 by default.  (The plain
  * FP64 sweep chooses its own shape by the number of sites; the setting applies
- * to FP64 sweeps with the FP32 local solve.)  A process-wide tuning setting
+ * to FP64 sweeps with the FP32 local solve and to those of fields that a later
+ * fix rounds to FP32.)  A process-wide tuning setting
  * (not part of the paper's method): Python's autotune_sweep_block() times the choices with
  * mcg_time_halfsweep and keeps the fastest.  Returns MCG_BAD_ARG otherwise. */
 int mcg_set_sweep_block(int precision, int threads);

@@ -1305,26 +1305,21 @@ int run_fix_phase(const std::vector<FieldDesc>& fields_in, FieldState* d_state, 
 template <typename T>
 int time_halfsweep(void* U, void* G, const Geom& g, int parity, int nreps, int flush_l2, float* ms,
                    cudaStream_t stream) {
-    // FP64: the exact half-sweep (the caller's field was not validated)
-    constexpr bool F64 = sizeof(T) == 8;
-    const int NT = F64 ? 128 : sweep_block(MCG_F32);
-    const int spb = F64 ? kUnvalidatedSites : NT;
+    // FP64: the kernel that reads the block setting, which the tuner sets by this
+    const int NT = sweep_block(sizeof(T) == 8 ? MCG_F64 : MCG_F32);
     int rc = 0;
     FieldDesc fd;
     fd.U = U;
     fd.G = G;
     fd.geo = g;
     fd.blk0 = 0;
-    fd.nblk = (g.vh + spb - 1) / spb;
+    fd.nblk = (g.vh + NT - 1) / NT;
     fd.norm = 1.0 / (9.0 * 8.0 * g.vh);
     FieldDesc* d_desc = (FieldDesc*)scratch_device("time.desc", sizeof(FieldDesc), &rc);
     if (rc) return rc;
     FieldState* d_state = (FieldState*)scratch_device("time.state", sizeof(FieldState), &rc);
     if (rc) return rc;
-    double* d_partial =
-        (double*)scratch_device("time.partial", sizeof(double) * fd.nblk * (F64 ? kUnvalidatedPartials : NT / 32), &rc);
-    if (rc) return rc;
-    LeftSites* d_left = (LeftSites*)scratch_device("time.left", sizeof(unsigned) + (size_t)g.vh, &rc);
+    double* d_partial = (double*)scratch_device("time.partial", sizeof(double) * fd.nblk * (NT / 32), &rc);
     if (rc) return rc;
     void* flush = nullptr;
     const size_t flush_bytes = (size_t)256 << 20;
@@ -1341,7 +1336,6 @@ int time_halfsweep(void* U, void* G, const Geom& g, int parity, int nreps, int f
     bt.state = d_state;
     bt.partial = d_partial;
     bt.ppb = NT / 32;
-    bt.left = d_left;
     bt.R_hist = nullptr;
     bt.hist_len = 0;
     bt.tol = 0;
@@ -1349,7 +1343,7 @@ int time_halfsweep(void* U, void* G, const Geom& g, int parity, int nreps, int f
     bt.reunit_every = 0;
     bt.omega = 1.0;
     bt.solve32 = 0;
-    if ((rc = F64 ? prepare_unvalidated() : prepare_halfsweep<T>(NT))) return rc;
+    if ((rc = prepare_halfsweep<T>(NT))) return rc;
     cudaEvent_t e0, e1;
     MCG_CK(cudaEventCreate(&e0));
     MCG_CK(cudaEventCreate(&e1));
@@ -1359,10 +1353,7 @@ int time_halfsweep(void* U, void* G, const Geom& g, int parity, int nreps, int f
             cudaMemsetAsync(flush, r & 0xff, flush_bytes, stream);
         }
         cudaEventRecord(e0, stream);
-        if (F64)
-            launch_unvalidated(parity != 0, bt, parity, fd.nblk, stream);
-        else
-            launch_halfsweep<T>(NT, parity != 0, bt, parity, fd.nblk, stream);
+        launch_halfsweep<T>(NT, parity != 0, bt, parity, fd.nblk, stream);
         cudaEventRecord(e1, stream);
         cudaError_t ce = cudaEventSynchronize(e1);
         if (ce != cudaSuccess) {
@@ -1374,7 +1365,7 @@ int time_halfsweep(void* U, void* G, const Geom& g, int parity, int nreps, int f
         cudaEventElapsedTime(&t, e0, e1);
         total += t;
     }
-    if (!F64) note_launches(nreps);
+    note_launches(nreps);
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     MCG_CK(cudaGetLastError());

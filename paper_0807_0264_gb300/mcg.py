@@ -539,7 +539,8 @@ def mcg_precondition_levels(U: torch.Tensor, dims, nsmear, params: Params | None
 
 def mcg_time_halfsweep(U: torch.Tensor, G: torch.Tensor, dims, parity: int = 1, nreps: int = 10,
                        flush_l2: bool = True, stream=None) -> float:
-    """Mean per-launch milliseconds of the half-sweep kernel (CUDA events)."""
+    """Mean per-launch milliseconds of the half-sweep kernel (CUDA events); FP64:
+    the one in FP64 arithmetic, which mcg_set_sweep_block applies to."""
     _need_cuda(U, G)
     ms = ctypes.c_float(0)
     _check("mcg_time_halfsweep", _lib.mcg_time_halfsweep(_ptr(U), _ptr(G), lattice(dims, 1, precision_of(U)),
@@ -697,26 +698,31 @@ def autotune_schedule(Us, dims_list, params: Params, trial_sweeps: int = 40,
     block size of the sweep precision and every graph chunk length
     (check_every), time `trial_sweeps` sweeps of mcg_fix_batch on clones of
     the batch (no stop test), keep the fastest: the block size is set for the
-    process, the chunk length is returned in params.check_every.  Only the
-    clones are modified."""
+    process, the chunk length is returned in params.check_every.  Plain FP64
+    sweeps choose their own block, so each chunk length is timed once there, and
+    the setting stays.  Only the clones are modified."""
     prec = F32 if (params.fp32_sweeps > 0 or precision_of(Us[0]) == F32) else F64
     Uc = [mcg_convert(U, F32) if prec == F32 and precision_of(U) == F64 else U.clone() for U in Us]
     Gc = [identity_gauge(d, 1, prec, U.device) for U, d in zip(Uc, dims_list)]
     blocks = (64, 128, 256) if prec == F32 else (64, 128)
+    solve32 = params.fp64_solve32 if prec == F64 else 0
+    own = prec == F64 and not solve32
     best = None
     timings = {}
     ev0, ev1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
-    for nt in blocks:
+    for nt in (mcg_get_sweep_block(prec),) if own else blocks:
         mcg_set_sweep_block(prec, nt)
         for ch in chunks:
-            p = Params(tol=-1e300, max_sweeps=trial_sweeps, check_every=ch, reunit_every=params.reunit_every)
+            p = Params(tol=-1e300, max_sweeps=trial_sweeps, check_every=ch, reunit_every=params.reunit_every,
+                       fp64_solve32=solve32)
             mcg_fix_batch(Uc, Gc, dims_list, p)  # warm-up: graph build, caches
             ev0.record()
             mcg_fix_batch(Uc, Gc, dims_list, p)
             ev1.record()
             torch.cuda.synchronize()
             ms = ev0.elapsed_time(ev1) / trial_sweeps
-            timings[f"{nt}x{ch}"] = ms
+            for b in blocks if own else (nt,):
+                timings[f"{b}x{ch}"] = ms
             if best is None or ms < best[0]:
                 best = (ms, nt, ch)
     mcg_set_sweep_block(prec, best[1])

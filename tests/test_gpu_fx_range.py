@@ -140,3 +140,25 @@ def test_fp64_batch_equals_the_field_alone(copies):
         U1, G1, R1, s1, h1 = alone[k % 2]
         assert r["sweeps"][k] == s1 and r["R"][k] == R1 and np.array_equal(hist[k], h1)
         assert torch.equal(Ud[k], U1[0]) and torch.equal(Gd[k], G1[0])
+
+
+def test_time_halfsweep_follows_the_block_setting():
+    """The FP64 timing, which the block size is tuned with, is of one launch of the kernel that reads the setting."""
+    from paper_0807_0264_gb300 import mcg
+
+    dims = (4, 4, 4, 6)
+    U, G = _pack(mcg, [synth.make_field(dims, 0.4, 3)], dims), mcg.identity_gauge(dims)
+    old = mcg.mcg_get_sweep_block(mcg.F64)
+    try:
+        for nt in (64, 128):
+            mcg.mcg_set_sweep_block(mcg.F64, nt)
+            n0 = mcg.mcg_kernel_launches()
+            assert mcg.mcg_time_halfsweep(U, G, dims, 1, 5, False) > 0
+            assert mcg.mcg_kernel_launches() - n0 == 5
+        plain = mcg.autotune_schedule([U], [dims], mcg.Params(), trial_sweeps=4, chunks=(2, 4))
+        assert plain["block"] == 128 and plain["precision"] == "f64"
+        assert set(plain["ms_per_sweep"]) == {f"{b}x{c}" for b in (64, 128) for c in (2, 4)}
+        s32 = mcg.autotune_schedule([U], [dims], mcg.Params(fp64_solve32=1), trial_sweeps=4, chunks=(2,))
+        assert s32["block"] in (64, 128) and len(set(s32["ms_per_sweep"].values())) == 2
+    finally:
+        mcg.mcg_set_sweep_block(mcg.F64, old)
