@@ -247,9 +247,11 @@ int mcg_reunitarise(void* M, int which, const mcg_lattice* lat, cudaStream_t str
  * FP64 fields with |rho| (6 |5-2eps| / 3 + 18 |1-eps| / 12) <= 1 take the steps
  * in 64-bit fixed point of unit 2^-60 (errors below the FP64 arithmetic's), on
  * a scratch copy of the field and up to 16 GiB of scratch for products that
- * neighbouring links share; without memory for the one they run in FP64 (one
- * step needs no scratch then), without memory for the other they multiply every
- * path out.  Calls on several streams are ordered on the GPU where they share
+ * neighbouring links share.  What the steps can do without (the copy for a single
+ * step, which then runs in FP64, and the products, without which every path is
+ * multiplied out) takes at most a quarter of the free memory and is given up
+ * when another call needs scratch that no longer fits; mcg_release() frees it
+ * for the caller.  Calls on several streams are ordered on the GPU where they share
  * scratch.
  */
 int mcg_smear(const void* U_in, void* U_out, const mcg_lattice* lat, double rho, double eps, int n,

@@ -18,6 +18,7 @@
 #include "../../include/mcg.h"
 #include "mcg_common.cuh"
 #include "mcg_internal.h"
+#include "mcg_scratch.h"
 
 namespace mcg {
 
@@ -73,12 +74,32 @@ void note_phase(int prec, double ms, long long site_updates) {
 // ---------------------------------------------------------------------------
 // scratch: grow-only named buffers per device
 // ---------------------------------------------------------------------------
-struct Buf {
-    void* p = nullptr;
-    size_t bytes = 0;
+struct DeviceMem {
+    static int alloc(void** p, size_t bytes) {
+        const cudaError_t e = cudaMalloc(p, bytes);
+        if (e != cudaSuccess) cudaGetLastError();  // reported by the caller, or no error at all
+        return (int)e;
+    }
+    static void free(void* p) { cudaFree(p); }
+    static void sync() { cudaDeviceSynchronize(); }
+    static size_t available() {
+        size_t f = 0, t = 0;
+        return cudaMemGetInfo(&f, &t) == cudaSuccess ? f : 0;
+    }
+};
+struct HostMem {
+    static int alloc(void** p, size_t bytes) {
+        const cudaError_t e = cudaMallocHost(p, bytes);
+        if (e != cudaSuccess) cudaGetLastError();
+        return (int)e;
+    }
+    static void free(void* p) { cudaFreeHost(p); }
+    static void sync() { cudaDeviceSynchronize(); }
+    static size_t available() { return 0; }  // no optional buffers
 };
 struct DeviceScratch {
-    std::map<std::string, Buf> dev, host;
+    ScratchCache<DeviceMem> dev;
+    ScratchCache<HostMem> host;
     cudaStream_t cap = nullptr;
     std::vector<cudaStream_t> side;  // branch streams of captured per-field chains
     std::vector<cudaEvent_t> side_ev;
@@ -99,43 +120,24 @@ void* scratch_device(const char* name, size_t bytes, int* rc) {
     std::lock_guard<std::mutex> lk(g_mu);
     DeviceScratch& ds = cur(rc);
     if (*rc) return nullptr;
-    Buf& b = ds.dev[name];
-    if (b.bytes < bytes) {
-        if (b.p) {
-            cudaDeviceSynchronize();
-            cudaFree(b.p);
-            b.p = nullptr;
-            b.bytes = 0;
-        }
-        cudaError_t e = cudaMalloc(&b.p, std::max<size_t>(bytes, 256));
-        if (e != cudaSuccess) {
-            *rc = cuda_fail(e, "cudaMalloc(scratch)");
-            return nullptr;
-        }
-        b.bytes = std::max<size_t>(bytes, 256);
-    }
-    return b.p;
+    int err = 0;
+    void* p = ds.dev.get(name, bytes, &err);
+    if (err) *rc = cuda_fail((cudaError_t)err, "cudaMalloc(scratch)");
+    return p;
 }
 
 void* scratch_device_optional(const char* name, size_t bytes) {
     std::lock_guard<std::mutex> lk(g_mu);
     int rc = 0;
     DeviceScratch& ds = cur(&rc);
-    if (rc) return nullptr;
-    Buf& b = ds.dev[name];
-    if (b.bytes >= bytes) return b.p;
-    void* p = nullptr;
-    if (cudaMalloc(&p, bytes) != cudaSuccess) {
-        cudaGetLastError();  // not the caller's error
-        return nullptr;
-    }
-    if (b.p) {
-        cudaDeviceSynchronize();
-        cudaFree(b.p);
-    }
-    b.p = p;
-    b.bytes = bytes;
-    return p;
+    return rc ? nullptr : ds.dev.get_optional(name, bytes);
+}
+
+size_t scratch_optional_room(const char* name) {
+    std::lock_guard<std::mutex> lk(g_mu);
+    int rc = 0;
+    DeviceScratch& ds = cur(&rc);
+    return rc ? 0 : ds.dev.optional_room(name);
 }
 
 int scratch_wait(const char* group, cudaStream_t st) {
@@ -163,22 +165,10 @@ void* scratch_host(const char* name, size_t bytes, int* rc) {
     std::lock_guard<std::mutex> lk(g_mu);
     DeviceScratch& ds = cur(rc);
     if (*rc) return nullptr;
-    Buf& b = ds.host[name];
-    if (b.bytes < bytes) {
-        if (b.p) {
-            cudaDeviceSynchronize();
-            cudaFreeHost(b.p);
-            b.p = nullptr;
-            b.bytes = 0;
-        }
-        cudaError_t e = cudaMallocHost(&b.p, std::max<size_t>(bytes, 256));
-        if (e != cudaSuccess) {
-            *rc = cuda_fail(e, "cudaMallocHost(scratch)");
-            return nullptr;
-        }
-        b.bytes = std::max<size_t>(bytes, 256);
-    }
-    return b.p;
+    int err = 0;
+    void* p = ds.host.get(name, bytes, &err);
+    if (err) *rc = cuda_fail((cudaError_t)err, "cudaMallocHost(scratch)");
+    return p;
 }
 
 cudaStream_t capture_stream(int* rc) {
@@ -228,10 +218,8 @@ void release_all() {
     for (auto& kv : g_scratch) {
         cudaSetDevice(kv.first);
         cudaDeviceSynchronize();
-        for (auto& b : kv.second.dev)
-            if (b.second.p) cudaFree(b.second.p);
-        for (auto& b : kv.second.host)
-            if (b.second.p) cudaFreeHost(b.second.p);
+        kv.second.dev.clear();
+        kv.second.host.clear();
         if (kv.second.cap) cudaStreamDestroy(kv.second.cap);
         for (auto s : kv.second.side) cudaStreamDestroy(s);
         for (auto ev : kv.second.side_ev) cudaEventDestroy(ev);

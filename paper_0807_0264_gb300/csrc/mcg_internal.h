@@ -47,9 +47,12 @@ void note_phase(int prec, double ms, long long site_updates);
 // Named, grow-only device and pinned-host buffers cached per device; freed by
 // mcg_release().
 void* scratch_device(const char* name, size_t bytes, int* rc);
-// The same for memory that the caller can do without: null, and no error, when
-// there is none (the old buffer, if any, is kept).
+// The same for memory that the caller can do without (mcg_scratch.h): null, and no
+// error, when there is none or it would take more than a quarter of what is free.
+// The pointer holds until the call's next scratch_device; room: the bytes that a
+// request would get.
 void* scratch_device_optional(const char* name, size_t bytes);
+size_t scratch_optional_room(const char* name);
 // Around an asynchronous use of a group of scratch buffers: the stream waits for
 // the group's last use, which may have been on another stream; the end of this
 // one.  Not for streams that are being captured.

@@ -314,17 +314,21 @@ static auto step_kernel(bool rect, bool shared, bool out64) {
 }
 
 // Scratch of the products at most: 9.9 million sites of a stout step, 3.3 million
-// of an over-improved one at a time.  A field beyond it, or with no memory for it,
-// takes the step that multiplies every path out.
+// of an over-improved one at a time, and fewer fields at a time where a quarter of
+// the free memory is less.  A field beyond that takes the step that multiplies
+// every path out.
 constexpr size_t kFxAuxBytes = (size_t)16 << 30;
 
 int run_smear_fx(const void* Uin, void* Uout, const Geom& g, int nfields, double rho, double eps, int n, bool* ran,
                  cudaStream_t st) {
     const size_t elems = link_elems(g) * (size_t)nfields;
-    void* tmp = scratch_device_optional("smear.tmp", 16 * elems);
+    // several steps need a second field in any arithmetic, one step only here
+    int rc = 0;
+    void* tmp = n >= 2 ? scratch_device("smear.tmp", 16 * elems, &rc) : scratch_device_optional("smear.tmp", 16 * elems);
+    if (rc) return rc;
     *ran = tmp != nullptr;
     if (!tmp) return 0;
-    if (int rc = scratch_wait("smear", st)) return rc;
+    if ((rc = scratch_wait("smear", st))) return rc;
     const bool rect = eps != 1.0;
     const FxSmear P = fx_smear_params(rho, eps, 1.0);
     // step k's source: tmp or Uout in turn, so that the last step reads tmp
@@ -336,6 +340,10 @@ int run_smear_fx(const void* Uin, void* Uout, const Geom& g, int nfields, double
     const size_t per_field = 16 * ((rect ? kFxAux<true> : kFxAux<false>) / 4) * link_elems(g);
     chunk = (int)std::min<size_t>(nfields, kFxAuxBytes / per_field);
     if (chunk > 0) aux = (int4*)scratch_device_optional("smear.products", per_field * chunk);
+    if (chunk > 0 && !aux) {
+        chunk = (int)std::min<size_t>(chunk, scratch_optional_room("smear.products") / per_field);
+        if (chunk > 0) aux = (int4*)scratch_device_optional("smear.products", per_field * chunk);
+    }
     if (!aux) chunk = nfields;
     for (int k = 0; k < n; ++k) {
         const bool last = k + 1 == n;
