@@ -47,12 +47,55 @@ __device__ __noinline__ void apply_link_f64(double2* u, const double2* w, const 
     for (int e = 0; e < 9; ++e) u[e * vh] = make_double2(a[e].x, a[e].y);
 }
 
+// A site whose transform the hand-off did not take in fixed point: no low half has
+// this value (fx_split)
+constexpr int kFxMarked = -0x7fffffff - 1;
+
+// The compact FP32 (or hi + lo) transform of a site, re-unitarised in FP64
+__device__ __forceinline__ void handoff_transform_f64(const float4* W, const float4* Wlo, size_t vh, cplx<double>* w) {
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+        const float4 v = W[q * vh], l = Wlo ? Wlo[q * vh] : make_float4(0.f, 0.f, 0.f, 0.f);
+        w[2 * q] = mk((double)v.x + (double)l.x, (double)v.y + (double)l.y);
+        w[2 * q + 1] = mk((double)v.z + (double)l.z, (double)v.w + (double)l.w);
+    }
+#pragma unroll
+    for (int e = 6; e < 9; ++e) w[e] = mk(0.0, 0.0);
+    m3_reunitarise(w);
+}
+// u <- w u wf^dag in FP64 where one of the transforms is marked
+__device__ __noinline__ void handoff_link_f64(double2* u, const int4* w, const int4* wf, const float4* W,
+                                              const float4* Wlo, const float4* Wf, const float4* Wflo, size_t vh) {
+    cplx<double> a[9], b[9], t[9];
+    auto transform = [&](const int4* x, const float4* hi, const float4* lo, cplx<double>* m) {
+        if (x->y == kFxMarked) {
+            handoff_transform_f64(hi, lo, vh, m);
+            return;
+        }
+#pragma unroll
+        for (int e = 0; e < 9; ++e) {
+            const cfx v = fx_load(x + e * vh);
+            m[e] = mk(fx_double(fx_join(v.re)), fx_double(fx_join(v.im)));
+        }
+    };
+    transform(w, W, Wlo, a);
+#pragma unroll
+    for (int e = 0; e < 9; ++e) b[e] = mk(u[e * vh].x, u[e * vh].y);
+    m3_mul(a, b, t);
+    transform(wf, Wf, Wflo, b);
+    m3_mul_nd(t, b, a);
+#pragma unroll
+    for (int e = 0; e < 9; ++e) u[e * vh] = make_double2(a[e].x, a[e].y);
+}
+
 // One thread per link.  WFX: the transform in fixed point, of an SU(3) field (the
-// hand-off).  Two products and 18 to 54 conversions per link, bound by the
-// integer multiplier.  A thread per link: the products need no more registers
-// than three blocks of 128 per SM leave, and small lattices fill more SMs.
+// hand-off; W and Wlo are what it came from, read for marked sites).  Two products
+// and 18 to 54 conversions per link, bound by the integer multiplier.  A thread
+// per link: the products need no more registers than three blocks of 128 per SM
+// leave, and small lattices fill more SMs.
 template <bool WFX>
-__global__ void __launch_bounds__(128, 3) k_apply_gauge_fx(double2* Uall, const void* Gall, Geom g, int nfields) {
+__global__ void __launch_bounds__(128, 3) k_apply_gauge_fx(double2* Uall, const void* Gall, const float4* W,
+                                                           const float4* Wlo, Geom g, int nfields) {
     const long long id = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (id >= 8LL * g.vh * nfields) return;
     const int f = (int)(id / (8LL * g.vh));
@@ -64,7 +107,8 @@ __global__ void __launch_bounds__(128, 3) k_apply_gauge_fx(double2* Uall, const 
     int c[4];
     eo_coords(g, p, s, c);
     const size_t iw = (size_t)f * gauge_elems(g) + gidx(g, p, 0, s);
-    const size_t iwf = (size_t)f * gauge_elems(g) + gidx(g, p ^ 1, 0, eo_neighbor(g, c, mu, +1));
+    const int sf = eo_neighbor(g, c, mu, +1);
+    const size_t iwf = (size_t)f * gauge_elems(g) + gidx(g, p ^ 1, 0, sf);
     double2* u = Uall + (size_t)f * link_elems(g) + lidx(g, mu, p, 0, s);
     cfx a[9], b[9];
     bool bad = false;
@@ -72,6 +116,7 @@ __global__ void __launch_bounds__(128, 3) k_apply_gauge_fx(double2* Uall, const 
         const int4* w = reinterpret_cast<const int4*>(Gall) + iw;
 #pragma unroll
         for (int e = 0; e < 9; ++e) a[e] = fx_load(w + e * vh);
+        bad = a[0].re.l == kFxMarked;
     } else {
         bad = fx_load_matrix(reinterpret_cast<const double2*>(Gall) + iw, 3 * vh, vh, a);
     }
@@ -82,6 +127,13 @@ __global__ void __launch_bounds__(128, 3) k_apply_gauge_fx(double2* Uall, const 
         const int4* w = reinterpret_cast<const int4*>(Gall) + iwf;
 #pragma unroll
         for (int e = 0; e < 9; ++e) b[e] = fx_load(w + e * vh);
+        if (bad || b[0].re.l == kFxMarked) {
+            const size_t i = (size_t)f * c12_gauge_chunks(g) + c12_gidx(g, p, 0, s);
+            const size_t j = (size_t)f * c12_gauge_chunks(g) + c12_gidx(g, p ^ 1, 0, sf);
+            handoff_link_f64(u, reinterpret_cast<const int4*>(Gall) + iw, w, W + i, Wlo ? Wlo + i : nullptr, W + j,
+                             Wlo ? Wlo + j : nullptr, vh);
+            return;
+        }
     } else {
         bad = fx_load_matrix(reinterpret_cast<const double2*>(Gall) + iwf, 3 * vh, vh, b) || bad;
     }
@@ -96,8 +148,19 @@ __global__ void __launch_bounds__(128, 3) k_apply_gauge_fx(double2* Uall, const 
 
 // ---- hand-off of the mixed schedule, pass 1 --------------------------------------
 // W (compact: rows 0 and 1, FP32 or hi + lo) re-unitarised, to scratch in fixed
-// point; Omega <- reunit(W Omega).  W is unitary to FP32 rounding, Omega a
-// validated transform.
+// point; Omega <- reunit(W Omega).  Omega is a validated transform, W unitary to
+// FP32 rounding: a site where it is not (or not finite) is marked for pass 2 and
+// done in FP64.
+__device__ __noinline__ void handoff_gauge_f64(const float4* W, const float4* Wlo, double2* G, size_t vh) {
+    cplx<double> w[9], o[9], t[9];
+    handoff_transform_f64(W, Wlo, vh, w);
+#pragma unroll
+    for (int e = 0; e < 9; ++e) o[e] = mk(G[e * vh].x, G[e * vh].y);
+    m3_mul(w, o, t);
+    m3_reunitarise(t);
+#pragma unroll
+    for (int e = 0; e < 9; ++e) G[e * vh] = make_double2(t[e].x, t[e].y);
+}
 __global__ void __launch_bounds__(128, 3) k_handoff_gauge_fx(const float4* __restrict__ W,
                                                               const float4* __restrict__ Wlo, int4* __restrict__ Wfx,
                                                               double2* __restrict__ G, Geom g, int nfields) {
@@ -110,22 +173,29 @@ __global__ void __launch_bounds__(128, 3) k_handoff_gauge_fx(const float4* __res
     const size_t off = (size_t)f * gauge_elems(g) + gidx(g, p, 0, s), vh = (size_t)g.vh;
     const size_t coff = (size_t)f * c12_gauge_chunks(g) + c12_gidx(g, p, 0, s);
     cfx w[9], o[9];
+    unsigned big = 0;
 #pragma unroll
     for (int q = 0; q < 3; ++q) {
         const float4 v = W[coff + q * vh];
+        big = max(max(big, max(fx_magnitude(v.x), fx_magnitude(v.y))), max(fx_magnitude(v.z), fx_magnitude(v.w)));
         w[2 * q].re = fx_of(v.x);
         w[2 * q].im = fx_of(v.y);
         w[2 * q + 1].re = fx_of(v.z);
         w[2 * q + 1].im = fx_of(v.w);
         if (Wlo) {
             const float4 l = Wlo[coff + q * vh];
+            big = max(max(big, max(fx_magnitude(l.x), fx_magnitude(l.y))), max(fx_magnitude(l.z), fx_magnitude(l.w)));
             w[2 * q].re = fx_split(fx_join(w[2 * q].re) + fx_join(fx_of(l.x)));
             w[2 * q].im = fx_split(fx_join(w[2 * q].im) + fx_join(fx_of(l.y)));
             w[2 * q + 1].re = fx_split(fx_join(w[2 * q + 1].re) + fx_join(fx_of(l.z)));
             w[2 * q + 1].im = fx_split(fx_join(w[2 * q + 1].im) + fx_join(fx_of(l.w)));
         }
     }
-    m3fx_reunitarise(w);
+    if (m3fx_reunitarise(w) || big > kFxMagnitude) {
+        Wfx[off] = make_int4(0, kFxMarked, 0, 0);
+        handoff_gauge_f64(W + coff, Wlo ? Wlo + coff : nullptr, G + off, vh);
+        return;
+    }
 #pragma unroll
     for (int e = 0; e < 9; ++e) {
         Wfx[off + e * vh] = fx_pack(w[e]);
@@ -240,7 +310,8 @@ __global__ void __launch_bounds__(256, 2) k_plaquette_fx(const void* Uall, Geom 
 }  // namespace
 
 int launch_apply_gauge_fx(void* U, const void* G, const Geom& g, int nfields, cudaStream_t st) {
-    k_apply_gauge_fx<false><<<blocks(8LL * g.vh * nfields, 128), 128, 0, st>>>((double2*)U, G, g, nfields);
+    k_apply_gauge_fx<false><<<blocks(8LL * g.vh * nfields, 128), 128, 0, st>>>((double2*)U, G, nullptr, nullptr, g,
+                                                                                   nfields);
     MCG_CK(cudaGetLastError());
     note_launches(1);
     return 0;
@@ -253,7 +324,8 @@ int launch_handoff_fx(const void* W32, const void* W32lo, double* U64, double* G
     if (rc) return rc;
     k_handoff_gauge_fx<<<blocks(2LL * g.vh * nfields, 128), 128, 0, st>>>(
         (const float4*)W32, (const float4*)W32lo, Wfx, (double2*)G64, g, nfields);
-    k_apply_gauge_fx<true><<<blocks(8LL * g.vh * nfields, 128), 128, 0, st>>>((double2*)U64, Wfx, g, nfields);
+    k_apply_gauge_fx<true><<<blocks(8LL * g.vh * nfields, 128), 128, 0, st>>>(
+        (double2*)U64, Wfx, (const float4*)W32, (const float4*)W32lo, g, nfields);
     MCG_CK(cudaGetLastError());
     note_launches(2);
     return 0;

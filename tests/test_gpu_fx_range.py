@@ -1,5 +1,7 @@
 """FP64 entry points at the limits of their fixed-point kernels: links that are not unitary though their rows are
 of unit norm, schedules and batches."""
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -162,3 +164,39 @@ def test_time_halfsweep_follows_the_block_setting():
         assert s32["block"] in (64, 128) and len(set(s32["ms_per_sweep"].values())) == 2
     finally:
         mcg.mcg_set_sweep_block(mcg.F64, old)
+
+
+# the hand-off of a transform W that is not near-unitary at some sites, or not finite: the FP64 form there, as in the
+# FP64 hand-off (~60 roundings of 1.1e-16; the links' transforms are unitary, entries at most 1)
+@pytest.mark.parametrize("lo", [False, True])
+def test_handoff_of_transforms_off_unitarity(lo):
+    from paper_0807_0264_gb300 import mcg
+
+    class Geom(ctypes.Structure):
+        _fields_ = [("n", ctypes.c_int * 4), ("vh", ctypes.c_int)]
+
+    fn = mcg.library()["_ZN3mcg14launch_handoffEPKvS1_PdS2_RKNS_4GeomEibP11CUstream_st"]
+    fn.argtypes = [ctypes.c_void_p] * 4 + [ctypes.POINTER(Geom), ctypes.c_int, ctypes.c_bool, ctypes.c_void_p]
+    dims = (4, 2, 6, 4)
+    vh = int(np.prod(dims)) // 2
+    g = Geom((ctypes.c_int * 4)(*dims), vh)
+    W = synth.random_gauge(dims, 5)[:, :2].reshape(2 * vh, 6).astype(np.complex64)
+    W[3] *= 1.5
+    W[11, 2] = np.nan
+    W[vh + 5, 4] += 0.3
+    W[vh + 9] *= np.complex64(1e20)
+    # compact storage: three chunks of two entries per matrix, (parity, chunk, site)
+    chunks = np.ascontiguousarray(W.view(np.float32).reshape(2, vh, 3, 4).transpose(0, 2, 1, 3))
+    Wd = torch.from_numpy(chunks).cuda()
+    Wl = torch.from_numpy(1e-9 * np.random.default_rng(1).standard_normal(chunks.shape).astype(np.float32)).cuda()
+    out = []
+    for keep in (True, False):
+        U = _pack(mcg, [synth.make_field(dims, 0.7, 2)], dims)
+        G = mcg.mcg_pack_gauge(torch.from_numpy(synth.random_gauge(dims, 8)).unsqueeze(0).cuda(), dims)
+        torch.cuda.synchronize()
+        assert fn(Wd.data_ptr(), Wl.data_ptr() if lo else None, U.data_ptr(), G.data_ptr(), ctypes.byref(g), 1, keep, None) == 0
+        torch.cuda.synchronize()
+        out.append((U.cpu(), G.cpu()))
+    for a, b in zip(*out):
+        assert a.isnan().any() and torch.equal(a.isnan(), b.isnan())
+        assert float((a - b).nan_to_num().abs().max()) < 1e-14
