@@ -1137,8 +1137,10 @@ int run_fix_phase(const std::vector<FieldDesc>& fields_in, FieldState* d_state, 
     const int nodes_per_chunk = (chained ? nf : 1) * chunk * 3;
     // every chunk sweeps each field that is not done `chunk` times: after these
     // all are at the cap (one chunk more, of launches that exit at entry, cost
-    // 70 us of 2 200 on 50 sweeps of a 16^3 x 32 FP32 field)
-    const int max_chunks = (phase_len + chunk - 1) / chunk;
+    // 70 us of 2 200 on 50 sweeps of a 16^3 x 32 FP32 field).  A field that stops
+    // in the chunk ahead of its restart loses up to a chunk of sweeps: one more
+    // chunk for each restart of a field.
+    int max_chunks = (phase_len + chunk - 1) / chunk;
     int status = 0;
     // The next chunk is launched before the host reads the state after the
     // current one, so the GPU does not wait for the host between chunks: a
@@ -1266,6 +1268,7 @@ int run_fix_phase(const std::vector<FieldDesc>& fields_in, FieldState* d_state, 
                         break;
                     }
                     ++nrestart[f];
+                    max_chunks = std::max(max_chunks, (phase_len + chunk - 1) / chunk + nrestart[f]);
                     valid_from[f] = c + 2;
                     creep_n[f] = 0;
                     last_sweep[f] = -1;

@@ -200,3 +200,28 @@ def test_handoff_of_transforms_off_unitarity(lo):
     for a, b in zip(*out):
         assert a.isnan().any() and torch.equal(a.isnan(), b.isnan())
         assert float((a - b).nan_to_num().abs().max()) < 1e-14
+
+
+# a field that stops in the chunk in flight when a restart is queued behind it begins again all the same, and sweeps up
+# to the phase's cap: each pass takes S sweeps of two chunks, five passes fit
+@pytest.mark.parametrize("copies", [1, 3])
+def test_restarts_up_to_the_cap(copies):
+    from paper_0807_0264_gb300 import mcg
+
+    dims = (4, 4, 4, 6)
+    U = _pack(mcg, [synth.make_field(dims, 0.4, 7, gauge=False)], dims)
+
+    def sweeps32(cap, chunk, restart):
+        prm = mcg.Params(tol=1e300, max_sweeps=100000, check_every=chunk, fp32_sweeps=cap, fp32_tol=1e-5, fp32_window=1,
+                         fp32_restart=restart)
+        if copies == 1:
+            return mcg.mcg_precondition_fix(U.clone(), mcg.identity_gauge(dims), dims, prm)[0]["sweeps_fp32"]
+        rs = mcg.mcg_precondition_fix(torch.cat([U] * copies), mcg.identity_gauge(dims, copies), dims, prm)
+        assert len({r["sweeps_fp32"] for r in rs}) == 1
+        return rs[0]["sweeps_fp32"]
+
+    S = sweeps32(1000, 20, 0)
+    assert 6 <= S < 100, S
+    chunk = (2 * S) // 3
+    assert chunk < S < 2 * chunk
+    assert sweeps32(5 * S, chunk, chunk) == 5 * S
