@@ -96,8 +96,8 @@ MCG_HD long long fx_from_bits(unsigned long long bits) {
     const long long sg = (long long)bits >> 63;
     return ((long long)v ^ sg) - sg;
 }
-// X 2^-60 rounded to FP64 (ties away from zero)
-MCG_HD unsigned long long fx_to_bits(long long X) {
+// X 2^-60 rounded to FP64 (ties away from zero; half = 511: towards zero)
+MCG_HD unsigned long long fx_to_bits(long long X, unsigned half = 512) {
     const long long sg = X >> 63;
     unsigned long long m = (unsigned long long)((X ^ sg) - sg);
 #ifdef __CUDA_ARCH__
@@ -107,7 +107,7 @@ MCG_HD unsigned long long fx_to_bits(long long X) {
 #endif
     // top bit to 62; the value is then m 2^(-60 - (z - 1))
     m = z > 0 ? m << ((z - 1) & 63) : m >> 1;
-    const unsigned long long q = (m + (1ULL << 9)) >> 10;  // 53 bits, implicit one at bit 52
+    const unsigned long long q = (m + half) >> 10;  // 53 bits, implicit one at bit 52
     // exponent field: 1023 + 2 - (z - 1), less the one the implicit bit adds
     const unsigned long long d = q + ((unsigned long long)(1025 - z) << 52);
     const unsigned long long s = (unsigned long long)sg & 0x8000000000000000ULL;

@@ -225,3 +225,17 @@ def test_restarts_up_to_the_cap(copies):
     chunk = (2 * S) // 3
     assert chunk < S < 2 * chunk
     assert sweeps32(5 * S, chunk, chunk) == 5 * S
+
+
+# round-off of long plain FP64 fixes is a random walk: each sweep stores every link twice and the transforms of its ends
+# once, ~6e-17 rms together; the bar is twice sqrt(n) of that
+@pytest.mark.parametrize("n,seed", [(1000, 3), (3000, 4)])
+def test_long_fixes_stay_on_the_gauge_orbit(n, seed):
+    from paper_0807_0264_gb300 import mcg
+
+    dims = (6, 4, 6, 8)
+    U0 = synth.make_field(dims, 2.0, seed)
+    U, G = _pack(mcg, [U0], dims), mcg.identity_gauge(dims)
+    mcg.mcg_fix(U, G, dims, mcg.Params(tol=-1e300, max_sweeps=n, check_every=50))
+    d = oracle.apply_gauge(dims, U0, mcg.mcg_unpack_gauge(G, dims)[0].cpu().numpy()) - mcg.mcg_unpack_links(U, dims)[0].cpu().numpy()
+    assert np.sqrt((np.abs(d) ** 2).mean()) < 2 * 6e-17 * np.sqrt(n)
