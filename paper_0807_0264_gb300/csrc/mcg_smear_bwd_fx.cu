@@ -4,8 +4,11 @@
 //
 // Gradients have no bound of their own, so each matrix carries a power of two:
 // pass 1 scales a link's gradient to components below 1/2 (exponent e), pass 2
-// brings the matrices it meets to the largest exponent among them (block
-// floating point: an error of 2^-57 of the largest neighbour).
+// brings the matrices that reach a link through its staples to the largest
+// exponent among them (block floating point: an error of 2^-57 of the largest,
+// times the staples' weight, which a power of two keeps between 1/2 and 1 until the
+// end).  The link's own part keeps its own exponent, so that it loses nothing beside
+// large neighbours, at rho = 0 not even a digit.
 #include <cuda_runtime.h>
 
 #include "mcg_common.cuh"
@@ -429,7 +432,7 @@ __global__ void __launch_bounds__(128, 3)
                     }
                 }
                 const bool dag = fj.dag;
-                const fx w = k < 2 ? P.wp : P.wr64;
+                const fx w = k < 2 ? P.gp : P.gr64;
                 const int ws = k < 2 ? 1 : 7, half = 1 << (ws - 1);
 #pragma unroll
                 for (int i = 0; i < 3; ++i)
@@ -451,14 +454,38 @@ __global__ void __launch_bounds__(128, 3)
     }
     int4* out = Gall + foff + lidx(g, lam, p, 0, s);
     constexpr int up = RECT ? 1 : 3;
-    const int sh = min(em - e_own + up, 63);
+    if (!RECT) {
 #pragma unroll
-    for (int e = 0; e < 9; ++e) {
-        const cfx v = fx_load(out + e * vh);
-        const long long re = (fx_join(v.re) >> sh) + (RECT ? S[2 * e] : fx_mul(fx_split(S[2 * e]), P.wp));
-        const long long im = (fx_join(v.im) >> sh) + (RECT ? S[2 * e + 1] : fx_mul(fx_split(S[2 * e + 1]), P.wp));
-        reinterpret_cast<double2*>(out)[e * vh] =
-            make_double2(fx_double_scaled(re, em + up), fx_double_scaled(im, em + up));
+        for (int e = 0; e < 18; ++e) S[e] = fx_mul(fx_split(S[e]), P.gp);
+    }
+    // the link's own part in units of 2^(e_own - 60), the staples' in 2^(em + up - gs
+    // - 60): one integer sum in units of 2^(em + up - 60) where that costs the own
+    // part no digit that FP64 holds, else (a link whose gradient is far below its
+    // neighbours') each to FP64 first
+    const int sh = em - e_own + up, gs = min(P.gs, 63);
+    if (sh <= 6) {
+#pragma unroll
+        for (int e = 0; e < 9; ++e) {
+            const cfx v = fx_load(out + e * vh);
+            const long long re = (fx_join(v.re) >> sh) + (S[2 * e] >> gs);
+            const long long im = (fx_join(v.im) >> sh) + (S[2 * e + 1] >> gs);
+            reinterpret_cast<double2*>(out)[e * vh] =
+                make_double2(fx_double_scaled(re, em + up), fx_double_scaled(im, em + up));
+        }
+    } else {
+#pragma unroll 1
+        for (int e = 0; e < 9; ++e) {
+            const cfx v = fx_load(out + e * vh);
+            long long re = S[0], im = S[1];
+#pragma unroll
+            for (int k = 1; k < 9; ++k) {
+                re = e == k ? S[2 * k] : re;
+                im = e == k ? S[2 * k + 1] : im;
+            }
+            reinterpret_cast<double2*>(out)[e * vh] =
+                make_double2(fx_double_scaled(fx_join(v.re), e_own) + fx_double_scaled(re, em + up - P.gs),
+                             fx_double_scaled(fx_join(v.im), e_own) + fx_double_scaled(im, em + up - P.gs));
+        }
     }
 }
 

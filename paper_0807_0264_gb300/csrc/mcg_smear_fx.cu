@@ -283,11 +283,15 @@ FxSmear fx_smear_params(double rho, double eps, double slack) {
     FxSmear P;
     P.wp = host_fx(rho * cp);
     P.wr = host_fx(8.0 * rho * cr);
-    P.wr64 = host_fx(64.0 * rho * cr);
+    const double weight = std::fabs(rho) * (6.0 * std::fabs(cp) + 18.0 * std::fabs(cr));
+    P.gs = weight > 0.0 ? -std::ilogb(weight) - 1 : 0;
+    if (P.gs < 0) P.gs = 0;  // weight = 1
+    P.gp = host_fx(std::ldexp(rho * cp, P.gs));
+    P.gr64 = host_fx(std::ldexp(64.0 * rho * cr, P.gs));
     P.third = fx_split(((1LL << 60) + 1) / 3);
     // 2^k / k! with 40 guard bits, rounded to 2^-60; terms until the bound
     // r^k / k! on the rest is below 2^-62, r = 4/3 of the staple weight
-    const double rad = slack * 4.0 / 3.0 * std::fabs(rho) * (6.0 * std::fabs(cp) + 18.0 * std::fabs(cr));
+    const double rad = slack * 4.0 / 3.0 * weight;
     unsigned __int128 t = (unsigned __int128)1 << 100;
     double rest = 1.0;
     P.nterms = 0;

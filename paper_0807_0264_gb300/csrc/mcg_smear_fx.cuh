@@ -35,7 +35,9 @@ constexpr int kFxTerms = 28;  // series terms of exp(iQ) at most
 // bounds the rows of the weighted staple sum by 1 and the spectral radius of Q by
 // 4/3.
 struct FxSmear {
-    fx wp, wr, wr64;     // rho times the plaquette weight; 8 and 64 times rho times the rectangle weight
+    fx wp, wr;           // rho times the plaquette weight; 8 times rho times the rectangle weight
+    fx gp, gr64;         // for gradients: wp and 8 wr times 2^gs, the weights of all staples
+    int gs;              // together then between 1/2 and 1 (small rho: no loss of digits)
     fx third;            // 1/3
     fx term[kFxTerms];   // i^k 2^k / k! without the factor i of odd k (sign of k % 4 in {2, 3}: minus)
     int nterms;          // even

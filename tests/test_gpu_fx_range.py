@@ -239,3 +239,23 @@ def test_long_fixes_stay_on_the_gauge_orbit(n, seed):
     mcg.mcg_fix(U, G, dims, mcg.Params(tol=-1e300, max_sweeps=n, check_every=50))
     d = oracle.apply_gauge(dims, U0, mcg.mcg_unpack_gauge(G, dims)[0].cpu().numpy()) - mcg.mcg_unpack_links(U, dims)[0].cpu().numpy()
     assert np.sqrt((np.abs(d) ** 2).mean()) < 2 * 6e-17 * np.sqrt(n)
+
+
+# links whose output gradients differ by many orders: a term keeps its own precision, as in FP64 arithmetic, where the
+# large ones near it do not reach it (rho = 0) or reach it by a small weight
+@pytest.mark.parametrize("eps", [1.0, -0.25])
+@pytest.mark.parametrize("rho", [0.0, 1e-18, 1e-9])
+def test_smear_backward_of_unequal_gradients(eps, rho):
+    from paper_0807_0264_gb300 import mcg
+
+    dims, rng = (4, 2, 6, 4), np.random.default_rng(9)
+    U = synth.make_field(dims, 0.7, 9)
+    G = rng.standard_normal(U.shape) + 1j * rng.standard_normal(U.shape)
+    G *= 10.0 ** rng.integers(-6, 7, U.shape[:2] + (1, 1))
+    got = mcg.mcg_smear_backward_step(_pack(mcg, [U], dims), _pack(mcg, [G], dims), dims, rho, eps)
+    got = mcg.mcg_unpack_links(got, dims)[0].cpu().numpy()
+    ref = oracle.smear_step_backward(dims, U, G, rho, eps)
+    # per link: ~30 roundings of 1.1e-16 of its own gradient, and of the weighted sum of up to 24 staples of its neighbours
+    own = np.abs(G).max(axis=(-2, -1))
+    bar = 5e-15 * own + 24 * 5e-15 * rho * np.abs(G).max()
+    assert (np.abs(got - ref).max(axis=(-2, -1)) < bar).all()
