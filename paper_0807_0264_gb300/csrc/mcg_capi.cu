@@ -890,9 +890,10 @@ long long mcg_bounds_violations(int reset) {
 #ifdef MCG_CHECK
     cudaDeviceSynchronize();
     const bool r = reset != 0;
-    return (long long)(bound_hits_field(r) + bound_hits_field_fx(r) + bound_hits_observables(r) + bound_hits_smear(r) + bound_hits_smear_fx(r) + bound_hits_smear_bwd_fx(r) +
+    return (long long)(bound_hits_field(r) + bound_hits_field_fx(r) + bound_hits_observables(r) +
+                       bound_hits_smear(r) + bound_hits_smear_fx(r) + bound_hits_smear_bwd_fx(r) +
                        bound_hits_sweep(r) + bound_hits_sweep_f32(r) + bound_hits_sweep_fx(r) +
-                       bound_hits_sweep_df(r));
+                       bound_hits_sweep_df(r) + bound_hits_wilson_fx(r));
 #else
     (void)reset;
     return -1;

@@ -74,6 +74,7 @@ unsigned long long bound_hits_sweep(bool reset);
 unsigned long long bound_hits_sweep_f32(bool reset);
 unsigned long long bound_hits_sweep_fx(bool reset);
 unsigned long long bound_hits_sweep_df(bool reset);
+unsigned long long bound_hits_wilson_fx(bool reset);
 void release_all();
 
 // ---- batched sweep machinery -------------------------------------------------

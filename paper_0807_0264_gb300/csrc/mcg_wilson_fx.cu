@@ -32,6 +32,15 @@ __device__ __forceinline__ int lex_moved(const Geom& g, const int c[4], int4 d, 
     return q[0] + g.n[0] * (q[1] + g.n[1] * (q[2] + g.n[2] * q[3]));
 }
 
+// entry e of site x of line field `line` (T - 1 of the temporal ones, the path of
+// the spatial ones), n of them
+__device__ __forceinline__ size_t line_idx(int V, int n, int line, int e, int x) {
+#ifdef MCG_CHECK
+    if (mcg_bad((unsigned)line >= (unsigned)n || (unsigned)e >= 9u || (unsigned)x >= (unsigned)V)) return 0;
+#endif
+    return ((size_t)line * 9 + e) * V + x;
+}
+
 // One step of up to three paths at once (blockIdx.y): Pout(x) = Pin(x) times the
 // link of direction `axis` at x + from, daggered for a backward step (from: the
 // site the link starts at); first: Pin is the identity.
@@ -40,7 +49,7 @@ __global__ void __launch_bounds__(WT, 3) k_path_step_fx(const double2* __restric
     const int V = 2 * g.vh, x = blockIdx.x * WT + threadIdx.x;
     if (x >= V) return;
     const PathStep st = ps.step[blockIdx.y];
-    const size_t off = (size_t)blockIdx.y * 9 * V + x;
+    const size_t off = line_idx(V, (int)gridDim.y, (int)blockIdx.y, 0, x);
     int c[4], q[4];
     lex_coords(g, x, c);
     const int y = lex_moved(g, c, make_int4(st.from[0], st.from[1], st.from[2], st.from[3]), q);
@@ -81,8 +90,8 @@ __global__ void __launch_bounds__(WT, 4) k_wilson_fx(const int4* __restrict__ P,
     long long sum = 0;
     if (x < V) {
         const PathStep st = ps.step[blockIdx.z];
-        const int4* Pz = P + (size_t)blockIdx.z * 9 * sV;
-        const int4* L = St + (size_t)blockIdx.y * 9 * sV;
+        const int4* Pz = P + line_idx(V, (int)gridDim.z, (int)blockIdx.z, 0, 0);
+        const int4* L = St + line_idx(V, (int)gridDim.y, (int)blockIdx.y, 0, 0);
         int c[4], q[4];
         lex_coords(g, x, c);
         const int xr = lex_moved(g, c, make_int4(st.from[0], st.from[1], st.from[2], st.from[3]), q);
@@ -90,8 +99,8 @@ __global__ void __launch_bounds__(WT, 4) k_wilson_fx(const int4* __restrict__ P,
         cfx a[9], b[9];
 #pragma unroll
         for (int e = 0; e < 9; ++e) {
-            a[e] = fx_load(L + e * sV + xr);
-            b[e] = fx_load(Pz + e * sV + xt);
+            a[e] = fx_load(L + line_idx(V, 1, 0, e, xr));
+            b[e] = fx_load(Pz + line_idx(V, 1, 0, e, xt));
         }
         facc t = facc_zero();
 #pragma unroll 1
@@ -154,5 +163,8 @@ void launch_wilson_fx(const void* P, const void* St, const Geom& g, const PathSt
     k_wilson_fx<<<dim3(nb, Tmax, npath), WT, 0, st>>>((const int4*)P, (const int4*)St, g, ps, partial);
     k_sum_loops<<<Tmax, 256, 0, st>>>(partial, nb, npath, scale, out);
 }
+
+// index-check counter of this unit (MCG_CHECK builds)
+MCG_BOUND_READER(bound_hits_wilson_fx)
 
 }  // namespace mcg
