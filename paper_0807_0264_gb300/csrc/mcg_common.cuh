@@ -278,13 +278,17 @@ __device__ __forceinline__ int eo_neighbor(const Geom& g, const int c[4], int mu
 // index a field beyond L2 was streamed once per direction (stout steps, tiled and
 // not: FP64 20^3 x 40 0.81 and 0.89 ms, FP32 16^3 x 32 68 and 71 us).  Steps with
 // rectangles reach two sites far and go by the direction first (over-improved
-// FP64, 12 x 10 x 14 x 22: 0.40 ms tiled, 0.37).
+// FP64, tiled and not: 12 x 10 x 14 x 22 0.41 and 0.37 ms, 16^3 x 32 1.30 and 1.23,
+// 20^3 x 40 3.14 and 3.03).  So do lattices whose last tile would leave more than a
+// sixteenth of the threads idle, all of them small (4 096 FP32 fields of 2^4, five
+// steps: 716 us tiled, 310 not).
 struct LinkItem {
     int f, kind, p, s;
 };
+__host__ __device__ __forceinline__ bool link_tiled(const Geom& g) { return (-g.vh & 63) * 16 <= g.vh; }
 template <bool TILED>
 __device__ __forceinline__ bool link_item(const Geom& g, int ndir, int nfields, LinkItem& r) {
-    if (TILED) {
+    if (TILED && link_tiled(g)) {
         const unsigned tiles = ((unsigned)g.vh + 63) / 64, b = blockIdx.x / ndir;
         r.kind = (int)(blockIdx.x - b * ndir);
         r.f = (int)(b / tiles);
@@ -303,7 +307,7 @@ __device__ __forceinline__ bool link_item(const Geom& g, int ndir, int nfields, 
     return true;
 }
 static inline unsigned link_blocks(bool tiled, const Geom& g, int ndir, int nfields) {
-    return tiled ? (unsigned)ndir * (((unsigned)g.vh + 63) / 64) * (unsigned)nfields
+    return tiled && link_tiled(g) ? (unsigned)ndir * (((unsigned)g.vh + 63) / 64) * (unsigned)nfields
                  : (unsigned)((2LL * ndir * g.vh * nfields + 127) / 128);
 }
 
