@@ -72,11 +72,12 @@ __global__ void __launch_bounds__(OT) k_vortex_remove(const cplx<T>* U, const in
         double c, sn;
         center_phase(m, c, sn);
         if (Ur) {
+            // all nine loads ahead of the stores (which may go to the same field)
+            cplx<T> u[9];
 #pragma unroll
-            for (int e = 0; e < 9; ++e) {
-                const size_t k = lo + lidx(g, mu, p, e, s);
-                Ur[k] = unphase_fast(U[k], m, c, sn);
-            }
+            for (int e = 0; e < 9; ++e) u[e] = U[lo + lidx(g, mu, p, e, s)];
+#pragma unroll
+            for (int e = 0; e < 9; ++e) Ur[lo + lidx(g, mu, p, e, s)] = unphase_fast(u[e], m, c, sn);
         }
         if (Zl) {
 #pragma unroll
