@@ -288,7 +288,7 @@ struct LinkItem {
 __host__ __device__ __forceinline__ bool link_tiled(const Geom& g) { return (-g.vh & 63) * 16 <= g.vh; }
 template <bool TILED>
 __device__ __forceinline__ bool link_item(const Geom& g, int ndir, int nfields, LinkItem& r) {
-    if (TILED && link_tiled(g)) {
+    if (TILED) {
         const unsigned tiles = ((unsigned)g.vh + 63) / 64, b = blockIdx.x / ndir;
         r.kind = (int)(blockIdx.x - b * ndir);
         r.f = (int)(b / tiles);
@@ -307,7 +307,7 @@ __device__ __forceinline__ bool link_item(const Geom& g, int ndir, int nfields, 
     return true;
 }
 static inline unsigned link_blocks(bool tiled, const Geom& g, int ndir, int nfields) {
-    return tiled && link_tiled(g) ? (unsigned)ndir * (((unsigned)g.vh + 63) / 64) * (unsigned)nfields
+    return tiled ? (unsigned)ndir * (((unsigned)g.vh + 63) / 64) * (unsigned)nfields
                  : (unsigned)((2LL * ndir * g.vh * nfields + 127) / 128);
 }
 

@@ -127,7 +127,7 @@ template <bool RECT>
 __global__ void __launch_bounds__(128, 3) k_smear_products_fx(const int4* __restrict__ Uin, int4* __restrict__ Aux,
                                                               Geom g, int nfields) {
     LinkItem it;
-    if (!link_item<!RECT>(g, 12, nfields, it)) return;
+    if (!(!RECT && link_tiled(g) ? link_item<true>(g, 12, nfields, it) : link_item<false>(g, 12, nfields, it))) return;
     const int f = it.f, p = it.p, s = it.s, pair = it.kind;
     const int da = pair / 3, pb = pair - 3 * da, db = pb < da ? pb : pb + 1;
     const size_t vh = (size_t)g.vh;
@@ -221,7 +221,7 @@ __global__ void __launch_bounds__(128, 3) k_smear_step_fx(const int4* __restrict
         s = r - p * g.vh;
     } else {
         LinkItem it;
-        if (!link_item<true>(g, 4, nfields, it)) return;
+        if (!(link_tiled(g) ? link_item<true>(g, 4, nfields, it) : link_item<false>(g, 4, nfields, it))) return;
         f = it.f;
         mu = it.kind;
         p = it.p;
@@ -335,6 +335,7 @@ int run_smear_fx(const void* Uin, void* Uout, const Geom& g, int nfields, double
     if ((rc = scratch_wait("smear", st))) return rc;
     const bool rect = eps != 1.0;
     const FxSmear P = fx_smear_params(rho, eps, 1.0);
+    const bool tiled = !rect && link_tiled(g);
     // step k's source: tmp or Uout in turn, so that the last step reads tmp
     auto buf = [&](int k) { return (n - 1 - k) % 2 == 0 ? tmp : Uout; };
     launch_to_fx(Uin, buf(0), elems, st);
@@ -358,11 +359,11 @@ int run_smear_fx(const void* Uin, void* Uout, const Geom& g, int nfields, double
             int4* dst = (int4*)(last ? Uout : buf(k + 1)) + off;
             if (aux) {
                 (rect ? k_smear_products_fx<true> : k_smear_products_fx<false>)
-                    <<<link_blocks(!rect, g, 12, nf), 128, 0, st>>>(src, aux, g, nf);
+                    <<<link_blocks(tiled, g, 12, nf), 128, 0, st>>>(src, aux, g, nf);
                 note_launches(1);
             }
             const auto step = step_kernel(rect, aux != nullptr, last);
-            step<<<link_blocks(!rect, g, 4, nf), 128, 0, st>>>(src, aux, dst, g, nf, P);
+            step<<<link_blocks(tiled, g, 4, nf), 128, 0, st>>>(src, aux, dst, g, nf, P);
             note_launches(1);
         }
     }
