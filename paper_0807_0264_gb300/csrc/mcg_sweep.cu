@@ -654,7 +654,11 @@ __device__ __forceinline__ double sum_partials_fx(const long long* __restrict__ 
     return ((double)hi * 4294967296.0 + (double)(lo & 0xffffffffLL)) * 0x1p-50;
 }
 
-// mode 0: end of a sweep; 1: fresh start (sweep = 0); 2: continue (new phase)
+// mode 0: end of a sweep; 1: fresh start (sweep = 0); 2: continue (new phase).
+// FX: the integer partials of a fixed-point sweep, in kernels of their own (chosen
+// inside, the kernel that ends the other sweeps took longer: 150 FP32 sweeps each of
+// the levels 0, 4, 10 and 20 of 20^3 x 40 68.8 -> 69.3 ms)
+template <bool FX>
 __device__ __forceinline__ void finalize_field(const SweepBatch& bt, int f, int mode) {
     FieldState* st = &bt.state[f];
     if (mode == 0 && st->done) return;
@@ -662,7 +666,7 @@ __device__ __forceinline__ void finalize_field(const SweepBatch& bt, int f, int 
     const size_t n = (size_t)fd.nblk * bt.ppb;
     const double* __restrict__ part = bt.partial + (size_t)fd.blk0 * bt.ppb;
     double R;
-    if (mode == 0 && bt.tps > 0) {
+    if (FX) {
         R = sum_partials_fx(reinterpret_cast<const long long*>(part), n);
     } else {
         double v = 0.0;
@@ -720,17 +724,20 @@ __device__ __forceinline__ void finalize_field(const SweepBatch& bt, int f, int 
         st->done = 2;
 }
 
-__global__ void __launch_bounds__(256) k_finalize(SweepBatch bt, int mode) { finalize_field(bt, blockIdx.x, mode); }
+template <bool FX>
+__global__ void __launch_bounds__(256) k_finalize(SweepBatch bt, int mode) {
+    finalize_field<FX>(bt, blockIdx.x, mode);
+}
 
 // End of an FP64 sweep: k_finalize in the first nf blocks, and the links and
 // Omega of the fields with reunit_pending set re-unitarised in the others (the
 // odd half-sweep sets it, from the sweep count alone).  With a kernel of its own
 // for the latter, of blocks that exit at entry on most sweeps, 50 sweeps of a 4^4
 // field took 1.42 ms, now 1.36 (1 % on larger fields).
-template <typename T>
+template <typename T, bool FX>
 __global__ void __launch_bounds__(256) k_finalize_reunit(SweepBatch bt) {
     if (blockIdx.x < bt.nf) {
-        finalize_field(bt, blockIdx.x, 0);
+        finalize_field<FX>(bt, blockIdx.x, 0);
         return;
     }
     const int blk = blockIdx.x - bt.nf;
@@ -869,15 +876,16 @@ static int enqueue_sweep(const SweepBatch& bt, int nt, cudaStream_t st) {
         // transformed by the re-unitarised W of the phase
         launch_halfsweep_df(false, bt, 0, bt.total_blocks, st);
         launch_halfsweep_df(true, bt, 1, bt.total_blocks, st);
-        k_finalize<<<bt.nf, 256, 0, st>>>(bt, 0);
+        k_finalize<false><<<bt.nf, 256, 0, st>>>(bt, 0);
     } else {
         launch_halfsweep<T>(nt, false, bt, 0, bt.total_blocks, st);
         launch_halfsweep<T>(nt, true, bt, 1, bt.total_blocks, st);
         // FP32 sweeps re-unitarise inside the half-sweep kernel
         if (sizeof(T) == 8 && bt.reunit_every > 0)
-            k_finalize_reunit<double><<<bt.nf + bt.total_blocks, 256, 0, st>>>(bt);
+            (bt.tps > 0 ? k_finalize_reunit<double, true>
+                        : k_finalize_reunit<double, false>)<<<bt.nf + bt.total_blocks, 256, 0, st>>>(bt);
         else
-            k_finalize<<<bt.nf, 256, 0, st>>>(bt, 0);
+            (bt.tps > 0 ? k_finalize<true> : k_finalize<false>)<<<bt.nf, 256, 0, st>>>(bt, 0);
     }
     return 0;
 }
@@ -1040,7 +1048,7 @@ int run_fix_phase(const std::vector<FieldDesc>& fields_in, FieldState* d_state, 
         if ((rc = fx.tps ? prepare_halfsweep_fx() : prepare_halfsweep<T>(NT))) return rc;
         k_functional<T><<<total, NT, 0, stream>>>(bt);
     }
-    k_finalize<<<nf, 256, 0, stream>>>(bt, fresh ? 1 : 2);
+    k_finalize<false><<<nf, 256, 0, stream>>>(bt, fresh ? 1 : 2);
     MCG_CK(cudaGetLastError());
     note_launches(2);
     if (phase_len <= 0) {
@@ -1201,7 +1209,7 @@ int run_fix_phase(const std::vector<FieldDesc>& fields_in, FieldState* d_state, 
         // goes on)
         if constexpr (std::is_same<T, float>::value) {
             k_functional<T><<<fields[f].nblk, NT, 0, stream>>>(chains[f]);
-            k_finalize<<<1, 256, 0, stream>>>(chains[f], 2);
+            k_finalize<false><<<1, 256, 0, stream>>>(chains[f], 2);
             e = cudaGetLastError();
             if (e != cudaSuccess) return cuda_fail(e, "restart");
             note_launches(2);
