@@ -286,6 +286,16 @@ struct LinkItem {
     int f, kind, p, s;
 };
 __host__ __device__ __forceinline__ bool link_tiled(const Geom& g) { return (-g.vh & 63) * 16 <= g.vh; }
+// The other order: threads per kind.  Whole warps, as one with links of two kinds
+// takes the paths of both, unless the blocks then go once more round the SMs (FP64
+// stout, five steps, us, in whole warps and not, tiled: 2^4 128, 147, 136; 256 fields of
+// 2^4, on 256 and 128 blocks, 191, 160, 352; four of 6 x 6 x 2 x 2 148, 167, 144).
+__host__ __device__ __forceinline__ int link_row(const Geom& g, int ndir, int nfields) {
+    const int row = 2 * g.vh, whole = (row + 31) & ~31;
+    if (row == whole) return row;
+    const long long n = (long long)ndir * nfields, per = 128 * 152;
+    return (n * whole + per - 1) / per > (n * row + per - 1) / per ? row : whole;
+}
 template <bool TILED>
 __device__ __forceinline__ bool link_item(const Geom& g, int ndir, int nfields, LinkItem& r) {
     if (TILED) {
@@ -296,19 +306,20 @@ __device__ __forceinline__ bool link_item(const Geom& g, int ndir, int nfields, 
         r.p = (int)(threadIdx.x >> 6);
         return r.s < g.vh;
     }
-    const long long per = 2LL * ndir * g.vh, id = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const int row = link_row(g, ndir, nfields);
+    const long long per = (long long)ndir * row, id = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (id >= per * nfields) return false;
     r.f = (int)(id / per);
     int k = (int)(id - r.f * per);
-    r.kind = k / (2 * g.vh);
-    k -= r.kind * 2 * g.vh;
+    r.kind = k / row;
+    k -= r.kind * row;
     r.p = k / g.vh;
     r.s = k - r.p * g.vh;
-    return true;
+    return k < 2 * g.vh;
 }
 static inline unsigned link_blocks(bool tiled, const Geom& g, int ndir, int nfields) {
     return tiled ? (unsigned)ndir * (((unsigned)g.vh + 63) / 64) * (unsigned)nfields
-                 : (unsigned)((2LL * ndir * g.vh * nfields + 127) / 128);
+                 : (unsigned)(((long long)ndir * link_row(g, ndir, nfields) * nfields + 127) / 128);
 }
 
 template <typename T>

@@ -209,7 +209,7 @@ __global__ void __launch_bounds__(128, 3) k_smear_step_fx(const int4* __restrict
                                                           int4* __restrict__ Uout, Geom g, int nfields,
                                                           const __grid_constant__ FxSmear P) {
     int f, mu, p, s;
-    if (RECT) {  // link_item<false>, which the step took 0.8 % longer with
+    if (RECT) {  // link_item<false> without whole warps, which the step took 0.8 % longer with
         const long long n = 8LL * g.vh * nfields;
         const long long id = (long long)blockIdx.x * blockDim.x + threadIdx.x;
         if (id >= n) return;
@@ -363,7 +363,8 @@ int run_smear_fx(const void* Uin, void* Uout, const Geom& g, int nfields, double
                 note_launches(1);
             }
             const auto step = step_kernel(rect, aux != nullptr, last);
-            step<<<link_blocks(tiled, g, 4, nf), 128, 0, st>>>(src, aux, dst, g, nf, P);
+            const unsigned nb = rect ? (unsigned)((8LL * g.vh * nf + 127) / 128) : link_blocks(tiled, g, 4, nf);
+            step<<<nb, 128, 0, st>>>(src, aux, dst, g, nf, P);
             note_launches(1);
         }
     }

@@ -275,3 +275,19 @@ def test_block_orders_of_stout_steps(dims):
     for U, s, s32 in zip(Us, S, S32):
         ref = oracle.smear(dims, U, 0.1, 1.0, 2)
         assert np.abs(s - ref).max() < 4e-14 and np.abs(s32 - ref).max() < 2e-5
+
+
+# the other block order, a kind's sites in whole warps or not (200 and 20 fields: the rule's other side), stout and
+# over-improved.  FP64: 2e-14 per step; FP32: ~500 roundings of 6e-8 per link and step
+@pytest.mark.parametrize("eps,rho", [(1.0, 0.1), (-0.25, 0.06)])
+@pytest.mark.parametrize("dims,copies", [((2, 2, 2, 2), 1), ((2, 2, 2, 2), 67), ((6, 6, 2, 2), 2), ((6, 6, 2, 2), 22), ((6, 6, 6, 2), 7)])
+def test_rows_of_whole_warps(dims, copies, eps, rho):
+    from paper_0807_0264_gb300 import mcg
+
+    Us = [synth.make_field(dims, 0.7, s) for s in range(3)]
+    Ud = _pack(mcg, Us * copies, dims)
+    S = mcg.mcg_unpack_links(mcg.mcg_smear(Ud, dims, rho, eps, 2), dims).cpu().numpy()
+    S32 = mcg.mcg_unpack_links(mcg.mcg_smear(mcg.mcg_convert(Ud, mcg.F32), dims, rho, eps, 2), dims).cpu().numpy()
+    refs = [oracle.smear(dims, U, rho, eps, 2) for U in Us]
+    for k in range(3 * copies):
+        assert np.abs(S[k] - refs[k % 3]).max() < 4e-14 and np.abs(S32[k] - refs[k % 3]).max() < 6e-5
