@@ -127,13 +127,7 @@ __global__ void __launch_bounds__(128, 3) k_apply_gauge_fx(double2* Uall, const 
         const int4* w = reinterpret_cast<const int4*>(Gall) + iwf;
 #pragma unroll
         for (int e = 0; e < 9; ++e) b[e] = fx_load(w + e * vh);
-        if (bad || b[0].re.l == kFxMarked) {
-            const size_t i = (size_t)f * c12_gauge_chunks(g) + c12_gidx(g, p, 0, s);
-            const size_t j = (size_t)f * c12_gauge_chunks(g) + c12_gidx(g, p ^ 1, 0, sf);
-            handoff_link_f64(u, reinterpret_cast<const int4*>(Gall) + iw, w, W + i, Wlo ? Wlo + i : nullptr, W + j,
-                             Wlo ? Wlo + j : nullptr, vh);
-            return;
-        }
+        bad = bad || b[0].re.l == kFxMarked;
     } else {
         bad = fx_load_matrix(reinterpret_cast<const double2*>(Gall) + iwf, 3 * vh, vh, b) || bad;
     }
@@ -142,6 +136,13 @@ __global__ void __launch_bounds__(128, 3) k_apply_gauge_fx(double2* Uall, const 
         return;
     }
     m3fx_mul_inplace<true>(a, b);
+    if (WFX && bad) {
+        const size_t i = (size_t)f * c12_gauge_chunks(g) + c12_gidx(g, p, 0, s);
+        const size_t j = (size_t)f * c12_gauge_chunks(g) + c12_gidx(g, p ^ 1, 0, sf);
+        handoff_link_f64(u, reinterpret_cast<const int4*>(Gall) + iw, reinterpret_cast<const int4*>(Gall) + iwf, W + i,
+                         Wlo ? Wlo + i : nullptr, W + j, Wlo ? Wlo + j : nullptr, vh);
+        return;
+    }
 #pragma unroll
     for (int e = 0; e < 9; ++e) fx_store(u + e * vh, a[e]);
 }
@@ -173,38 +174,38 @@ __global__ void __launch_bounds__(128, 3) k_handoff_gauge_fx(const float4* __res
     const size_t off = (size_t)f * gauge_elems(g) + gidx(g, p, 0, s), vh = (size_t)g.vh;
     const size_t coff = (size_t)f * c12_gauge_chunks(g) + c12_gidx(g, p, 0, s);
     cfx w[9], o[9];
-    unsigned big = 0;
+    float size = 0.f;  // squared norm of rows 0 and 1, 2 for a unitary W (NaN fails the test)
 #pragma unroll
     for (int q = 0; q < 3; ++q) {
         const float4 v = W[coff + q * vh];
-        big = max(max(big, max(fx_magnitude(v.x), fx_magnitude(v.y))), max(fx_magnitude(v.z), fx_magnitude(v.w)));
+        size = fmaf(v.x, v.x, fmaf(v.y, v.y, fmaf(v.z, v.z, fmaf(v.w, v.w, size))));
         w[2 * q].re = fx_of(v.x);
         w[2 * q].im = fx_of(v.y);
         w[2 * q + 1].re = fx_of(v.z);
         w[2 * q + 1].im = fx_of(v.w);
         if (Wlo) {
             const float4 l = Wlo[coff + q * vh];
-            big = max(max(big, max(fx_magnitude(l.x), fx_magnitude(l.y))), max(fx_magnitude(l.z), fx_magnitude(l.w)));
+            size = fmaf(l.x, l.x, fmaf(l.y, l.y, fmaf(l.z, l.z, fmaf(l.w, l.w, size))));
             w[2 * q].re = fx_split(fx_join(w[2 * q].re) + fx_join(fx_of(l.x)));
             w[2 * q].im = fx_split(fx_join(w[2 * q].im) + fx_join(fx_of(l.y)));
             w[2 * q + 1].re = fx_split(fx_join(w[2 * q + 1].re) + fx_join(fx_of(l.z)));
             w[2 * q + 1].im = fx_split(fx_join(w[2 * q + 1].im) + fx_join(fx_of(l.w)));
         }
     }
-    if (m3fx_reunitarise(w) || big > kFxMagnitude) {
-        Wfx[off] = make_int4(0, kFxMarked, 0, 0);
-        handoff_gauge_f64(W + coff, Wlo ? Wlo + coff : nullptr, G + off, vh);
-        return;
-    }
+    const bool bad = m3fx_reunitarise(w) || !(size < 2.1f);
 #pragma unroll
     for (int e = 0; e < 9; ++e) {
-        Wfx[off + e * vh] = fx_pack(w[e]);
+        Wfx[off + e * vh] = e == 0 && bad ? make_int4(0, kFxMarked, 0, 0) : fx_pack(w[e]);
         const double2 v = G[off + e * vh];
         o[e].re = fx_of(v.x);
         o[e].im = fx_of(v.y);
     }
     m3fx_mul_inplace<false>(w, o);
     m3fx_reunitarise(w);
+    if (bad) {  // not before the loads of Omega, which would wait for the branch
+        handoff_gauge_f64(W + coff, Wlo ? Wlo + coff : nullptr, G + off, vh);
+        return;
+    }
 #pragma unroll
     for (int e = 0; e < 9; ++e) fx_store(G + off + e * vh, w[e]);
 }
