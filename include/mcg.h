@@ -245,14 +245,17 @@ int mcg_reunitarise(void* M, int which, const mcg_lattice* lat, cudaStream_t str
  * U_in is validated first (see "Input validation"; synchronises), then the
  * steps run asynchronously on `stream`.
  * FP64 fields with |rho| (6 |5-2eps| / 3 + 18 |1-eps| / 12) <= 1 take the steps
- * in 64-bit fixed point of unit 2^-60 (errors below the FP64 arithmetic's), on
- * a scratch copy of the field and up to 16 GiB of scratch for products that
- * neighbouring links share.  What the steps can do without (the copy for a single
- * step, which then runs in FP64, and the products, without which every path is
- * multiplied out) takes at most a quarter of the free memory and is given up
- * when another call needs scratch that no longer fits; mcg_release() frees it
- * for the caller.  Calls on several streams are ordered on the GPU where they share
- * scratch.
+ * in 64-bit fixed point of unit 2^-60: absolute errors of about 2^-58 per product,
+ * below the FP64 arithmetic's for links with entries of order one.  The unit does
+ * not follow an entry's size: one far below 1 keeps its digits down to 2^-60 only
+ * (links within 1e-8 of the identity: eight digits fewer of the distance than FP64
+ * holds).  The steps work on a scratch copy of the field and up to 16 GiB of
+ * scratch for products that neighbouring links share.  What the steps can do
+ * without (the copy for a single step, which then runs in FP64, and the products,
+ * without which every path is multiplied out) takes at most a quarter of the free
+ * memory and is given up when another call needs scratch that no longer fits;
+ * mcg_release() frees it for the caller.  Calls on several streams are ordered on
+ * the GPU where they share scratch.
  */
 int mcg_smear(const void* U_in, void* U_out, const mcg_lattice* lat, double rho, double eps, int n,
               cudaStream_t stream);
@@ -294,7 +297,8 @@ int mcg_fix(void* U, void* G, const mcg_lattice* lat, const mcg_params* params, 
  * rounded to FP32, Newton from a = e0 on the KKT system with its certificate
  * that the multiplier lies above lambda_max(A), else FP32 Jacobi + secular);
  * MCG_F64: the solve of the exact sweep in FP64 arithmetic (the plain FP64
- * sweep of validated fields solves the same problem in fixed point, with this
+ * sweep of validated fields solves the same problem, and moves the links, in fixed
+ * point of unit 2^-58, with the condition that mcg_smear states, and with this
  * solve where its own does not settle).  In the hard case (b orthogonal
  * to the top eigenspace, a maximum that is not unique) any maximiser may be
  * returned.  n = 0 does nothing; n < 0, a null array (n > 0) or another

@@ -23,6 +23,11 @@
 // by Cauchy-Schwarz, below 2 sqrt(6) 2^59 < 2^62 in the middle one.  Values up
 // to 8 in magnitude are representable; every kernel states its operand bounds.
 //
+// The unit is absolute: an entry far below 1 keeps its digits down to 2^-60 (2^-58 in
+// the sweep) only, where FP64 keeps 53 bits of any size.  That matters to fields of
+// which every link is near the identity (1e-8 from it: eight digits fewer of the
+// distance), not to entries of order one.
+//
 // The functions are plain integer code, compiled for the host as well (the
 // host tests run them).
 #pragma once
