@@ -251,10 +251,11 @@ int mcg_reunitarise(void* M, int which, const mcg_lattice* lat, cudaStream_t str
  * (links within 1e-8 of the identity: eight digits fewer of the distance than FP64
  * holds).  The steps work on a scratch copy of the field and up to 16 GiB of
  * scratch for products that neighbouring links share.  What the steps can do
- * without (the copy for a single step, which then runs in FP64, and the products,
- * without which every path is multiplied out) takes at most a quarter of the free
- * memory and is given up when another call needs scratch that no longer fits;
- * mcg_release() frees it for the caller.  Calls on several streams are ordered on
+ * without (the copy for a single step, which runs in FP64 where there is no room for
+ * one field, and the products, without which every path is multiplied out) takes at
+ * most a quarter of the free memory, for fewer fields at a time if need be, and is
+ * given up when another call needs scratch that no longer fits; mcg_release() frees
+ * it for the caller.  Calls on several streams are ordered on
  * the GPU where they share scratch.
  */
 int mcg_smear(const void* U_in, void* U_out, const mcg_lattice* lat, double rho, double eps, int n,
@@ -529,7 +530,7 @@ int mcg_gribov_search(const mcg_field* copies, int ncopies, const int* config_of
  * staple.  In 64-bit fixed point, each link gathering its terms (reproducible
  * bits), under the rule of mcg_smear and for links that are near-unitary;
  * otherwise, while `stream` is being captured and where there is no memory for
- * the scratch (two fields), in FP64 with atomic adds (summation order, hence
+ * the scratch (two copies of one field), in FP64 with atomic adds (summation order, hence
  * the last bits, vary).
  * U: the step's input field (FP64); Gout, Gin: FP64, link layout, distinct. */
 int mcg_smear_backward_step(const void* U, const double* Gout, double* Gin, const mcg_lattice* lat, double rho,

@@ -341,6 +341,15 @@ int run_smear(const void* Uin, void* Uout, int prec, const Geom& g, int nfields,
         bool ran = false;
         rc = run_smear_fx(Uin, Uout, g, nfields, rho, eps, n, &ran, st);
         if (rc || ran) return rc;
+        // a single step whose copy of all fields is more than its share: fewer at a time
+        const size_t per = 16 * link_elems(g);
+        const int m = (int)std::min<size_t>(nfields, scratch_optional_room("smear.tmp") / per);
+        for (int f0 = 0; m > 0 && f0 < nfields; f0 += m) {
+            rc = run_smear_fx((const char*)Uin + per * f0, (char*)Uout + per * f0, g, std::min(m, nfields - f0), rho,
+                              eps, n, &ran, st);
+            if (rc || !ran) break;
+        }
+        if (rc || ran) return rc;
     }
     void* tmp = nullptr;
     if (n >= 2) {
@@ -756,27 +765,40 @@ __global__ void __launch_bounds__(256) k_ascent_gauge(const double* __restrict__
 int run_smear_step_backward(const void* U, const double* Gout, double* Gin, const Geom& g, int nfields, double rho,
                             double eps, cudaStream_t st) {
     const double cp = (5.0 - 2.0 * eps) / 3.0, cr = -(1.0 - eps) / 12.0;
-    const long long n = 8LL * g.vh * nfields;
-    unsigned* only = nullptr;
     // The FP64 kernel alone while a graph is captured (the fixed-point kernels
     // need scratch, which a graph that is launched later would share unordered
-    // with other calls) and where there is no memory for that scratch.
+    // with other calls) and where there is no memory for the scratch of one field.
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     MCG_CK(cudaStreamIsCapturing(st, &cap));
-    if (cap == cudaStreamCaptureStatusNone && smear_fx_applies(rho, eps)) {
-        int rc = run_smear_backward_fx(U, Gout, Gin, g, nfields, rho, eps, &only, st);
-        if (rc) return rc;
+    bool fx = cap == cudaStreamCaptureStatusNone && smear_fx_applies(rho, eps), used = false;
+    int most = nfields;  // fields at a time
+    for (int f0 = 0, nf = 0; f0 < nfields; f0 += nf) {
+        const size_t off = 16 * link_elems(g) * (size_t)f0;
+        const void* Uf = (const char*)U + off;
+        const double* Gof = (const double*)((const char*)Gout + off);
+        double* Gif = (double*)((char*)Gin + off);
+        unsigned* only = nullptr;
+        nf = std::min(most, nfields - f0);
+        while (fx) {
+            if (int rc = run_smear_backward_fx(Uf, Gof, Gif, g, nf, rho, eps, &only, st)) return rc;
+            if (only) break;
+            fx = nf > 1;
+            nf = most = fx ? (nf + 1) / 2 : nfields - f0;
+        }
+        used = used || only;
+        const long long n = 8LL * g.vh * nf;
+        if (only) {
+            k_zero_if<<<(unsigned)((18 * n + 255) / 256), 256, 0, st>>>(Gif, 18 * n, only);
+        } else {
+            MCG_CK(cudaMemsetAsync(Gif, 0, 16 * link_elems(g) * (size_t)nf, st));
+        }
+        k_smear_step_backward<<<(int)((n + ST - 1) / ST), ST, 0, st>>>((const cplx<double>*)Uf,
+                                                                        (const cplx<double>*)Gof, Gif, g, nf, rho, cp,
+                                                                        cr, only);
+        MCG_CK(cudaGetLastError());
+        note_launches(1);
     }
-    if (only) {
-        k_zero_if<<<(unsigned)((18 * n + 255) / 256), 256, 0, st>>>(Gin, 18 * n, only);
-    } else {
-        MCG_CK(cudaMemsetAsync(Gin, 0, 16 * link_elems(g) * (size_t)nfields, st));
-    }
-    k_smear_step_backward<<<(int)((n + ST - 1) / ST), ST, 0, st>>>((const cplx<double>*)U, (const cplx<double>*)Gout,
-                                                                    Gin, g, nfields, rho, cp, cr, only);
-    MCG_CK(cudaGetLastError());
-    note_launches(1);
-    return only ? scratch_mark("bwd", st) : 0;
+    return used ? scratch_mark("bwd", st) : 0;
 }
 
 int run_functional_matrix_grad(const void* U, int prec, double* G, const Geom& g, int nfields, cudaStream_t st) {

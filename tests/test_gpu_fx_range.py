@@ -291,3 +291,29 @@ def test_rows_of_whole_warps(dims, copies, eps, rho):
     refs = [oracle.smear(dims, U, rho, eps, 2) for U in Us]
     for k in range(3 * copies):
         assert np.abs(S[k] - refs[k % 3]).max() < 4e-14 and np.abs(S32[k] - refs[k % 3]).max() < 6e-5
+
+
+# batches whose scratch is more than its share of the free memory go a few fields at a time: the same bits
+@pytest.mark.parametrize("eps,rho", [(1.0, 0.1), (-0.25, 0.06)])
+def test_smearing_of_batches_beyond_the_scratch_share(eps, rho):
+    from paper_0807_0264_gb300 import mcg
+
+    dims, nf = (8, 8, 8, 8), 37
+    U = torch.cat([_pack(mcg, [synth.make_field(dims, 0.7, s) for s in range(2)], dims)] * 19)[:nf].contiguous()
+    G = torch.randn(U.shape, dtype=U.dtype, device="cuda", generator=torch.Generator(device="cuda").manual_seed(5))
+    step, back = mcg.mcg_smear(U, dims, rho, eps, 1), mcg.mcg_smear_backward_step(U, G, dims, rho, eps)
+    outs = [torch.empty_like(U), torch.empty_like(U)]
+    del outs[1]  # room in the caller's allocator for the gradient
+    torch.cuda.synchronize()
+    mcg.mcg_release()
+    free = torch.cuda.mem_get_info()[0] - (240 << 20)
+    assert free > 0
+    fill = torch.empty(free, dtype=torch.uint8, device="cuda")  # leaves 240 MB: a share of 60 MB, a copy takes 87
+    try:
+        mcg.mcg_smear(U, dims, rho, eps, 1, outs[0])
+        assert torch.equal(outs[0], step)
+        assert torch.equal(mcg.mcg_smear_backward_step(U, G, dims, rho, eps), back)
+    finally:
+        del fill
+        mcg.mcg_release()
+        torch.cuda.empty_cache()
